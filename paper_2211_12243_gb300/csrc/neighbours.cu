@@ -1,16 +1,16 @@
 // Bucketed neighbour search (§2.2.3).  The Morton-sorted particles are cut
 // into buckets of 32 (one warp each); buckets are grouped 32 at a time into
 // a fixed-arity bounding-box tree per periodic box.  One warp walks the tree
-// once for its whole bucket (the paper's single search per bucket).  Each
-// candidate bucket is staged in shared memory -- only its particles within
-// the search radius of the warp's bucket box, compacted -- and every lane
-// tests the staged particles against its own, appending matches to its
-// fixed-stride row of the list (or, for long lists, the overflow region).
+// once for its whole bucket (the paper's single search per bucket).  The
+// particles of the candidate buckets near the owners' boxes are collected
+// into tiles of 32 in shared memory; every lane tests a full tile against
+// its own particle and appends the matches to its fixed-stride row of the
+// list (or, for long lists, the overflow region).
 //
 // Membership r_ij < h_search,i is decided exactly as the definition states
 // in double precision: a float test on the fixed-point separation settles
-// every candidate farther than 1e-4 (relative, on r^2) from the boundary,
-// and the rest are re-tested with the double-precision minimum image.
+// every candidate outside a band around the boundary that covers the float
+// error, and the rest are re-tested with the double-precision minimum image.
 #include "hydro_internal.cuh"
 
 namespace hyd {
@@ -18,6 +18,7 @@ namespace hyd {
 namespace {
 
 constexpr int LIST_WARPS = 4;
+constexpr int LIST_CTAS = 6;   // resident CTAs per SM (80 registers; 5 and 8 were within 3 %)
 constexpr int STACK = 256;
 
 __device__ __forceinline__ uint32_t wmin(uint32_t v) {
@@ -138,7 +139,7 @@ __device__ __forceinline__ bool boxes_near(uint4 alo, uint4 ahi, uint4 blo, uint
 }
 
 struct ListArgs {
-    int64_t nbucket;
+    int64_t nbucket;         // buckets to build (of the queue in modes 1, 2)
     const int32_t *node_first, *node_cnt, *node_box, *box_root;
     int64_t nbucket_total;   // node ids below this are buckets
     const uint4 *lo, *hi;
@@ -151,30 +152,22 @@ struct ListArgs {
     int64_t capacity;
     DevCounters *cnt;
     int cap;   // fixed slots per particle (row s at s cap)
-    int mode;  // 0: write the fixed-stride rows (buckets with a row longer
-               //    than cap are queued in ovf_list);
-               // 1: count and reserve storage (queued buckets);
-               // 2: write at nbr_off (queued buckets)
     int32_t *ovf_list;      // queued bucket ids
     int *ovf_count;
-    bool nq_dev;            // modes 1, 2: warps past *ovf_count have no bucket
+    bool nq_dev;            // modes 1, 2: the queue's length is *ovf_count
+};
+
+// What a pass of k_build_lists does
+enum : int {
+    LIST_ROWS = 0,    // write the fixed-stride rows (a bucket with a row longer
+                      // than cap is queued in ovf_list)
+    LIST_COUNT = 1,   // count and reserve storage (queued buckets)
+    LIST_FILL = 2     // write at nbr_off (queued buckets)
 };
 
 __device__ __forceinline__ float u2f(uint32_t v) {
     return fmaf(i2f_small((int32_t)(v >> 11)), 2048.0f, i2f_small((int32_t)(v & 0x7FFu)));
 }
-
-// Per-lane state of the walk: the owner particle, its position relative to
-// the bucket's corner (float), and the exact-test data.
-struct Lane {
-    bool own;
-    int s;
-    uint32_t qx, qy, qz;
-    float rx, ry, rz;        // relative to the warp's origin
-    double x, y, z, hs, h2;
-    float lo2, hi2;          // float band around hs^2 (lo2 < 0 < hi2 = inf: always exact)
-    bool rel_ok;             // bucket extent + radius < L/4: relative coordinates are exact images
-};
 
 // circular gap (fixed-point units) between a point and an interval
 __device__ __forceinline__ uint32_t point_gap(uint32_t p, uint32_t b0, uint32_t b1) {
@@ -184,303 +177,384 @@ __device__ __forceinline__ uint32_t point_gap(uint32_t p, uint32_t b0, uint32_t 
     return e > w + 2u ? e - w - 2u : 0u;
 }
 
-// does the lane's sphere reach the box?
-__device__ __forceinline__ bool sphere_near(const Lane &L, uint4 blo, uint4 bhi, const Box &bx) {
-    float gx = u2f(point_gap(L.qx, blo.x, bhi.x)) * bx.s[0];
-    float gy = u2f(point_gap(L.qy, blo.y, bhi.y)) * bx.s[1];
-    float gz = u2f(point_gap(L.qz, blo.z, bhi.z)) * bx.s[2];
-    return L.own && gx * gx + gy * gy + gz * gz <= L.hi2;
-}
-
-// one staged candidate particle (registers of the lane that loads it)
-struct Cand {
-    double x, y, z;
-    uint32_t qx, qy, qz;
+// The warp's candidates, a ring of two tiles of 32: positions relative to the
+// bucket's corner (or the fixed-point ones) and sorted indices;
+// and the boxes its owners are culled by
+struct Tiles {
+    float4 r[64];
+    int32_t j[64];
+    int32_t stack[STACK];
+    uint4 lo[2], hi[2];      // fixed-point corners; .w: largest radius
+    float4 ctr[2], ext[2];   // relative centre (.w: squared reach), half widths
 };
 
-__device__ __forceinline__ void cand_load(const ListArgs &a, int j, Cand &c) {
-    c.x = a.xs[j]; c.y = a.ys[j]; c.z = a.zs[j];
-    c.qx = a.qx[j]; c.qy = a.qy[j]; c.qz = a.qz[j];
+// r < hs decided as the definition states it
+__device__ __forceinline__ bool list_exact(const ListArgs &a, const Box &bx, int s, int j) {
+    const double ex = fold64(__dsub_rn(a.xs[j], a.xs[s]), bx.L[0]);
+    const double ey = fold64(__dsub_rn(a.ys[j], a.ys[s]), bx.L[1]);
+    const double ez = fold64(__dsub_rn(a.zs[j], a.zs[s]), bx.L[2]);
+    const double h = a.hs[s];
+    return r2_exact(ex, ey, ez) < __dmul_rn(h, h);
 }
 
-struct Stage {
-    double *sx, *sy, *sz;
-    float4 *sr;              // position relative to the warp's origin; .w = index bits
-    uint32_t *sq;
-};
-
-// per-stage bytes: sr[32] float4 | sx sy sz [32] double | sq[96]
-constexpr size_t STAGE_BYTES = 32 * 16 + 3 * 32 * 8 + 96 * 4;
-
-// Stage this lane's candidate (keep = it can lie within the search radius
-// of some particle of the warp's bucket): the kept candidates are compacted
-// to the front in their original order; returns their number.
-__device__ __forceinline__ int cand_stage(const Stage &S, bool keep, int lane, const Cand &c, int j,
-                                          uint32_t ox, uint32_t oy, uint32_t oz, const Box &bx) {
-    const unsigned m = __ballot_sync(0xffffffffu, keep);
-    if (keep) {
-        const int pos = __popc(m & ((1u << lane) - 1u));
-        S.sx[pos] = c.x; S.sy[pos] = c.y; S.sz[pos] = c.z;
-        S.sq[pos] = c.qx; S.sq[32 + pos] = c.qy; S.sq[64 + pos] = c.qz;
-        S.sr[pos] = make_float4(qdiff(ox, c.qx, bx.s[0]), qdiff(oy, c.qy, bx.s[1]),
-                                qdiff(oz, c.qz, bx.s[2]), __int_as_float(j));
-    }
-    return __popc(m);
-}
-
-// can candidate c lie within rad2 of a point of the bucket box [lo, hi]?
-// (a lower bound of the periodic distance, as in sphere_near)
-__device__ __forceinline__ bool cand_near(const Cand &c, uint4 lo, uint4 hi, const Box &bx,
-                                          float rad2) {
-    float gx = u2f(point_gap(c.qx, lo.x, hi.x)) * bx.s[0];
-    float gy = u2f(point_gap(c.qy, lo.y, hi.y)) * bx.s[1];
-    float gz = u2f(point_gap(c.qz, lo.z, hi.z)) * bx.s[2];
-    return gx * gx + gy * gy + gz * gz <= rad2;
-}
-
-// Output row of a lane: where its matches go and how many fit.
-struct Row {
-    int32_t *out;
-    int lim;
-};
-
-// decide staged candidate k for this lane
-__device__ __forceinline__ void decide(const Lane &L, const Row &R, const Stage &S, const Box &bx,
-                                       int k, float r2, int &count) {
-    bool in = r2 < L.lo2;
-    if (!in && r2 <= L.hi2) {   // within the float band: decide in double
-        double ex = fold64(__dsub_rn(S.sx[k], L.x), bx.L[0]);
-        double ey = fold64(__dsub_rn(S.sy[k], L.y), bx.L[1]);
-        double ez = fold64(__dsub_rn(S.sz[k], L.z), bx.L[2]);
-        in = r2_exact(ex, ey, ez) < L.h2;
-    }
-    if (in) {
-        if (count < R.lim) R.out[count] = __float_as_int(S.sr[k].w);
-        count++;
-    }
-}
-
-// every lane scans the c staged candidates (four at a time for overlap)
-__device__ __forceinline__ void scan_stage(const Lane &L, const Row &R, const Stage &S,
-                                           const Box &bx, int c, int &count) {
-    if (!L.own) return;
-    if (L.rel_ok) {
-        for (int k = 0; k < c; k += 4) {
-            float r2[4];
-#pragma unroll
-            for (int u = 0; u < 4; u++) {
-                float4 r = S.sr[k + u];
-                float dx = r.x - L.rx, dy = r.y - L.ry, dz = r.z - L.rz;
-                r2[u] = dx * dx + dy * dy + dz * dz;
-            }
-#pragma unroll
-            for (int u = 0; u < 4; u++)
-                if (k + u < c) decide(L, R, S, bx, k + u, r2[u], count);
-        }
-    } else {
-        for (int k = 0; k < c; k++) {
-            float dx = qdiff(L.qx, S.sq[k], bx.s[0]);
-            float dy = qdiff(L.qy, S.sq[32 + k], bx.s[1]);
-            float dz = qdiff(L.qz, S.sq[64 + k], bx.s[2]);
-            decide(L, R, S, bx, k, dx * dx + dy * dy + dz * dz, count);
-        }
-    }
-}
-
-__global__ void __launch_bounds__(LIST_WARPS * 32, 5) k_build_lists(ListArgs a) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
+// Neighbour lists: a warp takes 32 / SPLIT owners of a bucket, each held by
+// SPLIT lanes.  One walk of the tree finds the buckets near the owners'
+// boxes; their particles near those boxes are collected into tiles of 32 in
+// shared memory, and a full tile is tested by all owners: per candidate one
+// broadcast read, the distance, two comparisons and one bit of the lane's
+// member mask, without a branch (lane group g of an owner takes the g-th part
+// of the tile).  The masks then give the members in the candidates' order,
+// which is the walk's -- internal nodes last pushed first, buckets in
+// ascending order -- whatever the split.
+//
+// Bound by instruction issue (about 11 instructions per candidate and warp).
+// Measured against lanes that each decided and appended one candidate at a
+// time, the owners culled by one box and the band 1e-4 wide (neighbour stage
+// with sort and gathers, 1 GB300): 128^3 lattice at 1.15 h 4.99 -> 1.47 ms (its
+// fifth lattice shell lies within 1e-4 of the radius, so the FP64 re-tests
+// took 72 % of the time), 1.07 M tube at 1.05 h 1.84 -> 1.14 ms, log-normal
+// box of 4 M at 1.05 h 6.5 -> 4.15 ms (two boxes instead of one: 20.8 ms with
+// one, whose few straddling buckets collected whole octants).  A warp per
+// (owner, bucket) pair with the bucket's particles on the lanes was slower
+// (128^3: 7.1 ms).  SPLIT > 1 shortens the serial walk of grids that leave the
+// GPU idle: 16^3 box 0.21 -> 0.12 ms.
+template <int MODE, int SPLIT>
+__global__ void __launch_bounds__(LIST_WARPS * 32, LIST_CTAS) k_build_lists(ListArgs a) {
+    constexpr int OW = 32 / SPLIT;            // owners of a warp
+    __shared__ Tiles tiles_all[LIST_WARPS];
+    __shared__ int over_all[LIST_WARPS];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int64_t b = blockIdx.x * (int64_t)LIST_WARPS + warp;
-    // per-warp shared memory: stack[STACK] | 2 stages
-    size_t per_warp = STACK * 4 + 2 * STAGE_BYTES;
-    unsigned char *base = smem_raw + per_warp * warp;
-    int32_t *stack = (int32_t *)base;
-    // the two staging buffers, addressed arithmetically (no local array)
-    auto stage = [&](int t) {
-        unsigned char *p = base + STACK * 4 + t * STAGE_BYTES;
-        Stage st;
-        st.sr = (float4 *)p;
-        st.sx = (double *)(p + 32 * 16);
-        st.sy = st.sx + 32;
-        st.sz = st.sy + 32;
-        st.sq = (uint32_t *)(st.sz + 32);
-        return st;
-    };
-    if (b >= a.nbucket) return;
-    if (a.mode != 0) {
-        if (a.nq_dev && b >= *a.ovf_count) return;
-        b = a.ovf_list[b];
-    }
-
-    const int f = a.node_first[b], c = a.node_cnt[b];
-    const Box bx = a.boxes[a.node_box[b]];
-    const uint4 qlo = a.lo[b], qhi = a.hi[b];
-    const uint32_t ox = qlo.x, oy = qlo.y, oz = qlo.z;   // the warp's origin
-    Lane L;
-    L.own = lane < c;
-    L.s = f + (L.own ? lane : 0);
-    L.qx = a.qx[L.s]; L.qy = a.qy[L.s]; L.qz = a.qz[L.s];
-    L.rx = qdiff(ox, L.qx, bx.s[0]);
-    L.ry = qdiff(oy, L.qy, bx.s[1]);
-    L.rz = qdiff(oz, L.qz, bx.s[2]);
-    L.x = a.xs[L.s]; L.y = a.ys[L.s]; L.z = a.zs[L.s]; L.hs = a.hs[L.s];
-    L.h2 = __dmul_rn(L.hs, L.hs);
-    {
-        float hf = (float)L.hs;
-        L.lo2 = hf * hf * (1.0f - 1e-4f);
-        L.hi2 = hf * hf * (1.0f + 1e-4f);
-        const double Lmin = fmin(bx.L[0], fmin(bx.L[1], bx.L[2]));
-        if (L.hs < Lmin * (1.0 / 4096.0)) { L.lo2 = -1.0f; L.hi2 = 3.0e38f; }
-    }
-    const float qh = __uint_as_float(qlo.w) * 1.00001f;
-    const float rad2 = qh * qh;
-    {
-        // relative coordinates from the bucket corner give exact minimum
-        // images while every candidate that can be inside lies within L/4
-        float ex = u2f(qhi.x - qlo.x) * bx.s[0], ey = u2f(qhi.y - qlo.y) * bx.s[1],
-              ez = u2f(qhi.z - qlo.z) * bx.s[2];
-        L.rel_ok = ex + 2.f * qh < 0.25f * (float)bx.L[0] && ey + 2.f * qh < 0.25f * (float)bx.L[1] &&
-                   ez + 2.f * qh < 0.25f * (float)bx.L[2];
-    }
-    int count = 0;
-    Row R;
-    R.out = nullptr;
-    R.lim = 0;
-    if (a.mode == 0) {
-        R.out = a.nbr_idx + (int64_t)L.s * a.cap;
-        R.lim = a.cap;
-    } else if (a.mode == 2) {
-        // storage was reserved in mode 1; a reservation that did not fit
-        // (the capacity flag is set and the host rebuilds) must not write
-        // past the buffer
-        const int64_t o = a.nbr_off[L.s];
-        R.out = a.nbr_idx + o;
-        R.lim = (int)max((int64_t)0, min(a.capacity - o, (int64_t)0x7fffffff));
-    }
-
-    int sp = 0;
-    int root = a.box_root[a.node_box[b]];
-    if (root < a.nbucket_total) {
-        // the whole box is one bucket
-        Cand cd;
-        const int rf = a.node_first[root], rc = a.node_cnt[root];
-        if (lane < rc) cand_load(a, rf + lane, cd);
-        __syncwarp();
-        const int kc = cand_stage(stage(0), lane < rc && cand_near(cd, qlo, qhi, bx, rad2), lane, cd,
-                                  rf + lane, ox, oy, oz, bx);
-        __syncwarp();
-        scan_stage(L, R, stage(0), bx, kc, count);
-    } else {
-        if (lane == 0) stack[0] = root;
-        sp = 1;
-    }
-    __syncwarp();
-    while (sp > 0) {
-        sp--;
-        int node = stack[sp];
-        __syncwarp();
-        const int nf = a.node_first[node], nc = a.node_cnt[node];
-        bool hit = false;
-        const int child = nf + lane;
-        uint4 clo = make_uint4(0, 0, 0, 0), chi = make_uint4(0, 0, 0, 0);
-        int cfirst = 0, ccnt = 0;
-        if (lane < nc) {
-            clo = a.lo[child];
-            chi = a.hi[child];
-            hit = boxes_near(qlo, qhi, clo, chi, bx, rad2);
-        }
-        unsigned m = __ballot_sync(0xffffffffu, hit);
-        if (nf < a.nbucket_total) {
-            // children are buckets: keep the ones some lane's sphere reaches,
-            // then stage bucket k+1 (global loads in flight) while scanning k
-            if (hit) { cfirst = a.node_first[child]; ccnt = a.node_cnt[child]; }
-            unsigned keep = 0;
-            unsigned mm = m;
-            while (mm) {
-                int k = __ffs(mm) - 1;
-                mm &= mm - 1;
-                uint4 blo, bhi;
-                blo.x = __shfl_sync(0xffffffffu, clo.x, k); blo.y = __shfl_sync(0xffffffffu, clo.y, k);
-                blo.z = __shfl_sync(0xffffffffu, clo.z, k);
-                bhi.x = __shfl_sync(0xffffffffu, chi.x, k); bhi.y = __shfl_sync(0xffffffffu, chi.y, k);
-                bhi.z = __shfl_sync(0xffffffffu, chi.z, k);
-                if (__any_sync(0xffffffffu, sphere_near(L, blo, bhi, bx))) keep |= 1u << k;
+    Tiles &W = tiles_all[warp];
+    const unsigned lt = (1u << lane) - 1u;
+    const int ol = lane & (OW - 1), slot = lane / OW;
+    const int64_t nb = MODE != LIST_ROWS && a.nq_dev ? (int64_t)*a.ovf_count : a.nbucket;
+    const int64_t nitem = nb * SPLIT;
+    for (int64_t item0 = blockIdx.x * (int64_t)LIST_WARPS; item0 < nitem;
+         item0 += gridDim.x * (int64_t)LIST_WARPS) {
+        const int64_t item = item0 + warp;
+        int64_t b = item / SPLIT;
+        const int sub = SPLIT > 1 ? (int)(item % SPLIT) * OW : 0;
+        const bool valid = item < nitem;
+        if (valid && MODE != LIST_ROWS) b = a.ovf_list[b];
+        const int bcnt = valid ? a.node_cnt[b] : 0;
+        bool over = false;
+        // (warp-uniform; the warps of a CTA meet at the end of LIST_ROWS)
+        if (bcnt > sub) {
+            const int f0 = a.node_first[b] + sub, nown = min(OW, bcnt - sub);
+            const int bid = a.node_box[b];
+            const Box bx = a.boxes[bid];
+            const uint4 corner = a.lo[b];
+            const uint32_t ox = corner.x, oy = corner.y, oz = corner.z;
+            const bool own = ol < nown;
+            const int s = f0 + min(ol, nown - 1);   // (the lanes past the owners repeat the last)
+            const uint32_t sqx = a.qx[s], sqy = a.qy[s], sqz = a.qz[s];
+            const double hs = a.hs[s];
+            const float hf = (float)hs;
+            const float rx = qdiff(ox, sqx, bx.s[0]), ry = qdiff(oy, sqy, bx.s[1]),
+                        rz = qdiff(oz, sqz, bx.s[2]);
+            // The owners' two boxes (fixed-point corners, largest radius).  A run
+            // of Morton-ordered particles that crosses a high-level cell
+            // boundary spans a box that may cover much of the domain; cut where
+            // consecutive owners differ in their highest coordinate bit, both
+            // parts are compact.
+            int cut;
+            {
+                const uint32_t nx = __shfl_down_sync(0xffffffffu, sqx, 1);
+                const uint32_t ny = __shfl_down_sync(0xffffffffu, sqy, 1);
+                const uint32_t nz = __shfl_down_sync(0xffffffffu, sqz, 1);
+                const uint32_t gap = lane < nown - 1 ? (sqx ^ nx) | (sqy ^ ny) | (sqz ^ nz) : 0u;
+                const uint32_t top = __reduce_max_sync(0xffffffffu, gap);
+                cut = __ffs(__ballot_sync(0xffffffffu, gap == top));   // owners [0, cut) and the rest
             }
-            if (!keep) continue;
-            int k = __ffs(keep) - 1;
-            keep &= keep - 1;
-            int cf = __shfl_sync(0xffffffffu, cfirst, k), cc = __shfl_sync(0xffffffffu, ccnt, k);
-            Cand cd;
-            if (lane < cc) cand_load(a, cf + lane, cd);
-            int buf = 0;
-            int kc = cand_stage(stage(buf), lane < cc && cand_near(cd, qlo, qhi, bx, rad2), lane, cd,
-                                cf + lane, ox, oy, oz, bx);
+            uint4 qlo, qhi;
             __syncwarp();
-            for (;;) {
-                int nk = keep ? __ffs(keep) - 1 : -1;
-                int nfst = 0, ncc = 0;
-                if (nk >= 0) {
-                    keep &= keep - 1;
-                    nfst = __shfl_sync(0xffffffffu, cfirst, nk);
-                    ncc = __shfl_sync(0xffffffffu, ccnt, nk);
-                    if (lane < ncc) cand_load(a, nfst + lane, cd);
+#pragma unroll
+            for (int t = 0; t < 2; t++) {
+                // (the lanes of the other part repeat one of this part's; a
+                // second part without owners repeats the last owner)
+                const int src = t == 0 ? min(lane, cut - 1) : max(lane, min(cut, nown - 1));
+                const uint32_t x = __shfl_sync(0xffffffffu, sqx, src);
+                const uint32_t y = __shfl_sync(0xffffffffu, sqy, src);
+                const uint32_t z = __shfl_sync(0xffffffffu, sqz, src);
+                const uint32_t r =
+                    __shfl_sync(0xffffffffu, __float_as_uint(__double2float_ru(hs)), src);
+                uint4 lo, hi;
+                lo.x = __reduce_min_sync(0xffffffffu, x); hi.x = __reduce_max_sync(0xffffffffu, x);
+                lo.y = __reduce_min_sync(0xffffffffu, y); hi.y = __reduce_max_sync(0xffffffffu, y);
+                lo.z = __reduce_min_sync(0xffffffffu, z); hi.z = __reduce_max_sync(0xffffffffu, z);
+                lo.w = hi.w = __reduce_max_sync(0xffffffffu, r);
+                if (lane == 0) { W.lo[t] = lo; W.hi[t] = hi; }
+                if (t == 0) { qlo = lo; qhi = hi; }
+                else {
+                    qlo.x = min(qlo.x, lo.x); qlo.y = min(qlo.y, lo.y); qlo.z = min(qlo.z, lo.z);
+                    qhi.x = max(qhi.x, hi.x); qhi.y = max(qhi.y, hi.y); qhi.z = max(qhi.z, hi.z);
+                    qlo.w = max(qlo.w, lo.w);
                 }
-                scan_stage(L, R, stage(buf), bx, kc, count);
-                if (nk < 0) break;
-                kc = cand_stage(stage(buf ^ 1), lane < ncc && cand_near(cd, qlo, qhi, bx, rad2), lane,
-                                cd, nfst + lane, ox, oy, oz, bx);
-                __syncwarp();
-                buf ^= 1;
             }
             __syncwarp();
-        } else {
-            int np = __popc(m);
-            if (sp + np > STACK) {
-                if (lane == 0) set_flag(a.cnt, ST_STACK);
-                break;
+            const float qh = __uint_as_float(qlo.w);
+            const float rad2 = (qh * 1.00001f) * (qh * 1.00001f);
+            const float Lmax = (float)fmax(bx.L[0], fmax(bx.L[1], bx.L[2]));
+            // Coordinates relative to the bucket's corner: their differences
+            // are one periodic image, the nearest one for every pair within
+            // the radius while the owners' box (seen from the corner) plus
+            // the radius stays below half a period; another image only makes
+            // a candidate look farther.
+            float big;
+            bool rel;
+            {
+                const float ex = u2f(qhi.x - ox) * bx.s[0], ey = u2f(qhi.y - oy) * bx.s[1],
+                            ez = u2f(qhi.z - oz) * bx.s[2];
+                big = fmaxf(ex, fmaxf(ey, ez)) + qh;
+                rel = ex + qh < 0.49f * (float)bx.L[0] && ey + qh < 0.49f * (float)bx.L[1] &&
+                      ez + qh < 0.49f * (float)bx.L[2];
             }
-            if (hit) stack[sp + __popc(m & ((1u << lane) - 1u))] = child;
-            sp += np;
+            // The band around hs^2 inside which a float distance does not
+            // decide: at r = hs the relative error of r^2 is at most 6.2e-7 X / hs
+            // (coordinates up to X rounded to 2^-24, their difference, three
+            // axes) + 8e-10 L / hs (positions cut to L / 2^32) + 5e-7 (the
+            // scale's, the squares' and the radius's rounding); two to three
+            // times that is taken.  Without relative coordinates X is the
+            // separation itself.
+            const float ihf = 1.f / hf;
+            const float eps = 2e-6f * (rel ? big : hf) * ihf + 2e-9f * Lmax * ihf + 1e-6f;
+            float lo2 = hf * hf * (1.0f - eps), hi2 = hf * hf * (1.0f + eps);
+            if (!(eps < 0.1f)) { lo2 = -1.0f; hi2 = 3.0e38f; }   // (every pair exactly)
+            // the boxes in relative coordinates, their reach widened likewise
+            if (lane < 2) {
+                const uint4 lo = W.lo[lane], hi = W.hi[lane];
+                const float x0 = u2f(lo.x - ox) * bx.s[0], x1 = u2f(hi.x - ox) * bx.s[0];
+                const float y0 = u2f(lo.y - oy) * bx.s[1], y1 = u2f(hi.y - oy) * bx.s[1];
+                const float z0 = u2f(lo.z - oz) * bx.s[2], z1 = u2f(hi.z - oz) * bx.s[2];
+                const float h = __uint_as_float(lo.w);
+                const float reach = h + (4e-6f * big + 2e-9f * Lmax + 1e-5f * h);
+                W.ctr[lane] = make_float4(0.5f * (x0 + x1), 0.5f * (y0 + y1), 0.5f * (z0 + z1),
+                                          reach * reach);
+                W.ext[lane] = make_float4(0.5f * (x1 - x0), 0.5f * (y1 - y0), 0.5f * (z1 - z0), 0.f);
+            }
             __syncwarp();
-        }
-    }
-    const bool own = L.own;
-    const int s = L.s;
+            int32_t *const row =
+                MODE == LIST_FILL ? a.nbr_idx + a.nbr_off[s] : a.nbr_idx + (int64_t)s * a.cap;
+            // (a reservation that did not fit -- the capacity flag is set and
+            // the host rebuilds -- must not write past the buffer)
+            const int lim = MODE == LIST_FILL
+                ? (int)max((int64_t)0, min(a.capacity - a.nbr_off[s], (int64_t)0x7fffffff))
+                : a.cap;
+            int count = 0;   // members of the owner's list so far
+            int head = 0, fill = 0;   // the ring's first tile (0 or 32) and candidates in it
 
-    if (a.mode == 2) return;
-    if (a.mode == 0) {
-        // each particle owns cap slots at s * cap; a longer list sends the
-        // whole bucket to the count-then-fill passes (overflow region)
-        unsigned over = __ballot_sync(0xffffffffu, own && count > a.cap);
-        if (over) {
-            if (lane == 0) a.ovf_list[atomicAdd(a.ovf_count, 1)] = (int32_t)b;
-            return;
+            // the members among the 32 candidates from `head`
+            auto test_tile = [&]() {
+                constexpr int PER = 32 / SPLIT;
+                const float4 *T = W.r + head + slot * PER;
+                unsigned in = 0, amb = 0;
+                if (rel) {
+#pragma unroll
+                    for (int k = 0; k < PER; k++) {
+                        const float4 c = T[k];
+                        const float dx = c.x - rx, dy = c.y - ry, dz = c.z - rz;
+                        const float r2 = dx * dx + dy * dy + dz * dz;
+                        if (r2 <= hi2) in |= 1u << k;
+                        if (r2 <= hi2 && r2 >= lo2) amb |= 1u << k;
+                    }
+                } else {
+#pragma unroll 4
+                    for (int k = 0; k < PER; k++) {
+                        const float4 c = T[k];
+                        const float dx = qdiff(sqx, __float_as_uint(c.x), bx.s[0]);
+                        const float dy = qdiff(sqy, __float_as_uint(c.y), bx.s[1]);
+                        const float dz = qdiff(sqz, __float_as_uint(c.z), bx.s[2]);
+                        const float r2 = dx * dx + dy * dy + dz * dz + c.w;
+                        if (r2 <= hi2) in |= 1u << k;
+                        if (r2 <= hi2 && r2 >= lo2) amb |= 1u << k;
+                    }
+                }
+                const int32_t *J = W.j + head + slot * PER;
+                while (amb) {   // within the float band: decide in double
+                    const int k = __ffs(amb) - 1;
+                    amb &= amb - 1;
+                    if (!list_exact(a, bx, s, J[k])) in &= ~(1u << k);
+                }
+                int pos = count, tot = __popc(in);
+                if (SPLIT > 1) {   // after the members the owner's lower lanes found
+                    const int mine = tot;
+                    tot = 0;
+#pragma unroll
+                    for (int t = 0; t < SPLIT; t++) {
+                        const int c = __shfl_sync(0xffffffffu, mine, t * OW + ol);
+                        if (t < slot) pos += c;
+                        tot += c;
+                    }
+                }
+                count += tot;
+                if (MODE != LIST_COUNT && own) {
+                    while (in) {
+                        const int k = __ffs(in) - 1;
+                        in &= in - 1;
+                        if (pos < lim) row[pos] = J[k];
+                        pos++;
+                    }
+                }
+                __syncwarp();
+                head ^= 32;
+                fill -= 32;
+            };
+
+            // one bucket's particles (lane k: particle cf + k): those near the
+            // owners' boxes join the ring
+            auto stage = [&](int cf, int cc, uint32_t px, uint32_t py, uint32_t pz) {
+                bool keep = false;
+                float4 c;
+                if (rel) {
+                    c = make_float4(qdiff(ox, px, bx.s[0]), qdiff(oy, py, bx.s[1]),
+                                    qdiff(oz, pz, bx.s[2]), 0.f);
+#pragma unroll
+                    for (int t = 0; t < 2; t++) {
+                        const float4 m = W.ctr[t], e = W.ext[t];
+                        const float gx = fmaxf(fabsf(c.x - m.x) - e.x, 0.f);
+                        const float gy = fmaxf(fabsf(c.y - m.y) - e.y, 0.f);
+                        const float gz = fmaxf(fabsf(c.z - m.z) - e.z, 0.f);
+                        keep |= gx * gx + gy * gy + gz * gz <= m.w;
+                    }
+                } else {
+                    c = make_float4(__uint_as_float(px), __uint_as_float(py), __uint_as_float(pz), 0.f);
+                    const float gx = u2f(point_gap(px, qlo.x, qhi.x)) * bx.s[0];
+                    const float gy = u2f(point_gap(py, qlo.y, qhi.y)) * bx.s[1];
+                    const float gz = u2f(point_gap(pz, qlo.z, qhi.z)) * bx.s[2];
+                    keep = gx * gx + gy * gy + gz * gz <= rad2;
+                }
+                keep = keep && lane < cc;
+                const unsigned m = __ballot_sync(0xffffffffu, keep);
+                if (keep) {
+                    const int at = (head + fill + __popc(m & lt)) & 63;
+                    W.r[at] = c;
+                    W.j[at] = cf + lane;
+                }
+                fill += __popc(m);
+                __syncwarp();
+                if (fill >= 32) test_tile();
+            };
+
+            const int root = a.box_root[bid];
+            int sp = 0;
+            __syncwarp();
+            if (root < a.nbucket_total) {
+                // the whole box is one bucket
+                const int rf = a.node_first[root], rc = a.node_cnt[root];
+                const int j = rf + min(lane, rc - 1);
+                stage(rf, rc, a.qx[j], a.qy[j], a.qz[j]);
+            } else {
+                if (lane == 0) W.stack[0] = root;
+                sp = 1;
+            }
+            __syncwarp();
+            while (sp > 0) {
+                sp--;
+                const int node = W.stack[sp];
+                __syncwarp();
+                const int nf = a.node_first[node], nc = a.node_cnt[node];
+                bool hit = false;
+                const int child = nf + lane;
+                if (lane < nc) {
+                    const uint4 clo = a.lo[child], chi = a.hi[child];
+#pragma unroll
+                    for (int t = 0; t < 2; t++) {
+                        const uint4 lo = W.lo[t];
+                        const float h = __uint_as_float(lo.w) * 1.00001f;
+                        hit |= boxes_near(lo, W.hi[t], clo, chi, bx, h * h);
+                    }
+                }
+                unsigned m = __ballot_sync(0xffffffffu, hit);
+                if (nf < a.nbucket_total) {
+                    // children are buckets: the next one's positions are in
+                    // flight while one is staged (and a tile tested)
+                    if (!m) continue;
+                    int cfirst = 0, ccnt = 0;
+                    if (hit) { cfirst = a.node_first[child]; ccnt = a.node_cnt[child]; }
+                    int k = __ffs(m) - 1;
+                    m &= m - 1;
+                    int cf = __shfl_sync(0xffffffffu, cfirst, k), cc = __shfl_sync(0xffffffffu, ccnt, k);
+                    int j = cf + min(lane, cc - 1);
+                    uint32_t px = a.qx[j], py = a.qy[j], pz = a.qz[j];
+                    for (;;) {
+                        const bool more = m != 0;
+                        k = more ? __ffs(m) - 1 : 0;
+                        m &= m - 1;
+                        const int cf1 = __shfl_sync(0xffffffffu, cfirst, k);
+                        const int cc1 = __shfl_sync(0xffffffffu, ccnt, k);
+                        uint32_t px1 = 0, py1 = 0, pz1 = 0;
+                        if (more) {
+                            j = cf1 + min(lane, cc1 - 1);
+                            px1 = a.qx[j]; py1 = a.qy[j]; pz1 = a.qz[j];
+                        }
+                        stage(cf, cc, px, py, pz);
+                        if (!more) break;
+                        cf = cf1; cc = cc1;
+                        px = px1; py = py1; pz = pz1;
+                    }
+                } else {
+                    const int np = __popc(m);
+                    if (sp + np > STACK) {
+                        if (lane == 0) set_flag(a.cnt, ST_STACK);
+                        break;
+                    }
+                    if (hit) W.stack[sp + __popc(m & lt)] = child;
+                    sp += np;
+                    __syncwarp();
+                }
+            }
+            if (fill > 0) {
+                // the last tile: the slots past its candidates hold points at
+                // infinity
+                if (lane >= fill) {
+                    W.r[head + lane] = rel ? make_float4(1.0e30f, 0.f, 0.f, 0.f)
+                                           : make_float4(0.f, 0.f, 0.f, INFINITY);
+                    W.j[head + lane] = 0;
+                }
+                __syncwarp();
+                test_tile();
+            }
+
+            if (MODE == LIST_ROWS) {
+                // each particle owns cap slots at s * cap; a longer list sends
+                // the whole bucket to the count-then-fill passes (which write
+                // nbr_off and nbr_cnt of all its particles)
+                over = __any_sync(0xffffffffu, own && count > a.cap);
+                if (own && slot == 0 && !over) {
+                    a.nbr_off[s] = (int64_t)s * a.cap;
+                    a.nbr_cnt[s] = count;
+                }
+            } else if (MODE == LIST_COUNT) {
+                // reserve storage in the overflow region for the warp's lists
+                const int mine = own && slot == 0 ? count : 0;
+                int incl = mine;
+                for (int o = 1; o < 32; o <<= 1) {
+                    int t = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += t;
+                }
+                const int total = __shfl_sync(0xffffffffu, incl, 31);
+                unsigned long long gbase = 0;
+                if (lane == 0) gbase = atomicAdd(&a.cnt->list_cursor, (unsigned long long)total);
+                gbase = __shfl_sync(0xffffffffu, gbase, 0);
+                const bool fits = (int64_t)gbase + total <= a.capacity;
+                if (!fits && lane == 0) set_flag(a.cnt, ST_LIST_CAPACITY);
+                if (own && slot == 0) {
+                    a.nbr_off[s] = (int64_t)gbase + (incl - mine);
+                    a.nbr_cnt[s] = fits ? mine : 0;   // (nothing stored for lists that do not fit)
+                }
+            }
         }
-        if (own) {
-            a.nbr_off[s] = (int64_t)s * a.cap;
-            a.nbr_cnt[s] = count;
+        if (MODE == LIST_ROWS) {
+            // a bucket is queued once, by the first of its warps
+            if (lane == 0) over_all[warp] = over;
+            if (SPLIT > 1) __syncthreads(); else __syncwarp();
+            if (valid && lane == 0 && warp % SPLIT == 0) {
+                int any = 0;
+                for (int t = 0; t < SPLIT; t++) any |= over_all[warp + t];
+                if (any) a.ovf_list[atomicAdd(a.ovf_count, 1)] = (int32_t)b;
+            }
+            if (SPLIT > 1) __syncthreads();
         }
-        return;
-    }
-    // mode 1: reserve storage in the overflow region for the warp's lists
-    int mine = own ? count : 0;
-    int incl = mine;
-    for (int o = 1; o < 32; o <<= 1) {
-        int t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
-    }
-    int total = __shfl_sync(0xffffffffu, incl, 31);
-    unsigned long long gbase = 0;
-    if (lane == 0) gbase = atomicAdd(&a.cnt->list_cursor, (unsigned long long)total);
-    gbase = __shfl_sync(0xffffffffu, gbase, 0);
-    int64_t start = (int64_t)gbase + (incl - mine);
-    if (own) {
-        a.nbr_off[s] = start;
-        a.nbr_cnt[s] = mine;
-    }
-    if ((int64_t)gbase + total > a.capacity) {
-        if (lane == 0) set_flag(a.cnt, ST_LIST_CAPACITY);
-        if (own) a.nbr_cnt[s] = 0;   // nothing stored for these lists
     }
 }
 
@@ -894,7 +968,7 @@ cudaError_t raise_tree(hydro_ctx *c, stream_t st) {
     return cudaSuccess;
 }
 
-static ListArgs list_args(hydro_ctx *c, int cap, int mode) {
+static ListArgs list_args(hydro_ctx *c, int cap) {
     // cap: slots per particle in the fixed-stride part of nbr_idx
     const Plan &P = c->plan;
     ListArgs a;
@@ -916,17 +990,24 @@ static ListArgs list_args(hydro_ctx *c, int cap, int mode) {
     a.capacity = (int64_t)c->d_nbr_idx.cap;
     a.cnt = c->d_cnt;
     a.cap = cap;
-    a.mode = mode;
     a.ovf_list = c->d_ovf.get();
     a.ovf_count = &c->d_cnt->ovf_buckets;
     a.nq_dev = false;
     return a;
 }
 
+// warps a bucket is divided among: one while that fills the GPU (24 warps
+// on each of the 152 SMs), else four
+static int list_split(int64_t nbucket) { return nbucket >= 152 * 24 ? 1 : 4; }
+
+template <int MODE>
 static cudaError_t launch_lists(const ListArgs &a, int64_t nbucket, stream_t st) {
-    size_t per_warp = STACK * 4 + 2 * STAGE_BYTES;
-    size_t smem = per_warp * LIST_WARPS;
-    k_build_lists<<<grid_for(nbucket, LIST_WARPS), LIST_WARPS * 32, smem, st>>>(a);
+    // the queue's length on the device: a grid of 8 CTAs per SM strides over it
+    const int split = a.nq_dev ? 4 : list_split(nbucket);
+    const int64_t ctas = (nbucket * split + LIST_WARPS - 1) / LIST_WARPS;
+    const unsigned grid = (unsigned)(a.nq_dev ? std::min<int64_t>(ctas, 152 * 8) : ctas);
+    if (split == 1) k_build_lists<MODE, 1><<<grid, LIST_WARPS * 32, 0, st>>>(a);
+    else k_build_lists<MODE, 4><<<grid, LIST_WARPS * 32, 0, st>>>(a);
     return launch_check();
 }
 
@@ -944,26 +1025,24 @@ cudaError_t build_lists(hydro_ctx *c, int cap, stream_t st) {
     c->list_cap = cap;
     HYD_CUDA(set_u64(&c->d_cnt->list_cursor, (unsigned long long)n * cap, st));
     HYD_CUDA(cudaMemsetAsync(&c->d_cnt->ovf_buckets, 0, sizeof(int), st));
-    return launch_lists(list_args(c, cap, 0), c->plan.nbucket, st);
+    return launch_lists<LIST_ROWS>(list_args(c, cap), c->plan.nbucket, st);
 }
 
 // the queued buckets: count and reserve in the overflow region, then fill
 cudaError_t build_lists_queued(hydro_ctx *c, int nq, stream_t st) {
-    ListArgs a = list_args(c, c->list_cap, 1);
+    ListArgs a = list_args(c, c->list_cap);
     a.nbucket = nq;   // warps index the queue
-    HYD_CUDA(launch_lists(a, nq, st));
-    a.mode = 2;
-    return launch_lists(a, nq, st);
+    HYD_CUDA(launch_lists<LIST_COUNT>(a, nq, st));
+    return launch_lists<LIST_FILL>(a, nq, st);
 }
 
 // the queued passes over as many warps as there are buckets; the count of
 // queued buckets is read by the warps themselves
 cudaError_t build_lists_queued_dev(hydro_ctx *c, stream_t st) {
-    ListArgs a = list_args(c, c->list_cap, 1);
+    ListArgs a = list_args(c, c->list_cap);
     a.nq_dev = true;
-    HYD_CUDA(launch_lists(a, c->plan.nbucket, st));
-    a.mode = 2;
-    return launch_lists(a, c->plan.nbucket, st);
+    HYD_CUDA(launch_lists<LIST_COUNT>(a, c->plan.nbucket, st));
+    return launch_lists<LIST_FILL>(a, c->plan.nbucket, st);
 }
 
 cudaError_t rebuild_active_lists_dev(hydro_ctx *c, stream_t st, bool guard) {

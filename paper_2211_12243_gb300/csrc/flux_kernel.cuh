@@ -26,6 +26,7 @@
 #include "hydro_internal.cuh"
 #include "pairgeom.cuh"
 #include "riemann.cuh"
+#include "riemann_f64.cuh"
 #include "mlp.cuh"
 
 namespace hyd {
@@ -164,7 +165,7 @@ __device__ __forceinline__ bool member_j(float r2, float hjf, const FluxArgs &a,
 }
 __device__ __forceinline__ bool member_j(double r2, double hj, const FluxArgs &, int64_t,
                                          int64_t, const Box &) {
-    return r2 < __dmul_rn(hj, hj);
+    return dlt_pos(r2, __dmul_rn(hj, hj));
 }
 
 struct FaceStats {
@@ -271,6 +272,117 @@ __device__ __forceinline__ bool face_state(const FluxArgs &a, const GasK<R> &K, 
     return true;
 }
 
+// W(r, h) with ih = 1/h
+__device__ __forceinline__ double kernel64(int kernel, double r, double ih) {
+    const double q = r * ih;
+    double w = 0.0;
+    if (dlt_pos(q, 1.0)) {
+        const double t = 1.0 - q, t2 = t * t;
+        if (kernel == 0) w = t2 * t2 * fma(4.0, q, 1.0);
+        else if (dlt_pos(0.5, q)) w = 2.0 * t2 * t;
+        else w = fma(6.0 * q * q, q - 1.0, 1.0);
+    }
+    const double kn = kernel == 0 ? 21.0 / (2.0 * 3.14159265358979323846) : 8.0 / 3.14159265358979323846;
+    return (kn * (ih * ih)) * (ih * w);
+}
+
+// face_state in FP64: the same face, states and limiters with the FP64
+// instructions that differ between the two sides of a face only once (the
+// pairwise limiter's bounds are symmetric in the two cells), comparisons on
+// the integer pipe and the divisions of fp64.cuh
+__device__ __forceinline__ bool face_state64(const FluxArgs &a, const GasK<double> &K,
+                                             const double *ri, const double *rj, const double d[3],
+                                             double r, double dt, double hl, double hr,
+                                             FaceState<double> &st, FaceStats &fs) {
+    const double oo = ri[R_OM] * rj[R_OM];
+    const double wi = oo * kernel64(a.kernel, r, rcp64(ri[R_H]));
+    const double wj = oo * kernel64(a.kernel, r, rcp64(rj[R_H]));
+    const double *Bi = ri + R_B, *Bj = rj + R_B;
+    double A[3];
+    A[0] = fma(fma(Bi[0], d[0], fma(Bi[1], d[1], Bi[2] * d[2])), wi,
+               fma(Bj[0], d[0], fma(Bj[1], d[1], Bj[2] * d[2])) * wj);
+    A[1] = fma(fma(Bi[1], d[0], fma(Bi[3], d[1], Bi[4] * d[2])), wi,
+               fma(Bj[1], d[0], fma(Bj[3], d[1], Bj[4] * d[2])) * wj);
+    A[2] = fma(fma(Bi[2], d[0], fma(Bi[4], d[1], Bi[5] * d[2])), wi,
+               fma(Bj[2], d[0], fma(Bj[4], d[1], Bj[5] * d[2])) * wj);
+    const double A2 = fma(A[0], A[0], fma(A[1], A[1], A[2] * A[2]));
+    if (!dpos(A2)) return false;
+    const double inA = rsqrt64(A2);
+    st.sA = dt * (A2 * inA);
+    st.nh[0] = A[0] * inA; st.nh[1] = A[1] * inA; st.nh[2] = A[2] * inA;
+
+    double Lf[5], Rf[5];
+    const double *Gi = ri + R_G, *Gj = rj + R_G;
+    const double hd[3] = {0.5 * d[0], 0.5 * d[1], 0.5 * d[2]};
+#pragma unroll
+    for (int f = 0; f < 5; f++) {
+        const double u = ri[R_RHO + f], v = rj[R_RHO + f];
+        double l = u + fma(hd[0], Gi[3 * f], fma(hd[1], Gi[3 * f + 1], hd[2] * Gi[3 * f + 2]));
+        double m = v - fma(hd[0], Gj[3 * f], fma(hd[1], Gj[3 * f + 1], hd[2] * Gj[3 * f + 2]));
+        if (a.limiter) {
+            // the values between the cells' by more than psi1 d, or past the
+            // mean by more than psi2 d towards the far cell (pair_limit)
+            const bool up = dlt(u, v);   // the owner's cell holds the lower value
+            const double lo = up ? u : v, hi = up ? v : u;
+            const double df = hi - lo, mean = 0.5 * (u + v);
+            double lox = fma(-a.psi1, df, lo), hix = fma(a.psi1, df, hi);
+            if ((f == 0 || f == 4) && !(dpos(lo) && dpos(lox))) {
+                // (a value that is not positive, or a bound that changes sign)
+                const double d1 = a.psi1 * df;
+                if (sgn_(lox) != sgn_(lo)) lox = lo == 0.0 ? 0.0 : lo / (1.0 + d1 / fabs(lo));
+                if (sgn_(hix) != sgn_(hi)) hix = hi == 0.0 ? 0.0 : hi / (1.0 + d1 / fabs(hi));
+            }
+            // the side with the lower value is held in [lox, mean + psi2 d],
+            // the other in [mean - psi2 d, hix]
+            const double low = up ? l : m, high = up ? m : l;
+            const double lo2 = dmax_(dmin_(low, fma(a.psi2, df, mean)), lox);
+            const double hi2 = dmin_(dmax_(high, fma(-a.psi2, df, mean)), hix);
+            l = up ? lo2 : hi2;
+            m = up ? hi2 : lo2;
+            if (dbits(u) == dbits(v)) l = m = u;
+        }
+        Lf[f] = l;
+        Rf[f] = m;
+    }
+    double av[3] = {0.0, 0.0, 0.0};
+    if (a.time_extrap) {
+        const double di = hl * (Gi[3] + Gi[7] + Gi[11]), dj = hr * (Gj[3] + Gj[7] + Gj[11]);
+        Lf[0] = fma(-di, ri[R_RHO], Lf[0]);
+        Rf[0] = fma(-dj, rj[R_RHO], Rf[0]);
+        const double iri = hl * rcp64(ri[R_RHO]), irj = hr * rcp64(rj[R_RHO]);
+#pragma unroll
+        for (int q = 0; q < 3; q++) {
+            const double ai = Gi[12 + q] * iri, aj = Gj[12 + q] * irj;
+            Lf[1 + q] -= ai;
+            Rf[1 + q] -= aj;
+            av[q] = ai + aj;
+        }
+        Lf[4] = fma(-di, K.g * ri[R_P], Lf[4]);
+        Rf[4] = fma(-dj, K.g * rj[R_P], Rf[4]);
+    }
+    if (!(dpos(Lf[0]) && dpos(Lf[4]) && dpos(Rf[0]) && dpos(Rf[4]))) {
+#pragma unroll
+        for (int f = 0; f < 5; f++) { Lf[f] = ri[R_RHO + f]; Rf[f] = rj[R_RHO + f]; }
+        fs.first_order++;
+    }
+    double vl[3], vr[3];
+#pragma unroll
+    for (int q = 0; q < 3; q++) {
+        st.vf[q] = 0.5 * ((ri[R_VX + q] + rj[R_VX + q]) - av[q]);
+        vl[q] = Lf[1 + q] - st.vf[q];
+        vr[q] = Rf[1 + q] - st.vf[q];
+    }
+    st.ul = fma(vl[0], st.nh[0], fma(vl[1], st.nh[1], vl[2] * st.nh[2]));
+    st.ur = fma(vr[0], st.nh[0], fma(vr[1], st.nh[1], vr[2] * st.nh[2]));
+#pragma unroll
+    for (int q = 0; q < 3; q++) {
+        st.wl[q] = fma(-st.ul, st.nh[q], vl[q]);
+        st.wr[q] = fma(-st.ur, st.nh[q], vr[q]);
+    }
+    st.rl = Lf[0]; st.pl = Lf[4]; st.rr = Rf[0]; st.pr = Rf[4];
+    return true;
+}
+
 // Toro's adaptive guess falls back to the two-shock value on this face (the
 // same tests as star_guess: not the PVRS value, and p_PVRS >= p_min so not
 // the two-rarefaction value, which is exact for two rarefactions).  These
@@ -300,7 +412,10 @@ __device__ __forceinline__ void face_finish(const FluxArgs &a, const GasK<R> &K,
     R F[5];
     if (RIEM == HYDRO_RIEMANN_HLLC) {
         R ps, ss;
-        hllc_flux<R>(K, rl, ul, pl, wl, rr, ur, pr, wr, nh, F, ps, ss);
+        if constexpr (sizeof(R) == 8)
+            hllc_flux64<SCHEME == HYDRO_MFM>(K, rl, ul, pl, wl, rr, ur, pr, wr, nh, F, ps, ss);
+        else
+            hllc_flux<R>(K, rl, ul, pl, wl, rr, ur, pr, wr, nh, F, ps, ss);
         if (SCHEME == HYDRO_MFM) {
             F[0] = R(0);
             F[1] = ps * nh[0]; F[2] = ps * nh[1]; F[3] = ps * nh[2];
@@ -309,10 +424,18 @@ __device__ __forceinline__ void face_finish(const FluxArgs &a, const GasK<R> &K,
     } else {
         R ps, us;
         R tol = sizeof(R) == 8 ? (R)a.p_tol : (R)a.ptolf;
-        const GasK<double> *kd = sizeof(R) == 4 && a.riemann_polish ? &a.Kd : nullptr;
-        const R cl = sqrt_(div_(K.g * pl, rl)), cr = sqrt_(div_(K.g * pr, rr));
-        StarOut so = star_solve<R>(K, rl, ul, pl, cl, rr, ur, pr, cr, p0, tol, a.max_newton, ps, us,
-                                   kd);
+        R cl, cr;
+        StarOut so;
+        if constexpr (sizeof(R) == 8) {
+            cl = sqrt64(K.g * pl * rcp64(rl));
+            cr = sqrt64(K.g * pr * rcp64(rr));
+            so = star_solve64(K, a.Kf, rl, ul, pl, cl, rr, ur, pr, cr, tol, a.max_newton, ps, us);
+        } else {
+            const GasK<double> *kd = a.riemann_polish ? &a.Kd : nullptr;
+            cl = sqrt_(div_(K.g * pl, rl));
+            cr = sqrt_(div_(K.g * pr, rr));
+            so = star_solve<R>(K, rl, ul, pl, cl, rr, ur, pr, cr, p0, tol, a.max_newton, ps, us, kd);
+        }
         fs.iters += so.iters;
         if (so.vacuum) { fs.vacuum++; return; }
         ps_out = ps;
@@ -323,7 +446,10 @@ __device__ __forceinline__ void face_finish(const FluxArgs &a, const GasK<R> &K,
         } else {
             R rs, uu, pp;
             int side;
-            star_sample<R>(K, rl, ul, pl, cl, rr, ur, pr, cr, ps, us, rs, uu, pp, side);
+            if constexpr (sizeof(R) == 8)
+                star_sample64(K, a.Kf, rl, ul, pl, cl, rr, ur, pr, cr, ps, us, rs, uu, pp, side);
+            else
+                star_sample<R>(K, rl, ul, pl, cl, rr, ur, pr, cr, ps, us, rs, uu, pp, side);
             R w0 = side < 0 ? wl[0] : wr[0];
             R w1 = side < 0 ? wl[1] : wr[1];
             R w2 = side < 0 ? wl[2] : wr[2];
@@ -586,7 +712,12 @@ k_fluxes(FluxArgs a, const R *__restrict__ rec) {
                     hl = (R)(a.toff[so] + 0.5 * dtd);
                     hr = (R)(a.toff[j] + 0.5 * dtd);
                 }
-                if (face_state<R>(a, K, ri, rj, d, sqrt_(r2), dtf, hl, hr, st, fs)) {
+                bool face;
+                if constexpr (sizeof(R) == 8)
+                    face = face_state64(a, K, ri, rj, d, sqrt64(r2), dtf, hl, hr, st, fs);
+                else
+                    face = face_state<R>(a, K, ri, rj, d, sqrt_(r2), dtf, hl, hr, st, fs);
+                if (face) {
                     bool deferred = false;
                     if constexpr (DEFER) {
                         // hard faces are queued for the learned-guess pass,

@@ -1,0 +1,94 @@
+// FP64 arithmetic for a GPU whose FP64 pipe is narrow.  GB300 issues a
+// double-precision instruction of a warp in 16 cycles per SM against a
+// quarter of a cycle in FP32, so the FP64 kernels are bound by the number of
+// FP64 instructions alone.  Comparisons are done on the bit patterns (integer
+// pipe), and reciprocals and reciprocal square roots start from the special
+// function unit's 20-bit approximations, refined by one third-order
+// (Householder) step from the defining equation: three FP64 instructions for
+// a reciprocal and five for a reciprocal square root, to about one unit in
+// the last place, instead of a division or square root rounded correctly.
+#pragma once
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+namespace hyd {
+
+__device__ __forceinline__ long long dbits(double v) { return __double_as_longlong(v); }
+
+// 0 < v (v not NaN), without the FP64 pipe
+__device__ __forceinline__ bool dpos(double v) {
+    return (unsigned long long)(dbits(v) - 1) < 0x7ff0000000000000ull;
+}
+
+// v < 0 (neither -0 nor NaN)
+__device__ __forceinline__ bool dneg(double v) {
+    const unsigned long long b = (unsigned long long)dbits(v);
+    return b > 0x8000000000000000ull && b <= 0xfff0000000000000ull;
+}
+
+// integer with the order of the doubles (-0 just below +0; NaN beyond infinity)
+__device__ __forceinline__ long long dkey(double v) {
+    const long long b = dbits(v);
+    return b ^ (long long)((unsigned long long)(b >> 63) >> 1);
+}
+__device__ __forceinline__ bool dlt(double a, double b) { return dkey(a) < dkey(b); }
+// a < b for a, b >= 0 (false when a is NaN)
+__device__ __forceinline__ bool dlt_pos(double a, double b) {
+    return (unsigned long long)dbits(a) < (unsigned long long)dbits(b);
+}
+__device__ __forceinline__ double dmin_(double a, double b) { return dlt(b, a) ? b : a; }
+__device__ __forceinline__ double dmax_(double a, double b) { return dlt(a, b) ? b : a; }
+__device__ __forceinline__ double dabs_(double v) {
+    return __longlong_as_double(dbits(v) & 0x7fffffffffffffffll);
+}
+
+__device__ __forceinline__ double rcp_seed(double x) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    return r;
+}
+__device__ __forceinline__ double rsqrt_seed(double x) {
+    double r;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    return r;
+}
+
+// 1 / x: with e = 1 - x r, 1 / x = r / (1 - e) = r (1 + e + e^2) + O(e^3)
+__device__ __forceinline__ double rcp64(double x) {
+    const double r = rcp_seed(x);
+    const double e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
+
+// 1 / x to about 2^-40 (one Newton step): for factors of small corrections
+__device__ __forceinline__ double rcp40(double x) {
+    const double r = rcp_seed(x);
+    return fma(r, fma(-x, r, 1.0), r);
+}
+
+// 1 / sqrt(x), x > 0: with e = 1 - x r^2, (1 - e)^(-1/2) = 1 + e/2 + 3 e^2/8 + O(e^3)
+__device__ __forceinline__ double rsqrt64(double x) {
+    const double r = rsqrt_seed(x);
+    const double e = fma(-x * r, r, 1.0);
+    return fma(r, e * fma(0.375, e, 0.5), r);
+}
+
+// sqrt(x) (0 where x is not positive), with a final correction of the residual
+__device__ __forceinline__ double sqrt64(double x) {
+    const double r = rsqrt64(x);
+    const double s = x * r;
+    return dpos(x) ? fma(fma(-s, s, x), 0.5 * r, s) : 0.0;
+}
+
+// t^n, n >= 1 uniform over the warp
+__device__ __forceinline__ double ipow64(double t, int n) {
+    double r = (n & 1) ? t : 1.0;
+    for (n >>= 1; n > 0; n >>= 1) {
+        t *= t;
+        if (n & 1) r *= t;
+    }
+    return r;
+}
+
+}  // namespace hyd

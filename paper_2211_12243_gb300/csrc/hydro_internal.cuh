@@ -488,11 +488,15 @@ namespace hyd {
 
 __device__ __forceinline__ void set_flag(DevCounters *c, int bit) { atomicOr(&c->flags, bit); }
 
-// one fold of a separation into [-L/2, L/2]; exact IEEE operations only
+// one fold of a separation into [-L/2, L/2]; exact IEEE operations only.
+// |d| is compared with L/2 on the bit patterns (integer pipe: a comparison in
+// FP64 costs as much as an addition); L/2 is L with its exponent one lower.
 __device__ __forceinline__ double fold64(double d, double L) {
-    double half = __dmul_rn(0.5, L);
-    if (d > half) return __dsub_rn(d, L);
-    if (d < -half) return __dadd_rn(d, L);
+    const long long b = __double_as_longlong(d);
+    const long long half = __double_as_longlong(L) - (1ll << 52);
+    if ((b & 0x7fffffffffffffffll) > half)
+        return __dadd_rn(d, __longlong_as_double(__double_as_longlong(L) |
+                                                 (~b & (long long)0x8000000000000000ull)));
     return d;
 }
 

@@ -2,6 +2,7 @@
 // from their records, and exact membership r_ij < h.
 #pragma once
 
+#include "fp64.cuh"
 #include "hydro_internal.cuh"
 
 namespace hyd {
@@ -59,8 +60,8 @@ struct Member {
         if (r2 > hi2) return false;
         return exact(j);
     }
-    // double path: r2 is already the exact value
-    __device__ __forceinline__ bool operator()(double r2, int64_t) const { return r2 < h2; }
+    // double path: r2 is already the exact value (r2, h2 >= 0)
+    __device__ __forceinline__ bool operator()(double r2, int64_t) const { return dlt_pos(r2, h2); }
 };
 
 }  // namespace hyd

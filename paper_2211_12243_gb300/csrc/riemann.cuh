@@ -4,6 +4,7 @@
 // FP64 path, float for the mixed path.
 #pragma once
 
+#include "fp64.cuh"
 #include "hydro_internal.cuh"
 
 namespace hyd {
@@ -35,6 +36,11 @@ struct GasK {
     R g2;     // (g+1)/(2g)
     R inv_g;  // 1/g
     R mzr;    // -(g+1)/(2g)
+    // FP64 solver: (g+1)/2; the coefficients of (1 + w)^z = 1 + z w + c2 w^2 +
+    // c3 w^3; 1/z and 2/(g-1) where they are integers (g = 5/3: 5 and 3; 7/5: 7
+    // and 5), else 0
+    R ig5, c2, c3;
+    int nz, n4;
     GasK() = default;
     __host__ __device__ explicit GasK(double gamma) {
         g = (R)gamma;
@@ -48,6 +54,15 @@ struct GasK {
         g2 = (R)((gamma + 1.0) / (2.0 * gamma));
         inv_g = (R)(1.0 / gamma);
         mzr = (R)(-(gamma + 1.0) / (2.0 * gamma));
+        const double zd = (gamma - 1.0) / (2.0 * gamma), i = 1.0 / zd, j = 2.0 / (gamma - 1.0);
+        ig5 = (R)(0.5 * (gamma + 1.0));
+        c2 = (R)(0.5 * zd * (zd - 1.0));
+        c3 = (R)(zd * (zd - 1.0) * (zd - 2.0) / 6.0);
+        const long ni = i < 16.5 ? (long)(i + 0.5) : 0, nj = j < 14.5 ? (long)(j + 0.5) : 0;
+        const double ei = i - (double)ni, ej = j - (double)nj;
+        const bool whole = ni >= 1 && nj >= 1 && ei < 1e-13 && ei > -1e-13 && ej < 1e-13 && ej > -1e-13;
+        nz = whole ? (int)ni : 0;
+        n4 = whole ? (int)nj : 0;
     }
 };
 

@@ -9,11 +9,14 @@
 // clamped.  The list covers every j with r < h_search, so g is exact for
 // any h <= h_search; a root beyond h_search is reported for a re-search.
 //
-// FP64 path: everything in double.  Mixed path: the Newton iteration runs in
-// float on the fixed-point separations, then one Newton step evaluated in
-// double-float (pairs of floats, Dekker/Knuth error-free transformations)
-// on the exact 64-bit separations refines h to double-class accuracy
-// without the GPU's scarce FP64 pipe; omega is taken from that evaluation.
+// Both paths iterate in float on the fixed-point separations.  FP64 path: the iteration is then
+// finished in double by a third-order (Halley) step -- g and g' summed in
+// double, g'', which only scales the square of the step, in float -- so that
+// one pass over the list in double is enough.  Mixed path: one Newton step
+// evaluated in double-float (pairs of floats, Dekker/Knuth error-free
+// transformations) on the exact 64-bit separations refines h to double-class
+// accuracy without the GPU's scarce FP64 pipe; omega is taken from that
+// evaluation.
 //
 // Tight lists (hydro_step only): once an upper bracket hi of the root is
 // known, no later iterate exceeds it, so the particle's list is compacted in
@@ -24,6 +27,7 @@
 // exactly on every entry, then walk only the members.  Compaction keeps the
 // order of the entries, so the members are summed in the same order as in
 // the full list.
+#include "fp64.cuh"
 #include "hydro_internal.cuh"
 #include "tile_rank.cuh"
 
@@ -38,6 +42,7 @@ struct DensArgs {
     int32_t *nbr_idx;
     double *hs;               // lowered to the compacted lists' radius
     const double *xs, *ys, *zs;
+    const uint32_t *qx, *qy, *qz;
     const int32_t *pbox;
     const Box *boxes;
     uint8_t *active;          // bit0: solve this particle; bit1: search failed
@@ -52,9 +57,8 @@ struct DensArgs {
     double *om;               // sorted out
     DevCounters *cnt;
     bool rank;                // full solve: rank the CTA's 128 particles by list length
-    const int32_t *list;      // a guard round: only these particles (the round's guard
-    const int *nlist;         // list, count on the device), taken by the warps 32 at a
-    int *cursor;              // time from a global cursor
+    const int32_t *list;      // the guard round's particles, their count on the device
+    const int *nlist;         // (k_density_list)
 };
 
 // Growth of the search radius hs after a failed solve.  First failure
@@ -66,96 +70,6 @@ __device__ __forceinline__ double search_growth(double N, double kf, double hs, 
     if (!(hs <= 1.3 * h)) return 2.0;
     double g = kf > 0.0 ? 1.1 * cbrt(N / kf) : 2.0;
     return fmin(fmax(g, 1.05), 2.0);
-}
-
-// ---------------------------------------------------------------- FP64 path
-__global__ void k_density_f64(DensArgs a, double *__restrict__ rec) {
-    int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (s >= a.n) return;
-    if (a.only_active && !(a.active[s] & 1)) return;
-    const Box bx = a.boxes[a.pbox[s]];
-    const double xi = a.xs[s], yi = a.ys[s], zi = a.zs[s];
-    double hsi = a.hs[s];
-    const double N = a.nngb ? a.nngb[s] : a.n_ngb;
-    const int64_t o = a.nbr_off[s];
-    int32_t *idx = a.nbr_idx + o;
-    int c = a.nbr_cnt[s];
-    const double Kn = kernel_Kn<double>(a.kernel);
-    double h = a.h[s];
-    if (!(h > 0.0) || h > hsi) h = hsi;
-    double lo = 0.0, hi = -1.0;
-    bool conv = false, fail = false;
-    double kf_fail = 0.0;   // N_enc(hsi) = Kn sum f at a failure
-    auto sep = [&](int j) {
-        double dx = fold64(a.xs[j] - xi, bx.L[0]);
-        double dy = fold64(a.ys[j] - yi, bx.L[1]);
-        double dz = fold64(a.zs[j] - zi, bx.L[2]);
-        return sqrt(dx * dx + dy * dy + dz * dz);
-    };
-    for (int it = 1; it <= a.max_iter; it++) {
-        double f = 0.0, mq = 0.0, ih = 1.0 / h;
-        // an upper bracket well inside the list radius: drop the entries
-        // beyond it (relative slack 1e-9 >> the rounding of r)
-        const bool shrink = a.compact && hi > 0.0 && hi < 0.8 * hsi;
-        const double keep = hi * (1.0 + 1e-9);
-        int w = 0;
-        for (int k = 0; k < c; k++) {
-            const int j = idx[k];
-            const double r = sep(j);
-            if (shrink && r < keep) idx[w++] = j;
-            double fv, mv;
-            kernel_f<double>(a.kernel, r * ih, fv, mv);
-            f += fv;
-            mq += mv;
-        }
-        if (shrink) { c = w; hsi = hi * (1.0 + 5e-10); }   // complete below this
-        double g = Kn * f - N;
-        double dg = Kn * mq * ih;
-        if (g == 0.0) { conv = true; break; }
-        if (g < 0.0) {
-            if (h >= hsi) { fail = true; kf_fail = Kn * f; break; }
-            lo = fmax(lo, h);
-        } else {
-            hi = (hi < 0.0 || h < hi) ? h : hi;
-        }
-        double hn = dg > 0.0 ? h - g / dg : -1.0;
-        if (hn > 0.0 && fabs(hn - h) <= a.tol * h && hn <= hsi) { h = hn; conv = true; break; }
-        if (hi < 0.0) {
-            if (!(hn > lo) || hn > 2.0 * h) hn = 2.0 * h;
-            if (hn > hsi) hn = hsi;
-        } else if (!(hn > lo && hn < hi)) {
-            hn = 0.5 * (lo + hi);
-        }
-        h = hn;
-    }
-    if (fail) {   // (no compaction happened: failing needs h >= hsi, below any bracket)
-        a.hs[s] = hsi * search_growth(N, kf_fail, hsi, a.h[s]);
-        a.active[s] = (a.active[s] & ACT_GUARD) | 3;
-        atomicAdd(&a.cnt->search_fail, 1);
-        set_flag(a.cnt, ST_SEARCH);
-        return;
-    }
-    if (!conv) set_flag(a.cnt, ST_NOCONV_H);
-    double sw = 0.0, ih = 1.0 / h;
-    const double keep = h * (1.0 + 1e-9);
-    int w = 0;
-    for (int k = 0; k < c; k++) {
-        const int j = idx[k];
-        const double r = sep(j);
-        if (a.compact && r < keep) idx[w++] = j;
-        sw += kernel_shape<double>(a.kernel, r * ih);
-    }
-    if (a.compact) {
-        // complete for every r < h (1 + 5e-10)
-        a.nbr_cnt[s] = w;
-        a.hs[s] = h * (1.0 + 5e-10);
-    }
-    sw *= kernel_norm<double>(a.kernel, h);
-    double om = 1.0 / sw;
-    a.h[s] = h;
-    a.om[s] = om;
-    rec[s * REC + R_H] = h;
-    rec[s * REC + R_OM] = om;
 }
 
 // ------------------------------------------------------- double-float tools
@@ -223,77 +137,170 @@ __device__ __forceinline__ df from_i64(long long v) {
     return df_add(s, {i2f_small(lo), 0.f});
 }
 
-// ---------------------------------------------------------------- mixed path
+// ------------------------------------------------- the iteration in float
 constexpr int DENS_THREADS = 128;
 static_assert(DENS_THREADS == RANK_THREADS, "the ranked tiles take 128 threads a round");
+// separations a warp that walks one list keeps in shared memory
+constexpr int DENS_CACHE = 1536;
 
-// one particle's float Newton solve, then the double-float refinement
-__device__ __forceinline__ void dens_one(const DensArgs &a, const uint64_t *__restrict__ q64x,
-                                         const uint64_t *__restrict__ q64y,
-                                         const uint64_t *__restrict__ q64z,
-                                         float *__restrict__ rec, int64_t s) {
-    if (s >= a.n) return;
-    if (a.only_active && !(a.active[s] & 1)) return;
-    const Box bx = a.boxes[a.pbox[s]];
-    const float *ri = rec + s * REC;
-    const uint32_t qxi = __float_as_uint(ri[R_X]), qyi = __float_as_uint(ri[R_Y]),
-                   qzi = __float_as_uint(ri[R_Z]);
-    const double hsi_d = a.hs[s];
-    float hsi = (float)hsi_d;
-    const float N = (float)(a.nngb ? a.nngb[s] : a.n_ngb);
-    const int64_t o = a.nbr_off[s];
-    int32_t *idx = a.nbr_idx + o;
-    int c = a.nbr_cnt[s];
-    const float Kn = kernel_Kn<float>(a.kernel);
-    float h = (float)a.h[s];
-    if (!(h > 0.f) || h > hsi) h = hsi;
-    float lo = 0.f, hi = -1.f;
-    bool conv = false, fail = false;
-    float comp = -1.f;   // radius the compacted list is complete for (none yet)
-    float kf_fail = 0.f;  // N_enc(hsi) = Kn sum f at a failure
-    const float ftol = 2e-6f;
-    // The float separation from the fixed-point positions is within
-    // 4e-7 r + 4e-10 L of the exact one, so keeping the entries with float
-    // r < X (1 + 1e-4) leaves the list complete for every r < X (1 + 5e-5)
-    // when X > L / 65536 (compaction is skipped below that).
-    const float xmin = (float)(fmin(bx.L[0], fmin(bx.L[1], bx.L[2])) * (1.0 / 65536.0));
-    auto sep_r = [&](int j) {
-        const float *rj = rec + (int64_t)j * REC;
-        float4 pj = *reinterpret_cast<const float4 *>(rj);
-        float dx = qdiff(qxi, __float_as_uint(pj.x), bx.s[0]);
-        float dy = qdiff(qyi, __float_as_uint(pj.y), bx.s[1]);
-        float dz = qdiff(qzi, __float_as_uint(pj.z), bx.s[2]);
+// float separations of a particle from its list's entries: from the float
+// records (mixed path) or the fixed-point positions (FP64 path).  Within
+// 4e-7 r + 4e-10 L of the exact ones.
+template <typename R>
+struct Separation;
+template <>
+struct Separation<float> {
+    const float *rec;
+    uint32_t qx, qy, qz;
+    float sx, sy, sz;
+    __device__ __forceinline__ Separation(const DensArgs &a, const float *rec_, int64_t s, const Box &bx)
+        : rec(rec_), sx(bx.s[0]), sy(bx.s[1]), sz(bx.s[2]) {
+        const float *ri = rec + s * REC;
+        qx = __float_as_uint(ri[R_X]); qy = __float_as_uint(ri[R_Y]); qz = __float_as_uint(ri[R_Z]);
+    }
+    __device__ __forceinline__ float operator()(int j) const {
+        const float4 pj = *reinterpret_cast<const float4 *>(rec + (int64_t)j * REC);
+        float dx = qdiff(qx, __float_as_uint(pj.x), sx);
+        float dy = qdiff(qy, __float_as_uint(pj.y), sy);
+        float dz = qdiff(qz, __float_as_uint(pj.z), sz);
         float r2 = dx * dx + dy * dy + dz * dz;
         return r2 > 0.f ? r2 * rsqrtf(r2) : 0.f;
-    };
-    for (int it = 1; it <= a.max_iter; it++) {
+    }
+};
+template <>
+struct Separation<double> {
+    const uint32_t *px, *py, *pz;
+    uint32_t qx, qy, qz;
+    float sx, sy, sz;
+    __device__ __forceinline__ Separation(const DensArgs &a, const double *, int64_t s, const Box &bx)
+        : px(a.qx), py(a.qy), pz(a.qz), sx(bx.s[0]), sy(bx.s[1]), sz(bx.s[2]) {
+        qx = px[s]; qy = py[s]; qz = pz[s];
+    }
+    __device__ __forceinline__ float operator()(int j) const {
+        float dx = qdiff(qx, px[j], sx);
+        float dy = qdiff(qy, py[j], sy);
+        float dz = qdiff(qz, pz[j], sz);
+        float r2 = dx * dx + dy * dy + dz * dz;
+        return r2 > 0.f ? r2 * rsqrtf(r2) : 0.f;
+    }
+};
+
+struct NewtonF {
+    float h;       // root (or where the iteration stopped)
+    float comp;    // radius the compacted list is complete for (-1: not compacted)
+    int c;         // entries of the list
+    int it;        // evaluations
+    bool conv, fail;
+    float kf;      // N_enc(hsi) = Kn sum f at a failure
+};
+
+// A particle's list walked by one lane (W = 1) or by the 32 of a warp (a guard
+// round's few particles, whose lists at the doubled radius are long): entry k
+// goes to lane k mod W, sums are folded over the lanes.  A warp keeps the
+// separations of the first CACHE entries; a lane on its own gathers them again
+// in every pass (a running step's h takes one or two passes; keeping 16 to 64
+// of a thread's separations in shared memory took its L1 and was between 7 %
+// faster and 50 % slower).
+template <int W>
+struct Walk {
+    static constexpr int CACHE = W == 1 ? 0 : DENS_CACHE;
+    float *rs;     // the warp's cache
+    int lane;      // 0 for W = 1
+    template <typename T>
+    __device__ __forceinline__ T sum(T v) const {
+        if (W > 1)
+            for (int o = W / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        return v;
+    }
+    // entry (j, r) of this lane, kept or not, moves behind the w kept before it
+    __device__ __forceinline__ void keep(bool on, int32_t *idx, int j, float r, int &w) const {
+        if (W == 1) {
+            if (on) {
+                idx[w] = j;
+                w++;
+            }
+        } else {
+            const unsigned m = __ballot_sync(0xffffffffu, on);
+            if (on) {
+                const int t = w + __popc(m & ((1u << lane) - 1u));
+                idx[t] = j;
+                if (t < CACHE) rs[t] = r;
+            }
+            w += __popc(m);
+            __syncwarp();
+        }
+    }
+};
+
+// the safeguarded Newton iteration of one particle over its list idx
+template <int W, typename Sep>
+__device__ __forceinline__ NewtonF newton_float(const DensArgs &a, const Sep &sep, int32_t *idx, int c,
+                                                float h, float hsi, float N, float xmin,
+                                                int max_iter, const Walk<W> &wk) {
+    NewtonF o;
+    o.comp = -1.f;
+    o.conv = o.fail = false;
+    o.kf = 0.f;
+    o.it = 0;
+    const float Kn = kernel_Kn<float>(a.kernel);
+    const float ftol = 2e-6f;
+    float lo = 0.f, hi = -1.f;
+    const int c0 = min(c, Walk<W>::CACHE);
+#pragma unroll 4
+    for (int k = wk.lane; k < c0; k += W) wk.rs[k] = sep(idx[k]);
+    for (int it = 1; it <= max_iter; it++) {
+        o.it = it;
         float f = 0.f, mq = 0.f, ih = 1.f / h;
         // an upper bracket well inside the list radius: drop the entries
-        // beyond it (no later iterate exceeds hi)
+        // beyond it (no later iterate exceeds hi).  Keeping the entries with
+        // float r < X (1 + 1e-4) leaves the list complete for every
+        // r < X (1 + 5e-5) when X > L / 65536 (compaction is skipped below that)
         const bool shrink = a.compact && hi > xmin && hi < 0.8f * hsi;
-        const float keep = hi * 1.0001f;
-        int w = 0;
-        for (int k = 0; k < c; k++) {
-            const int j = idx[k];
-            const float r = sep_r(j);
-            if (shrink && r < keep) idx[w++] = j;
-            float fv, mv;
-            kernel_f<float>(a.kernel, r * ih, fv, mv);
-            f += fv;
-            mq += mv;
+        if (shrink) {
+            const float keep = hi * 1.0001f;
+            int w = 0;
+            for (int k0 = 0; k0 < c; k0 += W) {
+                const int k = k0 + wk.lane;
+                const bool in = W == 1 || k < c;
+                const int j = in ? idx[k] : 0;
+                const float r = !in ? INFINITY : k < Walk<W>::CACHE ? wk.rs[k] : sep(j);
+                wk.keep(r < keep, idx, j, r, w);
+                float fv, mv;
+                kernel_f<float>(a.kernel, r * ih, fv, mv);
+                f += fv;
+                mq += mv;
+            }
+            c = w;
+            o.comp = hi * 1.00005f;
+            hsi = o.comp;
+        } else {
+            const int cs = min(c, Walk<W>::CACHE);
+            for (int k = wk.lane; k < cs; k += W) {
+                float fv, mv;
+                kernel_f<float>(a.kernel, wk.rs[k] * ih, fv, mv);
+                f += fv;
+                mq += mv;
+            }
+            for (int k = cs + wk.lane; k < c; k += W) {
+                float fv, mv;
+                kernel_f<float>(a.kernel, sep(idx[k]) * ih, fv, mv);
+                f += fv;
+                mq += mv;
+            }
         }
-        if (shrink) { c = w; comp = hi * 1.00005f; hsi = comp; }
+        f = wk.sum(f);
+        mq = wk.sum(mq);
         float g = Kn * f - N;
         float dg = Kn * mq * ih;
-        if (g == 0.f) { conv = true; break; }
+        if (g == 0.f) { o.conv = true; break; }
         if (g < 0.f) {
-            if (h >= hsi) { fail = true; kf_fail = Kn * f; break; }
+            if (h >= hsi) { o.fail = true; o.kf = Kn * f; break; }
             lo = fmaxf(lo, h);
         } else {
             hi = (hi < 0.f || h < hi) ? h : hi;
         }
         float hn = dg > 0.f ? h - g / dg : -1.f;
-        if (hn > 0.f && fabsf(hn - h) <= ftol * h && hn <= hsi) { h = hn; conv = true; break; }
+        if (hn > 0.f && fabsf(hn - h) <= ftol * h && hn <= hsi) { h = hn; o.conv = true; break; }
         if (hi < 0.f) {
             if (!(hn > lo) || hn > 2.f * h) hn = 2.f * h;
             if (hn > hsi) hn = hsi;
@@ -302,14 +309,208 @@ __device__ __forceinline__ void dens_one(const DensArgs &a, const uint64_t *__re
         }
         h = hn;
     }
-    if (fail) {   // (no compaction happened: failing needs h >= hsi, below any bracket)
-        a.hs[s] = hsi_d * search_growth((double)N, (double)kf_fail, hsi_d, a.h[s]);
-        a.active[s] = (a.active[s] & ACT_GUARD) | 3;
-        atomicAdd(&a.cnt->search_fail, 1);
-        set_flag(a.cnt, ST_SEARCH);
+    o.h = h;
+    o.c = c;
+    return o;
+}
+
+// the root left the list radius: the radius grows, the particle is searched again
+__device__ __forceinline__ void dens_fail(const DensArgs &a, int64_t s) {
+    a.active[s] = (a.active[s] & ACT_GUARD) | 3;
+    atomicAdd(&a.cnt->search_fail, 1);
+    set_flag(a.cnt, ST_SEARCH);
+}
+
+// ---------------------------------------------------------------- FP64 path
+// Bound by the FP64 pipe: 23 FP64 instructions per neighbour in one pass,
+// where five passes of Newton's iteration and one for omega, with a square
+// root rounded correctly per neighbour, took about 220 (1.07 M tube 11.1 ->
+// 2.95 ms, 300k log-normal box 4.7 -> 0.88 ms).
+// h^2 d^2f/dh^2 of f(r/h) in float
+__device__ __forceinline__ float kernel_curv(int kernel, float q) {
+    const float t = 1.f - q, q2 = q * q;
+    if (kernel == 0) return -60.f * q2 * t * t * (1.f - 2.f * q);
+    return q <= 0.5f ? -36.f * q2 + 72.f * q2 * q : 12.f * q * t * (q - t);
+}
+
+template <int W>
+__device__ __forceinline__ void dens_one(const DensArgs &a, double *__restrict__ rec,
+                                         const Walk<W> &wk, int64_t s) {
+    if (s >= a.n) return;
+    if (a.only_active && !(a.active[s] & 1)) return;
+    const Box bx = a.boxes[a.pbox[s]];
+    const double hsi_d = a.hs[s], hguess = a.h[s];
+    const double N = a.nngb ? a.nngb[s] : a.n_ngb;
+    int32_t *idx = a.nbr_idx + a.nbr_off[s];
+    const double Lmin = fmin(bx.L[0], fmin(bx.L[1], bx.L[2]));
+    const float xmin = (float)(Lmin * (1.0 / 65536.0));
+    const double Lmax = fmax(bx.L[0], fmax(bx.L[1], bx.L[2]));
+    const Separation<double> sep(a, rec, s, bx);
+    const float hsf = (float)hsi_d;
+    float hf = (float)hguess;
+    if (!(hf > 0.f) || hf > hsf) hf = hsf;
+    // (a radius below 1e-4 of the box leaves the float separations less than
+    // 4e-6 accurate: everything in double then)
+    const NewtonF o = newton_float<W>(a, sep, idx, a.nbr_cnt[s], hf, hsf, (float)N, xmin,
+                                      hsi_d > 1e-4 * Lmax ? a.max_iter : 0, wk);
+    const float slack = (float)(1e-9 * Lmax);   // (bounds the error of a float r)
+    int c = o.c;
+    // The same iteration in double from the float root (from the list radius
+    // where the float iteration found none): a step below 2e-6 h, taken to
+    // third order, leaves an error below 1e-16 h.
+    const double hsi = o.comp > 0.f ? (double)o.comp : hsi_d;
+    const double Kn = kernel_Kn<double>(a.kernel), iKn = a.kernel == 0 ? 1.0 / 14.0 : 3.0 / 32.0;
+    const double M = N * iKn;   // sum f at the root
+    double h = o.fail ? hsi_d : o.it > 0 ? (double)o.h : hguess;
+    if (!(h > 0.0) || h > hsi) h = hsi;
+    const double xi = a.xs[s], yi = a.ys[s], zi = a.zs[s];
+    double lo = 0.0, hi = -1.0, F = 0.0;
+    bool conv = false, fail = false;
+    double crad = o.comp > 0.f ? (double)o.comp : 0.0;
+    const int left = a.max_iter - o.it;   // evaluations left
+    for (int it = 1; it <= (left > 1 ? left : 1); it++) {
+        const double ih = 1.0 / h;   // (rounded correctly: its error is common to every q)
+        double f = 0.0, mq = 0.0;
+        float s2 = 0.f;
+        const float hh = narrow(h);
+        const float cut = hh * (1.f + 1e-5f) + slack, keep = hh * 1.0001f;
+        // (the first pass of a converged float root compacts the list)
+        const bool shrink = a.compact && it == 1 && o.conv && hh > xmin;
+        int w = 0;
+        for (int k0 = 0; k0 < c; k0 += W) {
+            const int k = k0 + wk.lane;
+            const bool in = W == 1 || k < c;
+            const int j = in ? idx[k] : 0;
+            const float rf = !in ? INFINITY : k < Walk<W>::CACHE ? wk.rs[k] : sep(j);
+            if (shrink) wk.keep(rf < keep, idx, j, rf, w);
+            if (rf >= cut) continue;   // W = 0
+            const double dx = fold64(a.xs[j] - xi, bx.L[0]);
+            const double dy = fold64(a.ys[j] - yi, bx.L[1]);
+            const double dz = fold64(a.zs[j] - zi, bx.L[2]);
+            const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+            const double q = dpos(r2) ? r2 * rsqrt64(r2) * ih : 0.0;
+            if (!dlt_pos(q, 1.0)) continue;
+            const double t = 1.0 - q, t2 = t * t;
+            if (a.kernel == 0) {
+                const double t3 = t2 * t;
+                f = fma(t3 * t, fma(4.0, q, 1.0), f);
+                mq = fma(20.0 * (q * q), t3, mq);
+            } else if (!dlt_pos(0.5, q)) {
+                const double q2 = q * q;
+                f += fma(6.0 * q2, q - 1.0, 1.0);
+                mq = fma(q2, fma(-18.0, q, 12.0), mq);
+            } else {
+                f = fma(2.0 * t2, t, f);
+                mq = fma(6.0 * q, t2, mq);
+            }
+            s2 += kernel_curv(a.kernel, narrow(q));
+        }
+        f = wk.sum(f);
+        mq = wk.sum(mq);
+        s2 = wk.sum(s2);
+        if (shrink) { c = w; crad = (double)hh * (1.0 + 5e-5); }
+        const double g = f - M;   // (g / Kn)
+        F = f;
+        if (g == 0.0) { conv = true; break; }
+        if (g < 0.0) {
+            if (h >= hsi) {
+                fail = true;
+                F = Kn * f;
+                break;
+            }
+            lo = fmax(lo, h);
+        } else {
+            hi = (hi < 0.0 || h < hi) ? h : hi;
+        }
+        const double x = mq > 0.0 ? -g * (h / mq) : -2.0 * h;   // Newton step
+        // Halley: x - x^2 g'' / (2 g'), g'' / g' = s2 / (h mq)
+        const double y = x * ih, u = 0.5 * (double)s2 / mq;
+        const double d = x * (1.0 - y * u);
+        if (fabs(x) <= 2e-6 * h && h + d <= hsi && (it <= left || fabs(x) <= a.tol * h)) {
+            // sum f at h + d: f + f' d + f'' d^2 / 2
+            F = f + mq * (d * ih) * (1.0 + u * (d * ih));
+            h += d;
+            conv = true;
+            break;
+        }
+        double hn = mq > 0.0 ? h + x : -1.0;
+        if (hi < 0.0) {
+            if (!(hn > lo) || hn > 2.0 * h) hn = 2.0 * h;
+            if (hn > hsi) hn = hsi;
+        } else if (!(hn > lo && hn < hi)) {
+            hn = 0.5 * (lo + hi);
+        }
+        h = hn;
+    }
+    const bool lead = wk.lane == 0;
+    if (fail) {
+        if (lead) {
+            a.hs[s] = hsi * search_growth(N, F, hsi, hguess);
+            dens_fail(a, s);
+        }
         return;
     }
-    if (!conv) set_flag(a.cnt, ST_NOCONV_H);
+    if (!conv) {
+        if (lead) set_flag(a.cnt, ST_NOCONV_H);
+        // sum f at the last h
+        F = 0.0;
+        for (int k = wk.lane; k < c; k += W) {
+            const int j = idx[k];
+            const double dx = fold64(a.xs[j] - xi, bx.L[0]);
+            const double dy = fold64(a.ys[j] - yi, bx.L[1]);
+            const double dz = fold64(a.zs[j] - zi, bx.L[2]);
+            F += kernel_shape<double>(a.kernel, sqrt(dx * dx + dy * dy + dz * dz) / h);
+        }
+        F = wk.sum(F);
+    }
+    if (!lead) return;
+    if (crad > 0.0) {
+        a.nbr_cnt[s] = c;
+        a.hs[s] = crad;
+        if (!(h < crad)) {   // the root left the compacted radius: search again
+            dens_fail(a, s);
+            return;
+        }
+    }
+    const double om = 1.0 / (kernel_norm<double>(a.kernel, h) * F);
+    a.h[s] = h;
+    a.om[s] = om;
+    rec[s * REC + R_H] = h;
+    rec[s * REC + R_OM] = om;
+}
+
+// ---------------------------------------------------------------- mixed path
+// one particle's float Newton solve, then the double-float refinement
+template <int W>
+__device__ __forceinline__ void dens_one(const DensArgs &a, const uint64_t *__restrict__ q64x,
+                                         const uint64_t *__restrict__ q64y,
+                                         const uint64_t *__restrict__ q64z,
+                                         float *__restrict__ rec, const Walk<W> &wk, int64_t s) {
+    if (s >= a.n) return;
+    if (a.only_active && !(a.active[s] & 1)) return;
+    const Box bx = a.boxes[a.pbox[s]];
+    const Separation<float> sep(a, rec, s, bx);
+    const double hsi_d = a.hs[s];
+    float hsi = (float)hsi_d;
+    const float N = (float)(a.nngb ? a.nngb[s] : a.n_ngb);
+    const int64_t o = a.nbr_off[s];
+    int32_t *idx = a.nbr_idx + o;
+    float h = (float)a.h[s];
+    if (!(h > 0.f) || h > hsi) h = hsi;
+    const float xmin = (float)(fmin(bx.L[0], fmin(bx.L[1], bx.L[2])) * (1.0 / 65536.0));
+    const NewtonF nf = newton_float<W>(a, sep, idx, a.nbr_cnt[s], h, hsi, N, xmin, a.max_iter, wk);
+    const bool lead = wk.lane == 0;
+    if (nf.fail) {   // (no compaction happened: failing needs h >= hsi, below any bracket)
+        if (lead) {
+            a.hs[s] = hsi_d * search_growth((double)N, (double)nf.kf, hsi_d, a.h[s]);
+            dens_fail(a, s);
+        }
+        return;
+    }
+    if (!nf.conv && lead) set_flag(a.cnt, ST_NOCONV_H);
+    h = nf.h;
+    const float comp = nf.comp;
+    const int c = nf.c;
     // one Newton step in double-float on exact 64-bit fixed-point separations
     const uint64_t xi64 = q64x[s], yi64 = q64y[s], zi64 = q64z[s];
     const float sx = (float)(bx.L[0] * 5.421010862427522e-20);  // L / 2^64
@@ -322,10 +523,12 @@ __device__ __forceinline__ void dens_one(const DensArgs &a, const uint64_t *__re
     const bool fin = a.compact && h > xmin;
     const float keep = h * 1.0001f;
     int w = 0;
-    for (int k = 0; k < c; k++) {
-        const int j = idx[k];
-        const float rf = sep_r(j);
-        if (fin && rf < keep) idx[w++] = j;
+    for (int k0 = 0; k0 < c; k0 += W) {
+        const int k = k0 + wk.lane;
+        const bool in = W == 1 || k < c;
+        const int j = in ? idx[k] : 0;
+        const float rf = !in ? INFINITY : k < Walk<W>::CACHE ? wk.rs[k] : sep(j);
+        if (fin) wk.keep(rf < keep, idx, j, rf, w);
         if (rf >= hcut) continue;
         long long ix = (long long)(q64x[j] - xi64);
         long long iy = (long long)(q64y[j] - yi64);
@@ -359,6 +562,14 @@ __device__ __forceinline__ void dens_one(const DensArgs &a, const uint64_t *__re
             MQ = df_add(MQ, mv);
         }
     }
+    if (W > 1) {
+        for (int o = W / 2; o > 0; o >>= 1) {
+            F = df_add(F, {__shfl_xor_sync(0xffffffffu, F.hi, o), __shfl_xor_sync(0xffffffffu, F.lo, o)});
+            MQ = df_add(MQ, {__shfl_xor_sync(0xffffffffu, MQ.hi, o),
+                             __shfl_xor_sync(0xffffffffu, MQ.lo, o)});
+        }
+        if (!lead) return;
+    }
     // g = Kn F - N, dg = Kn MQ / h  ->  h_new = h - (F - N/Kn) h / MQ
     double Fd = (double)F.hi + (double)F.lo;
     double MQd = (double)MQ.hi + (double)MQ.lo;
@@ -375,9 +586,7 @@ __device__ __forceinline__ void dens_one(const DensArgs &a, const uint64_t *__re
         if (!(hnew < crad)) {
             // the refinement left the compacted radius (an unconverged float
             // root): search again from a rebuilt list
-            a.active[s] = (a.active[s] & ACT_GUARD) | 3;
-            atomicAdd(&a.cnt->search_fail, 1);
-            set_flag(a.cnt, ST_SEARCH);
+            dens_fail(a, s);
             return;
         }
     }
@@ -398,29 +607,41 @@ __device__ __forceinline__ void dens_one(const DensArgs &a, const uint64_t *__re
 // each warp's gathers over the box); the full solve ranks the CTA's 128
 // particles by list length.  (Larger ranked tiles spread the repeated
 // gathers of the Newton iterations over more of the Morton curve: slower.)
+__device__ __forceinline__ int64_t dens_particle(const DensArgs &a) {
+    if (!a.rank) return blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    __shared__ unsigned rank_key[RANK_THREADS];
+    const int64_t base = blockIdx.x * (int64_t)RANK_THREADS;
+    rank_tile(rank_key, 1, a.nbr_cnt, base, a.n);
+    return base + rank_index(rank_key[threadIdx.x], 1);
+}
+
+__global__ void k_density_f64(DensArgs a, double *__restrict__ rec) {
+    dens_one<1>(a, rec, Walk<1>{nullptr, 0}, dens_particle(a));
+}
+
 __global__ void k_density_mixed(DensArgs a, const uint64_t *__restrict__ q64x,
                                 const uint64_t *__restrict__ q64y,
                                 const uint64_t *__restrict__ q64z, float *__restrict__ rec) {
-    int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (a.rank) {
-        __shared__ unsigned rank_key[RANK_THREADS];
-        const int64_t base = blockIdx.x * (int64_t)RANK_THREADS;
-        rank_tile(rank_key, 1, a.nbr_cnt, base, a.n);
-        s = base + rank_index(rank_key[threadIdx.x], 1);
-    }
-    dens_one(a, q64x, q64y, q64z, rec, s);
+    dens_one<1>(a, q64x, q64y, q64z, rec, Walk<1>{nullptr, 0}, dens_particle(a));
 }
 
-// a guard round's re-solve: the warps take the particles of the round's
-// guard list 32 at a time (its own kernel: the branch would cost the full
-// solve's kernel ten registers)
-__global__ void k_density_mixed_list(DensArgs a, const uint64_t *__restrict__ q64x,
-                                     const uint64_t *__restrict__ q64y,
-                                     const uint64_t *__restrict__ q64z, float *__restrict__ rec) {
+// A guard round's re-solve: a warp per particle of the round's guard list.
+// The particles are few (0.4 % of a log-normal box in the first round, fewer
+// later) and their lists long, so a thread each leaves most of the GPU idle
+// behind one serial walk (gradient stage of a 4 M log-normal box, which holds
+// the rounds: 7.15 -> 5.58 ms; 300k in FP64 9.5 -> 6.3 ms).
+template <typename R>
+__global__ void __launch_bounds__(DENS_THREADS)
+k_density_list(DensArgs a, const uint64_t *__restrict__ q64x, const uint64_t *__restrict__ q64y,
+               const uint64_t *__restrict__ q64z, R *__restrict__ rec) {
+    __shared__ float rs[DENS_THREADS / 32][DENS_CACHE];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const Walk<32> wk{rs[warp], lane};
     const int nl = *a.nlist;
-    for (int b0 = warp_chunk(a.cursor); b0 < nl; b0 = warp_chunk(a.cursor)) {
-        const int t = b0 + (threadIdx.x & 31);
-        if (t < nl) dens_one(a, q64x, q64y, q64z, rec, a.list[t]);
+    for (int t = blockIdx.x * (DENS_THREADS / 32) + warp; t < nl; t += gridDim.x * (DENS_THREADS / 32)) {
+        __syncwarp();
+        if constexpr (sizeof(R) == 8) dens_one<32>(a, rec, wk, a.list[t]);
+        else dens_one<32>(a, q64x, q64y, q64z, rec, wk, a.list[t]);
     }
 }
 
@@ -476,6 +697,7 @@ cudaError_t run_density(hydro_ctx *c, bool only_active, bool compact, stream_t s
     a.nbr_idx = c->d_nbr_idx.get();
     a.hs = c->d_hs.get();
     a.xs = c->d_xs.get(); a.ys = c->d_ys.get(); a.zs = c->d_zs.get();
+    a.qx = c->d_qx.get(); a.qy = c->d_qy.get(); a.qz = c->d_qz.get();
     a.pbox = c->d_pbox.get();
     a.boxes = c->d_boxes.get();
     a.active = c->d_active.get();
@@ -491,9 +713,8 @@ cudaError_t run_density(hydro_ctx *c, bool only_active, bool compact, stream_t s
     a.cnt = c->d_cnt;
     // ranked when the gradient kernel ranks (the same divergence)
     a.rank = c->grad_rank && !only_active;
-    a.list = nullptr;
-    a.nlist = nullptr;
-    a.cursor = nullptr;
+    a.list = c->d_guard_idx.get();
+    a.nlist = &c->d_cnt->nguard;
     HYD_CUDA(cudaMemsetAsync(&c->d_cnt->search_fail, 0, sizeof(int), st));
     if (c->cfg.precision == HYDRO_MIXED) {
         // 64-bit fixed-point copies for the refinement step (xs.. are sorted)
@@ -508,22 +729,17 @@ cudaError_t run_density(hydro_ctx *c, bool only_active, bool compact, stream_t s
                                                          c->d_boxes.get(), q64, q64 + n, q64 + 2 * n);
             HYD_CUDA(launch_check());
         }
-        if (guard && only_active) {
-            // the round's guard particles, few and scattered, each with a
-            // long list at its grown radius: one thread each, the warps
-            // drawing them from the guard list
-            HYD_CUDA(cudaMemsetAsync(&c->d_cnt->solve_cursor, 0, sizeof(int), st));
-            a.list = c->d_guard_idx.get();
-            a.nlist = &c->d_cnt->nguard;
-            a.cursor = &c->d_cnt->solve_cursor;
-            k_density_mixed_list<<<152 * 8, DENS_THREADS, 0, st>>>(a, q64, q64 + n, q64 + 2 * n,
+        if (guard && only_active)
+            k_density_list<float><<<152 * 8, DENS_THREADS, 0, st>>>(a, q64, q64 + n, q64 + 2 * n,
                                                                    c->d_recf.get());
-        } else {
+        else
             k_density_mixed<<<grid_for(n, DENS_THREADS), DENS_THREADS, 0, st>>>(
                 a, q64, q64 + n, q64 + 2 * n, c->d_recf.get());
-        }
+    } else if (guard && only_active) {
+        k_density_list<double><<<152 * 8, DENS_THREADS, 0, st>>>(a, nullptr, nullptr, nullptr,
+                                                                c->d_recd.get());
     } else {
-        k_density_f64<<<grid_for(n, 128), 128, 0, st>>>(a, c->d_recd.get());
+        k_density_f64<<<grid_for(n, DENS_THREADS), DENS_THREADS, 0, st>>>(a, c->d_recd.get());
     }
     return launch_check();
 }

@@ -100,7 +100,6 @@ struct DevCounters {
     unsigned long long rung_active;   // particles starting a step in this sub-step
     int nredo;                        // particles a guard round recomputes the gradients of
     int redo_cursor;                  // the guard round's gradient warps' place in theirs
-    int solve_cursor;                 // the guard round's density warps' place in the guard list
     int redo_pass;                    // the last gradient pass took only the redo list (1) or
                                       // every particle (0): where flags can be set
     unsigned long long flux_cursor;   // the flux kernel's bucket queue

@@ -45,6 +45,7 @@ struct FluxArgs {
     double dt;
     const double *dt_dev;
     double *dQ;              // 5 n, sorted SoA
+    double *dQe;             // FP64 path: 5 n, the rounding errors of the sums in dQ
     DevCounters *cnt;
     const unsigned char *mlp_blob;   // packed network (hard-face kernel)
     int mlp_stall;                   // error-path test hook (hydro_test_mlp_stall)
@@ -575,6 +576,19 @@ __device__ __forceinline__ unsigned long long wsum(unsigned long long v) {
     return v;
 }
 
+// FP64 path: the rounding error of fl(old + c), exactly (the larger term first),
+// is summed beside the sum that an atomic addition to `old` rounded, so the
+// total does not depend on the order in which the faces' additions happen to
+// arrive (at about twice the rate of the faces' own additions before, the
+// additions of concurrent warps interleave differently from run to run)
+__device__ __forceinline__ void add_error(double *err, double old, double c) {
+    const double s = old + c;
+    const bool swap = dlt_pos(dabs_(old), dabs_(c));
+    const double big = swap ? c : old, small = swap ? old : c;
+    const double e = small - (s - big);
+    if (dbits(e) & 0x7fffffffffffffffll) atomicAdd(err, e);
+}
+
 constexpr int FLUX_WARPS = 4;
 constexpr int QCAP = 64;
 
@@ -681,6 +695,8 @@ k_fluxes(FluxArgs a, const R *__restrict__ rec) {
         // solve the first nb queued faces, one per lane, and hand -c back
         auto solve = [&](int nb) {
             R c[5] = {R(0), R(0), R(0), R(0), R(0)};
+            R old[sizeof(R) == 8 ? 5 : 1];   // FP64: the partner's sums before the addition
+            bool added = false;
             int ol = 32 + lane;   // idle lanes: a key no owner has
             // room left in the CTA's deferred-face sub-buffer (read once per
             // batch): with less than HARD_MARGIN slots -- more than the warps
@@ -743,8 +759,14 @@ k_fluxes(FluxArgs a, const R *__restrict__ rec) {
                         face_finish<R, RIEM, SCHEME>(a, K, st, R(-1), c, fs, ps);
                         if (!LEAN && RIEM == HYDRO_RIEMANN_EXACT && a.rec_faces)
                             record_face<R>(a, K, st, ps, f + ol, j);
+                        if constexpr (sizeof(R) == 8) {
 #pragma unroll
-                        for (int q = 0; q < 5; q++) atomicAdd(&a.dQ[q * a.n + j], widen(c[q]));
+                            for (int q = 0; q < 5; q++) old[q] = atomicAdd(&a.dQ[q * a.n + j], c[q]);
+                            added = true;
+                        } else {
+#pragma unroll
+                            for (int q = 0; q < 5; q++) atomicAdd(&a.dQ[q * a.n + j], widen(c[q]));
+                        }
                         if (!LEAN && a.dM && c[0] != R(0)) {
                             const double cm = widen(c[0]);
                             for (int q = 0; q < 3; q++) {
@@ -776,6 +798,13 @@ k_fluxes(FluxArgs a, const R *__restrict__ rec) {
                 mine &= mine - 1;
 #pragma unroll
                 for (int q = 0; q < 5; q++) acc.sub(q, sm.cb[t][q]);
+            }
+            if constexpr (sizeof(R) == 8) {   // (the additions' answers arrived meanwhile)
+                if (added) {
+                    const int64_t j = sm.qj[lane];
+#pragma unroll
+                    for (int q = 0; q < 5; q++) add_error(&a.dQe[q * a.n + j], old[q], c[q]);
+                }
             }
             __syncwarp();
             if constexpr (DEFER) {
@@ -838,7 +867,10 @@ k_fluxes(FluxArgs a, const R *__restrict__ rec) {
         }
         if (own) {
 #pragma unroll
-            for (int q = 0; q < 5; q++) atomicAdd(&a.dQ[q * a.n + s], acc.get(q));
+            for (int q = 0; q < 5; q++) {
+                const double v = acc.get(q), o = atomicAdd(&a.dQ[q * a.n + s], v);
+                if (sizeof(R) == 8) add_error(&a.dQe[q * a.n + s], o, v);
+            }
         }
         if (!a.queue) break;
         __syncwarp();

@@ -121,12 +121,15 @@ bool decide_learned(hydro_ctx *c) {
 
 cudaError_t run_fluxes(hydro_ctx *c, double dt, const double *dt_dev, stream_t st) {
     const int64_t n = c->plan.n;
+    const bool fp64 = c->cfg.precision == HYDRO_FP64;
     HYD_CUDA(c->d_dQ.ensure((size_t)5 * n));
+    if (fp64) HYD_CUDA(c->d_dQe.ensure((size_t)5 * n));
     if (c->grav_live) HYD_CUDA(c->d_dM.ensure((size_t)3 * n));
     // the entropy flux only matters where mass moves (MFV)
     const bool ent_flux = c->ent_live && c->cfg.scheme == HYDRO_MFV;
     auto clear = [&]() -> cudaError_t {
         HYD_CUDA(cudaMemsetAsync(c->d_dQ.get(), 0, sizeof(double) * 5 * n, st));
+        if (fp64) HYD_CUDA(cudaMemsetAsync(c->d_dQe.get(), 0, sizeof(double) * 5 * n, st));
         if (c->grav_live) HYD_CUDA(cudaMemsetAsync(c->d_dM.get(), 0, sizeof(double) * 3 * n, st));
         if (ent_flux) HYD_CUDA(cudaMemsetAsync(c->d_dS.get(), 0, sizeof(double) * n, st));
         // flux_pairs, newton_iters, guess_fallbacks, vacuum, first_order,
@@ -156,6 +159,7 @@ cudaError_t run_fluxes(hydro_ctx *c, double dt, const double *dt_dev, stream_t s
     a.dt = dt;
     a.dt_dev = dt_dev;
     a.dQ = c->d_dQ.get();
+    a.dQe = fp64 ? c->d_dQe.get() : nullptr;
     a.cnt = c->d_cnt;
     a.mlp_blob = c->d_mlp_blob.get();
     a.mlp_stall = c->mlp_stall;

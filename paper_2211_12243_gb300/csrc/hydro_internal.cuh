@@ -176,6 +176,7 @@ struct hydro_ctx {
     hyd::DevBuf<int32_t> d_pbox;
     hyd::DevBuf<double> d_Q;          // 6 n
     hyd::DevBuf<double> d_dQ;         // 5 n
+    hyd::DevBuf<double> d_dQe;        // 5 n (FP64): rounding errors of the sums in d_dQ
     hyd::DevBuf<float> d_recf;        // 32 n (MIXED)
     hyd::DevBuf<double> d_recd;       // 32 n (FP64)
     hyd::DevBuf<double> d_out;        // staging of outputs (up to 27 n)

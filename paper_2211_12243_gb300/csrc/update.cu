@@ -20,6 +20,7 @@ struct UpdArgs {
     const Box *boxes;
     double *Q;             // 6 n sorted (updated in place)
     const double *dQ;      // 5 n sorted
+    const double *dQe;     // their rounding errors (FP64; NULL: none kept)
     const double *xs, *ys, *zs, *h, *om;
     double dt;
     const double *dt_dev;
@@ -55,6 +56,10 @@ __global__ void k_update(UpdArgs a) {
     double E0 = a.Q[4 * n + s], U0 = a.Q[5 * n + s];
     double dm = a.dQ[s], dpx = a.dQ[n + s], dpy = a.dQ[2 * n + s], dpz = a.dQ[3 * n + s];
     double dE = a.dQ[4 * n + s];
+    if (a.dQe) {
+        dm += a.dQe[s]; dpx += a.dQe[n + s]; dpy += a.dQe[2 * n + s]; dpz += a.dQe[3 * n + s];
+        dE += a.dQe[4 * n + s];
+    }
     double vx0 = px0 / m0, vy0 = py0 / m0, vz0 = pz0 / m0;
     double dU = dE - (vx0 * dpx + vy0 * dpy + vz0 * dpz) + 0.5 * (vx0 * vx0 + vy0 * vy0 + vz0 * vz0) * dm;
     double m1 = m0 + dm, px1 = px0 + dpx, py1 = py0 + dpy, pz1 = pz0 + dpz;
@@ -161,13 +166,17 @@ __global__ void __launch_bounds__(1024) k_sums_final(const double *__restrict__ 
 
 __global__ void k_export_dQ(int64_t n, const int32_t *__restrict__ perm,
                             const double *__restrict__ Q, const double *__restrict__ dQ,
-                            double *__restrict__ out) {
+                            const double *__restrict__ dQe, double *__restrict__ out) {
     int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (s >= n) return;
     double m0 = Q[s];
     double vx = Q[n + s] / m0, vy = Q[2 * n + s] / m0, vz = Q[3 * n + s] / m0;
     double dm = dQ[s], dpx = dQ[n + s], dpy = dQ[2 * n + s], dpz = dQ[3 * n + s];
     double dE = dQ[4 * n + s];
+    if (dQe) {
+        dm += dQe[s]; dpx += dQe[n + s]; dpy += dQe[2 * n + s]; dpz += dQe[3 * n + s];
+        dE += dQe[4 * n + s];
+    }
     double dU = dE - (vx * dpx + vy * dpy + vz * dpz) + 0.5 * (vx * vx + vy * vy + vz * vz) * dm;
     int64_t o = perm[s];
     out[6 * o + 0] = dm;
@@ -198,6 +207,7 @@ cudaError_t run_update(hydro_ctx *c, hydro_particles *p, double dt, const double
     a.boxes = c->d_boxes.get();
     a.Q = c->d_Q.get();
     a.dQ = c->d_dQ.get();
+    a.dQe = c->cfg.precision == HYDRO_FP64 ? c->d_dQe.get() : nullptr;
     a.xs = c->d_xs.get(); a.ys = c->d_ys.get(); a.zs = c->d_zs.get();
     a.h = c->d_hsorted.get();
     a.om = c->d_omsorted.get();
@@ -243,6 +253,7 @@ cudaError_t run_check_inputs(hydro_ctx *c, const hydro_particles *p, stream_t st
 cudaError_t export_dQ(hydro_ctx *c, double *dQ, stream_t st) {
     const int64_t n = c->plan.n;
     k_export_dQ<<<grid_for(n, 256), 256, 0, st>>>(n, c->d_perm.get(), c->d_Q.get(), c->d_dQ.get(),
+                                                   c->cfg.precision == HYDRO_FP64 ? c->d_dQe.get() : nullptr,
                                                    dQ);
     return launch_check();
 }

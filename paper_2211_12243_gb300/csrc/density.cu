@@ -370,7 +370,7 @@ __device__ __forceinline__ void dens_one(const DensArgs &a, double *__restrict__
     const int left = a.max_iter - o.it;   // evaluations left
     for (int it = 1; it <= (left > 1 ? left : 1); it++) {
         const double ih = 1.0 / h;   // (rounded correctly: its error is common to every q)
-        double f = 0.0, mq = 0.0;
+        double f = 0.0, f1 = 0.0, mq = 0.0;
         float s2 = 0.f;
         const float hh = narrow(h);
         const float cut = hh * (1.f + 1e-5f) + slack, keep = hh * 1.0001f;
@@ -391,21 +391,24 @@ __device__ __forceinline__ void dens_one(const DensArgs &a, double *__restrict__
             const double q = dpos(r2) ? r2 * rsqrt64(r2) * ih : 0.0;
             if (!dlt_pos(q, 1.0)) continue;
             const double t = 1.0 - q, t2 = t * t;
+            double fn;
             if (a.kernel == 0) {
                 const double t3 = t2 * t;
-                f = fma(t3 * t, fma(4.0, q, 1.0), f);
+                fn = fma(t3 * t, fma(4.0, q, 1.0), f);
                 mq = fma(20.0 * (q * q), t3, mq);
             } else if (!dlt_pos(0.5, q)) {
                 const double q2 = q * q;
-                f += fma(6.0 * q2, q - 1.0, 1.0);
+                fn = f + fma(6.0 * q2, q - 1.0, 1.0);
                 mq = fma(q2, fma(-18.0, q, 12.0), mq);
             } else {
-                f = fma(2.0 * t2, t, f);
+                fn = fma(2.0 * t2, t, f);
                 mq = fma(6.0 * q, t2, mq);
             }
+            f = f1;   // (two sums by turns: their rounding is most of h's error)
+            f1 = fn;
             s2 += kernel_curv(a.kernel, narrow(q));
         }
-        f = wk.sum(f);
+        f = wk.sum(f + f1);
         mq = wk.sum(mq);
         s2 = wk.sum(s2);
         if (shrink) { c = w; crad = (double)hh * (1.0 + 5e-5); }

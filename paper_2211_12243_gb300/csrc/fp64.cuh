@@ -32,6 +32,9 @@ __device__ __forceinline__ long long dkey(double v) {
     const long long b = dbits(v);
     return b ^ (long long)((unsigned long long)(b >> 63) >> 1);
 }
+__device__ __forceinline__ double dunkey(long long k) {
+    return __longlong_as_double(k ^ (long long)((unsigned long long)(k >> 63) >> 1));
+}
 __device__ __forceinline__ bool dlt(double a, double b) { return dkey(a) < dkey(b); }
 // a < b for a, b >= 0 (false when a is NaN)
 __device__ __forceinline__ bool dlt_pos(double a, double b) {

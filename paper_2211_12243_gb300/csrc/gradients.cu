@@ -44,6 +44,8 @@ struct GradArgs {
     int *cursor;                         // ... taken by the warps 32 at a time
     int rank_rounds;                     // dense pass: rank tiles of 128 x this many particles
                                          // by list length (0: no ranking)
+    bool pad_c;                          // FP64 records hold the sound speed in their R_PAD slot
+                                         // (k_primitives; the entropy switch uses the slot)
 };
 
 template <typename R>
@@ -69,12 +71,217 @@ __device__ __forceinline__ void load10<double>(const double *p, double v[10]) {
     }
 }
 
+// grad_one in FP64, bound by the FP64 pipe: 72 FP64 instructions per
+// neighbour where the general form issued about 190 (gradient stage of the
+// 1.07 M tube 9.66 -> 5.34 ms, 32^3 lattice 0.38 -> 0.23 ms).  The
+// sound speeds are formed once per particle (k_primitives), 1/r and r come
+// from one refined reciprocal square root, extremes are kept as ordered
+// integers, and membership is decided from the fused r^2 (the definition's
+// rounding only matters within 1e-14 of h^2) and remembered for the second pass.
+template <bool LEAN>
+__device__ __forceinline__ void grad_one64(const GradArgs &a, double *__restrict__ rec, int64_t s) {
+    if (!(s < a.n && (!a.only_redo || (a.active[s] & ACT_REDO)) && (LEAN || !a.ract || a.ract[s]))) {
+        if (!LEAN && s < a.n && a.ract && !a.ract[s]) {
+            // not starting a step: no pairs, no CFL limit in this sub-step
+            a.dt_part[s] = INFINITY;
+            a.npair[s] = 0;
+        }
+        return;
+    }
+    const Box bx = a.boxes[a.pbox[s]];
+    double ri[10];
+    load10<double>(rec + s * REC, ri);
+    const double h = a.h[s], h2 = __dmul_rn(h, h);
+    const double h2lo = h2 * (1.0 - 1e-14), h2hi = h2 * (1.0 + 1e-14);
+    const double ih = 1.0 / h, norm = kernel_norm<double>(a.kernel, h);
+    const double fi[5] = {ri[R_RHO], ri[R_VX], ri[R_VY], ri[R_VZ], ri[R_P]};
+    auto sound = [&](const double *r, double rho, double p) {
+        return a.pad_c ? r[R_PAD] : sqrt(div_(a.gamma * p, rho));
+    };
+    const double ci = sound(rec + s * REC, ri[R_RHO], ri[R_P]);
+    auto separation = [&](const double *rj, double d[3]) {
+        d[0] = fold64(__dsub_rn(rj[0], ri[0]), bx.L[0]);
+        d[1] = fold64(__dsub_rn(rj[1], ri[1]), bx.L[1]);
+        d[2] = fold64(__dsub_rn(rj[2], ri[2]), bx.L[2]);
+    };
+    // r < h; r2: the fused r^2
+    auto member = [&](const double d[3], double r2) {
+        if (dlt_pos(r2, h2lo)) return true;
+        if (!dlt_pos(r2, h2hi)) return false;
+        return dlt_pos(r2_exact(d[0], d[1], d[2]), h2);
+    };
+    double E[6] = {0, 0, 0, 0, 0, 0}, S[5][3];
+    long long mx[5], mn[5];   // extremes of the fields (dkey)
+#pragma unroll
+    for (int f = 0; f < 5; f++) {
+        S[f][0] = S[f][1] = S[f][2] = 0.0;
+        mx[f] = mn[f] = dkey(fi[f]);
+    }
+    double vs = 0.0;
+    int mypairs = 0;
+    unsigned long long members = 0;   // of the first 64 entries
+    const int64_t o = a.nbr_off[s];
+    const int c = a.nbr_cnt[s];
+    // software pipeline: the index two entries ahead and the record of the
+    // next entry are in flight while an entry is summed
+    int jc = 0 < c ? a.nbr_idx[o] : 0;
+    int jn = 1 < c ? a.nbr_idx[o + 1] : 0;
+    double rn[10], cn = 0.0;
+    if (0 < c) {
+        load10<double>(rec + (int64_t)jc * REC, rn);
+        if (a.pad_c) cn = rec[(int64_t)jc * REC + R_PAD];
+    }
+    for (int k = 0; k < c; k++) {
+        const int j = jc;
+        double rj[10], cj = cn;
+#pragma unroll
+        for (int q = 0; q < 10; q++) rj[q] = rn[q];
+        if (k + 1 < c) {
+            load10<double>(rec + (int64_t)jn * REC, rn);
+            if (a.pad_c) cn = rec[(int64_t)jn * REC + R_PAD];
+        }
+        jc = jn;
+        jn = k + 2 < c ? a.nbr_idx[o + k + 2] : 0;
+        if (j == s) continue;
+        double d[3];
+        separation(rj, d);
+        const double r2 = fma(d[0], d[0], fma(d[1], d[1], d[2] * d[2]));
+        if (!member(d, r2)) continue;
+        mypairs++;
+        if (k < 64) members |= 1ull << k;
+        const double ir = dpos(r2) ? rsqrt64(r2) : 0.0, r = r2 * ir;   // (coincident particles: r = 0)
+        const double w = rj[R_OM] * (norm * kernel_shape<double>(a.kernel, r * ih));
+        const double wd[3] = {w * d[0], w * d[1], w * d[2]};
+        E[0] = fma(wd[0], d[0], E[0]);
+        E[1] = fma(wd[0], d[1], E[1]);
+        E[2] = fma(wd[0], d[2], E[2]);
+        E[3] = fma(wd[1], d[1], E[3]);
+        E[4] = fma(wd[1], d[2], E[4]);
+        E[5] = fma(wd[2], d[2], E[5]);
+        const double fj[5] = {rj[R_RHO], rj[R_VX], rj[R_VY], rj[R_VZ], rj[R_P]};
+        double df[5];
+#pragma unroll
+        for (int f = 0; f < 5; f++) {
+            df[f] = fj[f] - fi[f];
+            S[f][0] = fma(wd[0], df[f], S[f][0]);
+            S[f][1] = fma(wd[1], df[f], S[f][1]);
+            S[f][2] = fma(wd[2], df[f], S[f][2]);
+            const long long kf = dkey(fj[f]);
+            mx[f] = kf > mx[f] ? kf : mx[f];
+            mn[f] = kf < mn[f] ? kf : mn[f];
+        }
+        if (!a.pad_c) cj = sqrt(div_(a.gamma * rj[R_P], rj[R_RHO]));
+        const double wdot = fma(d[0], df[1], fma(d[1], df[2], d[2] * df[3])) * ir;
+        const double sig = ci + cj - (dneg(wdot) ? wdot : 0.0);
+        vs = sig > vs ? sig : vs;
+    }
+    // B = E^-1, N_cond (Eq. 19)
+    const double c00 = E[3] * E[5] - E[4] * E[4];
+    const double c01 = E[4] * E[2] - E[1] * E[5];
+    const double c02 = E[1] * E[4] - E[3] * E[2];
+    const double det = E[0] * c00 + E[1] * c01 + E[2] * c02;
+    double B[6], ncond;
+    if (det != 0.0 && isfinite(det)) {
+        const double id = 1.0 / det;
+        B[0] = c00 * id;
+        B[1] = c01 * id;
+        B[2] = c02 * id;
+        B[3] = (E[0] * E[5] - E[2] * E[2]) * id;
+        B[4] = (E[2] * E[1] - E[0] * E[4]) * id;
+        B[5] = (E[0] * E[3] - E[1] * E[1]) * id;
+        const double nE = E[0] * E[0] + E[3] * E[3] + E[5] * E[5] +
+                          2.0 * (E[1] * E[1] + E[2] * E[2] + E[4] * E[4]);
+        const double nB = B[0] * B[0] + B[3] * B[3] + B[5] * B[5] +
+                          2.0 * (B[1] * B[1] + B[2] * B[2] + B[4] * B[4]);
+        ncond = sqrt(nB * nE) / 3.0;
+    } else {
+        for (int k = 0; k < 6; k++) B[k] = 0.0;
+        ncond = INFINITY;
+    }
+    double G[5][3];
+#pragma unroll
+    for (int f = 0; f < 5; f++) {
+        G[f][0] = B[0] * S[f][0] + B[1] * S[f][1] + B[2] * S[f][2];
+        G[f][1] = B[1] * S[f][0] + B[3] * S[f][1] + B[4] * S[f][2];
+        G[f][2] = B[2] * S[f][0] + B[4] * S[f][1] + B[5] * S[f][2];
+    }
+    double alpha[5] = {1, 1, 1, 1, 1};
+    if (a.limiter) {
+        // largest extrapolations to the midpoints, doubled (dx . grad f)
+        long long dp[5] = {0, 0, 0, 0, 0}, dm[5] = {0, 0, 0, 0, 0};
+        auto pos3 = [&](int j, double v[3]) {
+            const double *pj = rec + (int64_t)j * REC;
+            const double2 t = *reinterpret_cast<const double2 *>(pj);
+            v[0] = t.x; v[1] = t.y; v[2] = pj[2];
+        };
+        int jc2 = 0 < c ? a.nbr_idx[o] : 0;
+        int jn2 = 1 < c ? a.nbr_idx[o + 1] : 0;
+        double pn[3];
+        if (0 < c) pos3(jc2, pn);
+        for (int k = 0; k < c; k++) {
+            const int j = jc2;
+            const double pj[3] = {pn[0], pn[1], pn[2]};
+            if (k + 1 < c) pos3(jn2, pn);
+            jc2 = jn2;
+            jn2 = k + 2 < c ? a.nbr_idx[o + k + 2] : 0;
+            if (k < 64 ? !((members >> k) & 1ull) : j == s) continue;
+            double d[3];
+            separation(pj, d);
+            if (k >= 64 && !member(d, fma(d[0], d[0], fma(d[1], d[1], d[2] * d[2])))) continue;
+#pragma unroll
+            for (int f = 0; f < 5; f++) {
+                const long long e = dkey(fma(d[0], G[f][0], fma(d[1], G[f][1], d[2] * G[f][2])));
+                dp[f] = e > dp[f] ? e : dp[f];
+                dm[f] = e < dm[f] ? e : dm[f];
+            }
+        }
+        const double ratio = a.ncond_crit / ncond;
+        double beta = a.beta_max * (ratio * ratio < 1.0 ? ratio * ratio : 1.0);
+        beta = beta > a.beta_min ? beta : a.beta_min;
+#pragma unroll
+        for (int f = 0; f < 5; f++) {
+            const double up = dunkey(dp[f]), dn = dunkey(dm[f]);
+            const double rp = dpos(up) ? 2.0 * (dunkey(mx[f]) - fi[f]) * rcp64(up) : INFINITY;
+            const double rm = dneg(dn) ? 2.0 * (dunkey(mn[f]) - fi[f]) * rcp64(dn) : INFINITY;
+            const double al = beta * (rp < rm ? rp : rm);
+            alpha[f] = al < 1.0 ? al : 1.0;
+        }
+    }
+    double *rs = rec + s * REC;
+#pragma unroll
+    for (int k = 0; k < 6; k++) rs[R_B + k] = B[k];
+#pragma unroll
+    for (int f = 0; f < 5; f++)
+#pragma unroll
+        for (int q = 0; q < 3; q++) rs[R_G + 3 * f + q] = alpha[f] * G[f][q];
+    if (!LEAN && a.outB)
+        for (int k = 0; k < 6; k++) a.outB[k * a.n + s] = B[k];
+    if (!LEAN && a.outG)
+        for (int f = 0; f < 5; f++)
+            for (int q = 0; q < 3; q++) a.outG[(3 * f + q) * a.n + s] = G[f][q];
+    if (!LEAN && a.outA)
+        for (int f = 0; f < 5; f++) a.outA[f * a.n + s] = alpha[f];
+    if (!LEAN && a.outN) a.outN[s] = ncond;
+    // CFL timestep of Eq. 31 with the signal velocity of Eq. 32
+    a.dt_part[s] = vs > 0.0 ? a.c_cfl * h / vs : INFINITY;
+    a.npair[s] = mypairs;
+    // N_cond guard (§2.3.5)
+    if (!(ncond <= a.ncond_crit)) {
+        a.active[s] |= ACT_NCOND;
+        atomicAdd(&a.cnt->ncond_fail, 1);
+    }
+}
+
 // MINB: resident CTAs per SM the register allocation must allow (1: no
 // bound; 5, 6: the variants hydro_autotune times)
 // LEAN: compiled without the staged outputs (outB, outG, outA, outN) and
 // the individual-timestep mask, which hydro_step does not use
 template <typename R, bool LEAN>
 __device__ __forceinline__ void grad_one(const GradArgs &a, R *__restrict__ rec, int64_t s) {
+    if constexpr (sizeof(R) == 8) {
+        grad_one64<LEAN>(a, rec, s);
+        return;
+    }
     int mypairs = 0;
     if (s < a.n && (!a.only_redo || (a.active[s] & ACT_REDO)) && (LEAN || !a.ract || a.ract[s])) {
         const Box bx = a.boxes[a.pbox[s]];
@@ -347,7 +554,8 @@ struct EntArgs {
     const double *A0;      // entropic function at the start of the step (sorted)
     double *A1;            // the value the step uses (sorted out)
     uint8_t *cand;         // 1: the energies did not give the pressure (sorted)
-    double gamma, alpha2, alpha3;
+    double gamma;          // (set with the switch off too)
+    double alpha2, alpha3;
 };
 
 // primitives from the sorted conserved state and omega (§2.3.2, Eq. 23),
@@ -399,6 +607,9 @@ __global__ void k_primitives(int64_t n, const double *__restrict__ Q,
             r[R_VZ] = (R)(pz / m);
             r[R_P] = (R)pd;
             r[R_OM] = (R)w;
+            // the sound speed, for the neighbours' signal velocities (the
+            // entropy switch takes the slot for A)
+            if (!ent.A1) r[R_PAD] = (R)sqrt(div_(ent.gamma * pd, rho));
         } else {
             // float record: only E - E_kin needs double (cancellation); 1/m
             // from a float reciprocal and one Newton step in double (relative
@@ -566,6 +777,7 @@ cudaError_t run_primitives(hydro_ctx *c, stream_t st, bool only_guard) {
     const bool mixed = c->cfg.precision == HYDRO_MIXED;
     const uint8_t *ract = c->rung_live ? c->d_ract.get() : nullptr;
     EntArgs ent = {};
+    ent.gamma = c->cfg.gamma;
     if (c->ent_live) {
         ent.A0 = c->d_A0.get();
         ent.A1 = c->d_A1.get();
@@ -668,6 +880,7 @@ cudaError_t run_gradients(hydro_ctx *c, double *B_out, double *grad_out, double 
     a.list = nullptr;
     a.nlist = nullptr;
     a.cursor = nullptr;
+    a.pad_c = c->cfg.precision == HYDRO_FP64 && !c->ent_live;
     a.rank_rounds = c->grad_rank == 2 ? rank_rounds(n) : c->grad_rank;
     unsigned grid = a.rank_rounds ? grid_for(n, RANK_THREADS * a.rank_rounds) : grid_for(n, 128);
     size_t smem = a.rank_rounds ? sizeof(unsigned) * RANK_THREADS * a.rank_rounds : 0;

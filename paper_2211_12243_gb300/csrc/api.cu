@@ -916,7 +916,7 @@ int hydro_mlp_gradient(hydro_ctx *c, const float *x, const float *t, int64_t n, 
     cudaStream_t st = (cudaStream_t)stream;
     API_CUDA(cudaMemsetAsync(grad, 0, kMlpParams * sizeof(float), st));
     API_CUDA(cudaMemsetAsync(loss, 0, sizeof(float), st));
-    API_CUDA(mlp_gradient(c, x, t, n, n, 0, 0, 0, quant ? 1 : 0, grad, loss, st));
+    API_CUDA(mlp_gradient(c, x, t, n, quant ? 1 : 0, grad, loss, st));
     return HYDRO_OK;
 }
 
@@ -958,7 +958,6 @@ int hydro_mlp_train(hydro_ctx *c, const float *faces, int64_t n, int64_t steps, 
     cudaStream_t st = (cudaStream_t)stream;
     API_CUDA(c->d_mlp_x.ensure((size_t)12 * n));
     API_CUDA(c->d_mlp_t.ensure((size_t)n));
-    API_CUDA(c->d_mlp_grad.ensure(kMlpParams));
     API_CUDA(c->d_mlp_m.ensure(kMlpParams));
     API_CUDA(c->d_mlp_v.ensure(kMlpParams));
     API_CUDA(c->d_mlp_loss.ensure((size_t)std::max<int64_t>(steps, 1)));
@@ -974,19 +973,16 @@ int hydro_mlp_train(hydro_ctx *c, const float *faces, int64_t n, int64_t steps, 
                                c->d_mlp_box.get(), st));
         API_CUDA(cudaStreamSynchronize(st));   // w is a host temporary
     }
-    API_CUDA(cudaMemsetAsync(c->d_mlp_grad.get(), 0, kMlpParams * sizeof(float), st));
     API_CUDA(cudaMemsetAsync(c->d_mlp_m.get(), 0, kMlpParams * sizeof(float), st));
     API_CUDA(cudaMemsetAsync(c->d_mlp_v.get(), 0, kMlpParams * sizeof(float), st));
     API_CUDA(cudaMemsetAsync(c->d_mlp_loss.get(), 0, std::max<int64_t>(steps, 1) * sizeof(float), st));
     for (int64_t s = 1; s <= steps; s++) {
-        API_CUDA(mlp_gradient(c, c->d_mlp_x.get(), c->d_mlp_t.get(), n, batch, 1, seed,
-                              (uint64_t)s, 1, c->d_mlp_grad.get(), c->d_mlp_loss.get() + (s - 1),
-                              st));
         // cosine decay of the learning rate to lr / 20 over the run
         const double frac = steps > 1 ? (double)(s - 1) / (double)(steps - 1) : 0.0;
         const double lr_s = lr * (0.05 + 0.95 * 0.5 * (1.0 + std::cos(3.141592653589793 * frac)));
-        API_CUDA(mlp_adam(c, c->d_mlp_grad.get(), c->d_mlp_m.get(), c->d_mlp_v.get(), (float)lr_s,
-                          (int)std::min<int64_t>(s, 1 << 30), st));
+        API_CUDA(mlp_train_step(c, c->d_mlp_x.get(), c->d_mlp_t.get(), n, batch, seed, (uint64_t)s,
+                                c->d_mlp_m.get(), c->d_mlp_v.get(), c->d_mlp_loss.get() + (s - 1),
+                                (float)lr_s, (int)std::min<int64_t>(s, 1 << 30), st));
     }
     if (loss && steps > 0)
         API_CUDA(cudaMemcpyAsync(loss, c->d_mlp_loss.get(), steps * sizeof(float),

@@ -437,11 +437,13 @@ cudaError_t mlp_pack(hydro_ctx *c, stream_t st);
 cudaError_t mlp_predict(hydro_ctx *c, const float *faces, int64_t n, float *out, stream_t st);
 cudaError_t mlp_features(hydro_ctx *c, const float *faces, int64_t n, float *x, float *t,
                          stream_t st);
-cudaError_t mlp_gradient(hydro_ctx *c, const float *x, const float *t, int64_t n, int64_t nb,
-                         int random, uint64_t seed, uint64_t step, int quant, float *grad,
-                         float *loss, stream_t st);
-cudaError_t mlp_adam(hydro_ctx *c, float *grad, float *m, float *v, float lr, int step,
-                     stream_t st);
+// gradient and loss over all n samples
+cudaError_t mlp_gradient(hydro_ctx *c, const float *x, const float *t, int64_t n, int quant,
+                         float *grad, float *loss, stream_t st);
+// one minibatch of nb random samples: gradient, then the Adam update
+cudaError_t mlp_train_step(hydro_ctx *c, const float *x, const float *t, int64_t n, int64_t nb,
+                           uint64_t seed, uint64_t step, float *m, float *v, float *loss, float lr,
+                           int adam_step, stream_t st);
 cudaError_t mlp_normalise(hydro_ctx *c, const float *x, const float *t, int64_t n, double *acc,
                           int *box, stream_t st);
 

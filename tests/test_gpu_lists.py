@@ -75,3 +75,21 @@ def test_lists_match_oracle(orc, hyd, name):
     assert np.array_equal(off.cpu().numpy(), off_o)
     assert np.array_equal(idx.cpu().numpy(), idx_o)
     H.close()
+
+
+def test_export_of_rows_longer_than_shared_memory(orc, hyd):
+    import torch
+    n = 1500
+    x, y, z = _uniform(n, (1, 1, 1), 20)
+    hs = np.full(n, 0.49)
+    hs[::3] = 0.9   # (beyond half the box: nearly every particle; rows of over 1024 entries)
+    H = hyd.Hydro(hyd.default_config())
+    H.set_boxes(np.array([0, n], dtype=np.int64), np.ones(3))
+    dev = lambda v: torch.as_tensor(np.ascontiguousarray(v, dtype=np.float64), device="cuda")
+    st = {"x": dev(x), "y": dev(y), "z": dev(z), "h": dev(hs)}
+    off, idx = H.build_neighbours(st, dev(hs))
+    off_o, idx_o = orc.neighbours(x, y, z, np.ones(3), hs, use_grid=False)
+    assert np.diff(off_o).max() > 1024
+    assert np.array_equal(off.cpu().numpy(), off_o)
+    assert np.array_equal(idx.cpu().numpy(), idx_o)
+    H.close()

@@ -322,6 +322,9 @@ __device__ __forceinline__ void dens_fail(const DensArgs &a, int64_t s) {
 }
 
 // ---------------------------------------------------------------- FP64 path
+// float evaluations before the iteration starts again in double
+constexpr int FLOAT_ITER = 12;
+
 // Bound by the FP64 pipe: 23 FP64 instructions per neighbour in one pass,
 // where five passes of Newton's iteration and one for omega, with a square
 // root rounded correctly per neighbour, took about 220 (1.07 M tube 11.1 ->
@@ -352,22 +355,23 @@ __device__ __forceinline__ void dens_one(const DensArgs &a, double *__restrict__
     // (a radius below 1e-4 of the box leaves the float separations less than
     // 4e-6 accurate: everything in double then)
     const NewtonF o = newton_float<W>(a, sep, idx, a.nbr_cnt[s], hf, hsf, (float)N, xmin,
-                                      hsi_d > 1e-4 * Lmax ? a.max_iter : 0, wk);
+                                      hsi_d > 1e-4 * Lmax ? min(a.max_iter, FLOAT_ITER) : 0, wk);
     const float slack = (float)(1e-9 * Lmax);   // (bounds the error of a float r)
     int c = o.c;
     // The same iteration in double from the float root (from the list radius
-    // where the float iteration found none): a step below 2e-6 h, taken to
+    // where it lies beyond, from the guess where the float iteration did not
+    // settle): a step below 2e-6 h, taken to
     // third order, leaves an error below 1e-16 h.
     const double hsi = o.comp > 0.f ? (double)o.comp : hsi_d;
     const double Kn = kernel_Kn<double>(a.kernel), iKn = a.kernel == 0 ? 1.0 / 14.0 : 3.0 / 32.0;
     const double M = N * iKn;   // sum f at the root
-    double h = o.fail ? hsi_d : o.it > 0 ? (double)o.h : hguess;
+    double h = o.fail ? hsi_d : o.conv ? (double)o.h : hguess;
     if (!(h > 0.0) || h > hsi) h = hsi;
     const double xi = a.xs[s], yi = a.ys[s], zi = a.zs[s];
     double lo = 0.0, hi = -1.0, F = 0.0;
     bool conv = false, fail = false;
     double crad = o.comp > 0.f ? (double)o.comp : 0.0;
-    const int left = a.max_iter - o.it;   // evaluations left
+    const int left = a.max_iter - (o.conv || o.fail ? o.it : 0);   // evaluations left
     for (int it = 1; it <= (left > 1 ? left : 1); it++) {
         const double ih = 1.0 / h;   // (rounded correctly: its error is common to every q)
         double f = 0.0, f1 = 0.0, mq = 0.0;

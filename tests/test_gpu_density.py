@@ -71,3 +71,25 @@ def test_guard_resolves_long_lists(orc, hyd, precision, n, n_ngb):
         # a float E may put a particle on the other side of the threshold
         assert np.mean(err > 1e-12) < 2e-3
     H.close()
+
+
+@pytest.mark.parametrize("n", [4099, 20011])
+def test_density_where_the_float_iteration_does_not_settle(orc, hyd, n):
+    """near-coincident pairs: the float sums jump by two at a time and the
+    iteration may wander at its tolerance; FP64 converges from the guess"""
+    import torch
+    rng = np.random.default_rng(n)
+    c = rng.random((3, n))
+    c[:, n - n // 2:] = c[:, :n // 2] + 1e-8
+    c = np.minimum(c, 1 - 1e-12)
+    h0 = np.full(n, np.cbrt(24.0 / np.pi / n))
+    h, om, _, st = orc.density(orc.config(), *c, np.ones(3), h0)
+    assert st == 0
+    H = hyd.Hydro(hyd.default_config())
+    H.set_boxes(np.array([0, n], dtype=np.int64), np.ones(3))
+    dev = lambda v: torch.as_tensor(np.ascontiguousarray(v), device="cuda")
+    s = {"x": dev(c[0]), "y": dev(c[1]), "z": dev(c[2]), "h": dev(h0), "omega": dev(np.zeros(n))}
+    H.build_neighbours(s, dev(h * 1.2), export=False)
+    H.density(s)
+    assert np.max(np.abs(s["h"].cpu().numpy() / h - 1)) < 1e-12
+    H.close()

@@ -9,8 +9,11 @@ namespace hyd {
 namespace {
 
 constexpr int SORT_THREADS = 256;
+// keys per CTA of a radix pass: 256 times this many rounds.  A CTA's rounds
+// are a serial chain, so the tiles shrink until there are a few CTAs per SM
+// (rounds 16, 4 and 1; the histograms and scatters of 32,768 keys 91 -> 22 us,
+// of 300,007 keys 92 -> 45 us)
 constexpr int SORT_ROUNDS = 16;
-constexpr int SORT_TILE = SORT_THREADS * SORT_ROUNDS;   // keys per CTA
 constexpr int SCAN_THREADS = 1024;
 constexpr int SCAN_ITEMS = 2;
 constexpr int SCAN_TILE = SCAN_THREADS * SCAN_ITEMS;
@@ -43,7 +46,8 @@ __device__ __forceinline__ int box_of(const int64_t *box_off, int64_t nbox, int6
 __global__ void k_morton(int64_t n, const double *__restrict__ x, const double *__restrict__ y,
                          const double *__restrict__ z, const int64_t *__restrict__ box_off,
                          int64_t nbox, const Box *__restrict__ boxes,
-                         unsigned long long *__restrict__ keys, int32_t *__restrict__ vals) {
+                         unsigned long long *__restrict__ keys, int32_t *__restrict__ vals,
+                         bool zero) {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     int b = nbox > 1 ? box_of(box_off, nbox, i) : 0;
@@ -56,25 +60,128 @@ __global__ void k_morton(int64_t n, const double *__restrict__ x, const double *
     uint32_t qz = min((uint32_t)(z[i] / Lmax * 1024.0), 1023u);
     uint32_t m = (spread10(qx) << 2) | (spread10(qy) << 1) | spread10(qz);
     keys[i] = ((unsigned long long)b << 30) | m;
-    vals[i] = (int32_t)i;
+    vals[i] = zero ? 0 : (int32_t)i;
 }
 
+// Up to RANK_SORT_MAX keys of at most 32 bits are sorted by counting instead:
+// the place of a key is the number of keys before it in (key, index) order, an
+// n^2 comparison that the whole GPU shares, in two launches where the four
+// radix passes take twelve small ones: 8,192 keys 13 us, 16,384 keys 36 us (45 us
+// by the passes), 32,768 keys 121 us (against 45 us; before the tiles shrank
+// with n, the passes took 98 us from 8,192 to 300,000 keys).
+constexpr int64_t RANK_SORT_MAX = 16384;
+constexpr int RANK_I = 256, RANK_J = 256;   // keys ranked by a CTA, keys they are compared with
+
+__global__ void __launch_bounds__(RANK_I) k_rank_count(int64_t n,
+                                                       const unsigned long long *__restrict__ keys,
+                                                       int32_t *__restrict__ rank) {
+    __shared__ __align__(16) uint32_t kj[RANK_J];
+    const int64_t i0 = blockIdx.x * (int64_t)RANK_I, j0 = blockIdx.y * (int64_t)RANK_J;
+    const int nj = (int)min((int64_t)RANK_J, n - j0);
+    if (threadIdx.x < nj) kj[threadIdx.x] = (uint32_t)keys[j0 + threadIdx.x];
+    __syncthreads();
+    const int64_t i = i0 + threadIdx.x;
+    if (i >= n) return;
+    const uint32_t k = (uint32_t)keys[i];
+    int c = 0;
+    if (j0 + RANK_J <= i0) {          // every j before every i: equal keys count
+        const uint4 *k4 = reinterpret_cast<const uint4 *>(kj);
+#pragma unroll 8
+        for (int t = 0; t < RANK_J / 4; t++) {
+            const uint4 v = k4[t];
+            c += (v.x <= k) + (v.y <= k) + (v.z <= k) + (v.w <= k);
+        }
+    } else if (j0 > i0 && nj == RANK_J) {   // after
+        const uint4 *k4 = reinterpret_cast<const uint4 *>(kj);
+#pragma unroll 8
+        for (int t = 0; t < RANK_J / 4; t++) {
+            const uint4 v = k4[t];
+            c += (v.x < k) + (v.y < k) + (v.z < k) + (v.w < k);
+        }
+    } else {
+        for (int t = 0; t < nj; t++) c += kj[t] < k || (kj[t] == k && j0 + t < i);
+    }
+    if (c) atomicAdd(&rank[i], c);
+}
+static_assert(RANK_I == RANK_J, "a block of j lies before, at or after a block of i");
+
+__global__ void k_rank_scatter(int64_t n, const int32_t *__restrict__ rank,
+                               int32_t *__restrict__ perm) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i < n) perm[rank[i]] = (int32_t)i;
+}
+
+// copies of the digits' totals that the tiles add to by turns (adds to one
+// address wait for one another)
+constexpr int TOTAL_COPIES = 8;
+constexpr int OFFS_THREADS = 1024;
+
 // per-tile digit histogram, digit-major: hist[d * ntiles + tile]
+template <int ROUNDS>
 __global__ void k_radix_hist(int64_t n, const unsigned long long *__restrict__ keys, int shift,
-                             int64_t ntiles, int64_t *__restrict__ hist) {
+                             int64_t ntiles, int64_t *__restrict__ hist,
+                             unsigned long long *__restrict__ total) {
     __shared__ int h[256];
     for (int t = threadIdx.x; t < 256; t += blockDim.x) h[t] = 0;
     __syncthreads();
-    int64_t base = blockIdx.x * (int64_t)SORT_TILE;
-    for (int r = 0; r < SORT_ROUNDS; r++) {
+    int64_t base = blockIdx.x * (int64_t)(SORT_THREADS * ROUNDS);
+    for (int r = 0; r < ROUNDS; r++) {
         int64_t i = base + r * SORT_THREADS + threadIdx.x;
         if (i < n) atomicAdd(&h[(keys[i] >> shift) & 255u], 1);
     }
     __syncthreads();
-    for (int t = threadIdx.x; t < 256; t += blockDim.x) hist[(int64_t)t * ntiles + blockIdx.x] = h[t];
+    for (int t = threadIdx.x; t < 256; t += blockDim.x) {
+        hist[(int64_t)t * ntiles + blockIdx.x] = h[t];
+        if (h[t]) atomicAdd(&total[(blockIdx.x % TOTAL_COPIES) * 256 + t], (unsigned long long)h[t]);
+    }
+}
+
+__device__ __forceinline__ int64_t warp_incl_scan(int64_t v) {
+    int lane = threadIdx.x & 31;
+    for (int o = 1; o < 32; o <<= 1) {
+        int64_t t = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += t;
+    }
+    return v;
+}
+
+// Where the keys of digit blockIdx.x go, tile by tile: the keys of the lower
+// digits (their totals), then the digit's counts in the tiles before, scanned
+// by the CTA 1024 tiles at a time.  One launch per pass in place of the three
+// of a general scan over all digits and tiles (32,768 keys: 31 -> 10 us for the
+// four passes).
+__global__ void __launch_bounds__(OFFS_THREADS)
+k_radix_offsets(int64_t ntiles, const int64_t *__restrict__ hist,
+                const unsigned long long *__restrict__ total, int64_t *__restrict__ offs) {
+    __shared__ int64_t wsum[32];
+    const int d = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // inclusive scan over the CTA; all: its sum
+    auto scan = [&](int64_t v, int64_t &all) {
+        const int64_t x = warp_incl_scan(v);
+        __syncthreads();
+        if (lane == 31) wsum[warp] = x;
+        __syncthreads();
+        const int64_t w = warp_incl_scan(wsum[lane]);
+        all = __shfl_sync(0xffffffffu, w, 31);
+        const int64_t before = __shfl_sync(0xffffffffu, w, max(warp - 1, 0));
+        return x + (warp > 0 ? before : 0);
+    };
+    int64_t base = 0, v = 0;
+    for (int t = threadIdx.x; t < TOTAL_COPIES * 256; t += OFFS_THREADS)
+        if ((t & 255) < d) v += (int64_t)total[t];
+    scan(v, base);
+    for (int64_t t0 = 0; t0 < ntiles; t0 += OFFS_THREADS) {
+        const int64_t t = t0 + threadIdx.x;
+        v = t < ntiles ? hist[d * ntiles + t] : 0;
+        int64_t sum;
+        const int64_t x = scan(v, sum);
+        if (t < ntiles) offs[d * ntiles + t] = base + x - v;
+        base += sum;
+    }
 }
 
 // stable scatter: within a tile, elements keep their order per digit
+template <int ROUNDS>
 __global__ void k_radix_scatter(int64_t n, const unsigned long long *__restrict__ keys,
                                 const int32_t *__restrict__ vals, int shift, int64_t ntiles,
                                 const int64_t *__restrict__ offs,
@@ -90,8 +197,8 @@ __global__ void k_radix_scatter(int64_t n, const unsigned long long *__restrict_
         goff[t] = offs[(int64_t)t * ntiles + blockIdx.x];
     }
     unsigned lt = (1u << lane) - 1u;
-    int64_t tile0 = blockIdx.x * (int64_t)SORT_TILE;
-    for (int r = 0; r < SORT_ROUNDS; r++) {
+    int64_t tile0 = blockIdx.x * (int64_t)(SORT_THREADS * ROUNDS);
+    for (int r = 0; r < ROUNDS; r++) {
         for (int t = threadIdx.x; t < W * 256; t += blockDim.x) (&cnt[0][0])[t] = 0;
         __syncthreads();
         int64_t i = tile0 + r * SORT_THREADS + threadIdx.x;
@@ -122,15 +229,6 @@ __global__ void k_radix_scatter(int64_t n, const unsigned long long *__restrict_
         }
         __syncthreads();
     }
-}
-
-__device__ __forceinline__ int64_t warp_incl_scan(int64_t v) {
-    int lane = threadIdx.x & 31;
-    for (int o = 1; o < 32; o <<= 1) {
-        int64_t t = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += t;
-    }
-    return v;
 }
 
 // exclusive scan of one tile; block total to sums[blockIdx.x]
@@ -256,13 +354,35 @@ cudaError_t exclusive_scan_i64(const int64_t *in, int64_t *out, int64_t n, int64
     return launch_check();
 }
 
-static int64_t scan_tmp_size(int64_t n) {
-    int64_t t = 0;
-    while (n > SCAN_TILE) {
-        n = (n + SCAN_TILE - 1) / SCAN_TILE;
-        t += n;
+template <int ROUNDS>
+static cudaError_t radix_sort(hydro_ctx *c, int64_t n, int bits, stream_t st) {
+    constexpr int64_t TILE = SORT_THREADS * ROUNDS;
+    const int64_t ntiles = (n + TILE - 1) / TILE, nh = 256 * ntiles;
+    const int passes = (bits + 7) / 8;
+    HYD_CUDA(c->d_scan_tmp.ensure(2 * nh + TOTAL_COPIES * 256 * passes));
+    int64_t *hist = c->d_scan_tmp.get();
+    int64_t *offs = hist + nh;
+    unsigned long long *total = reinterpret_cast<unsigned long long *>(offs + nh);
+    HYD_CUDA(cudaMemsetAsync(total, 0, TOTAL_COPIES * 256 * passes * sizeof(unsigned long long), st));
+    unsigned long long *ka = c->d_keys.get(), *kb = c->d_keys_alt.get();
+    int32_t *va = c->d_perm.get(), *vb = c->d_perm_alt.get();
+    for (int shift = 0; shift < bits; shift += 8) {
+        k_radix_hist<ROUNDS><<<(unsigned)ntiles, SORT_THREADS, 0, st>>>(n, ka, shift, ntiles, hist,
+                                                                        total);
+        HYD_CUDA(launch_check());
+        k_radix_offsets<<<256, OFFS_THREADS, 0, st>>>(ntiles, hist, total, offs);
+        HYD_CUDA(launch_check());
+        total += TOTAL_COPIES * 256;
+        k_radix_scatter<ROUNDS><<<(unsigned)ntiles, SORT_THREADS, 0, st>>>(n, ka, va, shift, ntiles,
+                                                                           offs, kb, vb);
+        HYD_CUDA(launch_check());
+        unsigned long long *tk = ka; ka = kb; kb = tk;
+        int32_t *tv = va; va = vb; vb = tv;
     }
-    return t + 16;
+    if (va != c->d_perm.get())
+        HYD_CUDA(cudaMemcpyAsync(c->d_perm.get(), va, n * sizeof(int32_t),
+                                 cudaMemcpyDeviceToDevice, st));
+    return cudaSuccess;
 }
 
 cudaError_t sort_particles(hydro_ctx *c, const hydro_particles *p, stream_t st) {
@@ -272,34 +392,27 @@ cudaError_t sort_particles(hydro_ctx *c, const hydro_particles *p, stream_t st) 
     HYD_CUDA(c->d_keys_alt.ensure(n));
     HYD_CUDA(c->d_perm.ensure(n));
     HYD_CUDA(c->d_perm_alt.ensure(n));
-    int64_t ntiles = (n + SORT_TILE - 1) / SORT_TILE;
-    int64_t nh = 256 * ntiles;
-    HYD_CUDA(c->d_scan_tmp.ensure(2 * nh + scan_tmp_size(nh)));
-    k_morton<<<grid_for(n, 256), 256, 0, st>>>(n, p->x, p->y, p->z, c->d_box_off.get(),
-                                                 c->plan.nbox, c->d_boxes.get(), c->d_keys.get(),
-                                                 c->d_perm.get());
-    HYD_CUDA(launch_check());
+    // (the ranking's counts, zero at first, or the radix passes' values)
     int bits = 30;
     while ((1ll << (bits - 30)) < c->plan.nbox) bits++;
-    int64_t *hist = c->d_scan_tmp.get();
-    int64_t *offs = hist + nh;
-    int64_t *tmp = offs + nh;
-    unsigned long long *ka = c->d_keys.get(), *kb = c->d_keys_alt.get();
-    int32_t *va = c->d_perm.get(), *vb = c->d_perm_alt.get();
-    for (int shift = 0; shift < bits; shift += 8) {
-        k_radix_hist<<<(unsigned)ntiles, SORT_THREADS, 0, st>>>(n, ka, shift, ntiles, hist);
+    const bool ranked = n <= RANK_SORT_MAX && bits <= 32;
+    int32_t *vals = ranked ? c->d_perm_alt.get() : c->d_perm.get();
+    k_morton<<<grid_for(n, 256), 256, 0, st>>>(n, p->x, p->y, p->z, c->d_box_off.get(),
+                                                 c->plan.nbox, c->d_boxes.get(), c->d_keys.get(),
+                                                 vals, ranked);
+    HYD_CUDA(launch_check());
+    if (ranked) {
+        const dim3 grid(grid_for(n, RANK_I), grid_for(n, RANK_J));
+        k_rank_count<<<grid, RANK_I, 0, st>>>(n, c->d_keys.get(), vals);
         HYD_CUDA(launch_check());
-        HYD_CUDA(exclusive_scan_i64(hist, offs, nh, tmp, st));
-        k_radix_scatter<<<(unsigned)ntiles, SORT_THREADS, 0, st>>>(n, ka, va, shift, ntiles, offs,
-                                                                   kb, vb);
-        HYD_CUDA(launch_check());
-        unsigned long long *tk = ka; ka = kb; kb = tk;
-        int32_t *tv = va; va = vb; vb = tv;
+        k_rank_scatter<<<grid_for(n, 256), 256, 0, st>>>(n, vals, c->d_perm.get());
+        return launch_check();
     }
-    if (va != c->d_perm.get())
-        HYD_CUDA(cudaMemcpyAsync(c->d_perm.get(), va, n * sizeof(int32_t),
-                                 cudaMemcpyDeviceToDevice, st));
-    return cudaSuccess;
+    if (n >= 152 * 4 * SORT_THREADS * SORT_ROUNDS)
+        return radix_sort<SORT_ROUNDS>(c, n, bits, st);
+    if (n >= 152 * 2 * SORT_THREADS * SORT_ROUNDS / 4)
+        return radix_sort<SORT_ROUNDS / 4>(c, n, bits, st);
+    return radix_sort<1>(c, n, bits, st);
 }
 
 cudaError_t gather_state(hydro_ctx *c, const hydro_particles *p, const double *h_in,

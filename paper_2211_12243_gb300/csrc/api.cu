@@ -376,8 +376,11 @@ int hydro_set_boxes(hydro_ctx *c, int64_t nbox, const int64_t *box_off, const do
         for (int a = 0; a < 3; a++) {
             boxes[k].L[a] = box_len[3 * k + a];
             boxes[k].s[a] = (float)(box_len[3 * k + a] / 4294967296.0);
+            boxes[k].rL[a] = 1.0 / box_len[3 * k + a];
         }
         boxes[k].pad = 0.f;
+        boxes[k].Lmax = std::max(box_len[3 * k], std::max(box_len[3 * k + 1], box_len[3 * k + 2]));
+        boxes[k].rLmax = 1.0 / boxes[k].Lmax;
     }
     API_CUDA(upload(c->d_boxes, boxes));
     API_CUDA(upload(c->d_box_off, P.box_off));

@@ -677,20 +677,6 @@ __global__ void k_grow_search(int64_t n, uint8_t *__restrict__ active, double *_
     }
 }
 
-__global__ void k_fixed64(int64_t n, const double *__restrict__ xs, const double *__restrict__ ys,
-                          const double *__restrict__ zs, const int32_t *__restrict__ pbox,
-                          const Box *__restrict__ boxes, uint64_t *__restrict__ qx,
-                          uint64_t *__restrict__ qy, uint64_t *__restrict__ qz) {
-    int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (s >= n) return;
-    const Box bx = boxes[pbox[s]];
-    const double two64 = 18446744073709551616.0;
-    double t;
-    t = xs[s] / bx.L[0] * two64; qx[s] = t >= two64 ? 0ull : (uint64_t)t;
-    t = ys[s] / bx.L[1] * two64; qy[s] = t >= two64 ? 0ull : (uint64_t)t;
-    t = zs[s] / bx.L[2] * two64; qz[s] = t >= two64 ? 0ull : (uint64_t)t;
-}
-
 inline unsigned grid_for(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
 }  // namespace
@@ -724,18 +710,7 @@ cudaError_t run_density(hydro_ctx *c, bool only_active, bool compact, stream_t s
     a.nlist = &c->d_cnt->nguard;
     HYD_CUDA(cudaMemsetAsync(&c->d_cnt->search_fail, 0, sizeof(int), st));
     if (c->cfg.precision == HYDRO_MIXED) {
-        // 64-bit fixed-point copies for the refinement step (xs.. are sorted)
-        // (positions are fixed within a step: the solves of selected
-        // particles reuse the copies of the step's first, full solve; the
-        // sub-steps of individual timesteps move every particle)
-        HYD_CUDA(c->d_q64.ensure((size_t)3 * n));
-        uint64_t *q64 = c->d_q64.get();
-        if (!only_active || c->rung_live) {
-            k_fixed64<<<grid_for(n, 256), 256, 0, st>>>(n, c->d_xs.get(), c->d_ys.get(),
-                                                         c->d_zs.get(), c->d_pbox.get(),
-                                                         c->d_boxes.get(), q64, q64 + n, q64 + 2 * n);
-            HYD_CUDA(launch_check());
-        }
+        const uint64_t *q64 = c->d_q64.get();   // (gather_state)
         if (guard && only_active)
             k_density_list<float><<<152 * 8, DENS_THREADS, 0, st>>>(a, q64, q64 + n, q64 + 2 * n,
                                                                    c->d_recf.get());

@@ -84,6 +84,34 @@ __device__ __forceinline__ double sqrt64(double x) {
     return dpos(x) ? fma(fma(-s, s, x), 0.5 * r, s) : 0.0;
 }
 
+// a / b from y = 1/b (within an ulp): each step adds the exactly computed
+// remainder a - b q times y.  One step leaves the quotient within a hair of half
+// an ulp; two give the correctly rounded one (the remainder of a quotient within
+// one ulp is exact, and its product with y is far below the distance of any
+// quotient from a rounding boundary).
+__device__ __forceinline__ double div1(double a, double b, double y) {
+    const double q = a * y;
+    return fma(fma(-q, b, a), y, q);
+}
+__device__ __forceinline__ double div2(double a, double b, double y) {
+    const double q = div1(a, b, y);
+    return fma(fma(-q, b, a), y, q);
+}
+
+// finite, without the FP64 pipe
+__device__ __forceinline__ bool dfinite(double v) {
+    return ((unsigned)(dbits(v) >> 52) & 0x7ffu) != 0x7ffu;
+}
+
+// floor(q 2^64) for 0 <= q < 1 (0 below 2^-64)
+__device__ __forceinline__ unsigned long long fixed64(double q) {
+    const unsigned long long b = (unsigned long long)dbits(q);
+    const int e = (int)(b >> 52);
+    const unsigned long long m = (b & 0xfffffffffffffull) | (1ull << 52);
+    const int shift = e - 1011;
+    return shift >= 0 ? m << shift : shift > -64 && e > 0 ? m >> -shift : 0ull;
+}
+
 // t^n, n >= 1 uniform over the warp
 __device__ __forceinline__ double ipow64(double t, int n) {
     double r = (n & 1) ? t : 1.0;

@@ -65,6 +65,8 @@ struct Box {
     double L[3];      // lengths
     float s[3];       // L / 2^32 (metres per fixed-point unit)
     float pad;
+    double rL[3];     // 1 / L
+    double Lmax, rLmax;   // the longest side and 1 / Lmax
 };
 
 // scalars the device reads every step

@@ -2,6 +2,7 @@
 // array of §2.2.1: spatially close particles become contiguous so that a
 // bucket of 32 is a compact region, §2.2.3), a stable LSD radix sort, and the
 // gathers/scatters between the caller's order and the sorted order.
+#include "fp64.cuh"
 #include "hydro_internal.cuh"
 
 namespace hyd {
@@ -27,11 +28,29 @@ __device__ __forceinline__ uint32_t spread10(uint32_t v) {
     return v;
 }
 
-__device__ __forceinline__ uint32_t to_fixed(double x, double L) {
-    double t = x / L * 4294967296.0;
-    if (t >= 4294967296.0) t -= 4294967296.0;
-    if (t < 0.0) t = 0.0;
-    return (uint32_t)t;
+// The position as a fraction of the box in 64-bit fixed point, and its leading
+// 32 bits: floor(x / L 2^64) and floor(x / L 2^32) of the correctly rounded
+// quotient, by five FP64 instructions (fp64.cuh) and integer operations.  A
+// position at or beyond L comes back in at 0 (q64) or wraps once (q32), a
+// negative one is 0.
+__device__ __forceinline__ uint32_t to_fixed(double x, double L, double rL, uint64_t &q64) {
+    const double t = div2(x, L, rL);
+    if (dpos(t) && dlt_pos(t, 1.0)) {
+        q64 = fixed64(t);
+        return (uint32_t)(q64 >> 32);
+    }
+    q64 = 0;
+    double u = t * 4294967296.0;
+    if (u >= 4294967296.0) u -= 4294967296.0;
+    if (u < 0.0) u = 0.0;
+    return (uint32_t)u;
+}
+
+// floor(x / Lmax 1024), at most 1023
+__device__ __forceinline__ uint32_t to_cell(double x, const Box &bx) {
+    const double t = div2(x, bx.Lmax, bx.rLmax);
+    if (!dpos(t)) return 0u;
+    return dlt_pos(t, 1.0) ? (uint32_t)(fixed64(t) >> 54) : 1023u;
 }
 
 __device__ __forceinline__ int box_of(const int64_t *box_off, int64_t nbox, int64_t i) {
@@ -54,10 +73,7 @@ __global__ void k_morton(int64_t n, const double *__restrict__ x, const double *
     const Box bx = boxes[b];
     // cubic cells of side Lmax / 1024 on every axis, so that a run of
     // consecutive keys is a compact region also in elongated boxes
-    const double Lmax = fmax(bx.L[0], fmax(bx.L[1], bx.L[2]));
-    uint32_t qx = min((uint32_t)(x[i] / Lmax * 1024.0), 1023u);
-    uint32_t qy = min((uint32_t)(y[i] / Lmax * 1024.0), 1023u);
-    uint32_t qz = min((uint32_t)(z[i] / Lmax * 1024.0), 1023u);
+    const uint32_t qx = to_cell(x[i], bx), qy = to_cell(y[i], bx), qz = to_cell(z[i], bx);
     uint32_t m = (spread10(qx) << 2) | (spread10(qy) << 1) | spread10(qz);
     keys[i] = ((unsigned long long)b << 30) | m;
     vals[i] = zero ? 0 : (int32_t)i;
@@ -275,7 +291,8 @@ __global__ void k_gather_state(int64_t n, const int32_t *__restrict__ perm,
                                double *__restrict__ zs, uint32_t *__restrict__ qx,
                                uint32_t *__restrict__ qy, uint32_t *__restrict__ qz,
                                double *__restrict__ hsorted, double *__restrict__ hs,
-                               int32_t *__restrict__ pbox, R *__restrict__ rec) {
+                               int32_t *__restrict__ pbox, R *__restrict__ rec,
+                               uint64_t *__restrict__ q64) {
     int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (s >= n) return;
     int o = perm[s];
@@ -283,8 +300,12 @@ __global__ void k_gather_state(int64_t n, const int32_t *__restrict__ perm,
     const Box bx = boxes[b];
     double px = x[o], py = y[o], pz = z[o];
     xs[s] = px; ys[s] = py; zs[s] = pz;
-    uint32_t ux = to_fixed(px, bx.L[0]), uy = to_fixed(py, bx.L[1]), uz = to_fixed(pz, bx.L[2]);
+    uint64_t wx, wy, wz;
+    const uint32_t ux = to_fixed(px, bx.L[0], bx.rL[0], wx), uy = to_fixed(py, bx.L[1], bx.rL[1], wy),
+                   uz = to_fixed(pz, bx.L[2], bx.rL[2], wz);
     qx[s] = ux; qy[s] = uy; qz[s] = uz;
+    // (mixed path: the density refinement's positions)
+    if (sizeof(R) == 4) { q64[s] = wx; q64[n + s] = wy; q64[2 * n + s] = wz; }
     double h = h_in[o];
     hsorted[s] = h;
     double r = h_search ? h_search[o] : margin * h;
@@ -425,18 +446,19 @@ cudaError_t gather_state(hydro_ctx *c, const hydro_particles *p, const double *h
     const bool mixed = c->cfg.precision == HYDRO_MIXED;
     if (mixed) {
         HYD_CUDA(c->d_recf.ensure((size_t)n * REC));
+        HYD_CUDA(c->d_q64.ensure((size_t)3 * n));
         k_gather_state<float><<<grid_for(n, 256), 256, 0, st>>>(
             n, c->d_perm.get(), c->d_box_off.get(), c->plan.nbox, c->d_boxes.get(), p->x, p->y,
             p->z, h_in, h_search, margin, c->d_xs.get(), c->d_ys.get(), c->d_zs.get(),
             c->d_qx.get(), c->d_qy.get(), c->d_qz.get(), c->d_hsorted.get(), c->d_hs.get(),
-            c->d_pbox.get(), c->d_recf.get());
+            c->d_pbox.get(), c->d_recf.get(), c->d_q64.get());
     } else {
         HYD_CUDA(c->d_recd.ensure((size_t)n * REC));
         k_gather_state<double><<<grid_for(n, 256), 256, 0, st>>>(
             n, c->d_perm.get(), c->d_box_off.get(), c->plan.nbox, c->d_boxes.get(), p->x, p->y,
             p->z, h_in, h_search, margin, c->d_xs.get(), c->d_ys.get(), c->d_zs.get(),
             c->d_qx.get(), c->d_qy.get(), c->d_qz.get(), c->d_hsorted.get(), c->d_hs.get(),
-            c->d_pbox.get(), c->d_recd.get());
+            c->d_pbox.get(), c->d_recd.get(), nullptr);
     }
     HYD_CUDA(launch_check());
     if (want_Q) {

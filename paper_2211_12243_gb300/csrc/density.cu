@@ -195,12 +195,14 @@ struct NewtonF {
 };
 
 // A particle's list walked by one lane (W = 1) or by the 32 of a warp (a guard
-// round's few particles, whose lists at the doubled radius are long): entry k
-// goes to lane k mod W, sums are folded over the lanes.  A warp keeps the
-// separations of the first CACHE entries; a lane on its own gathers them again
-// in every pass (a running step's h takes one or two passes; keeping 16 to 64
-// of a thread's separations in shared memory took its L1 and was between 7 %
-// faster and 50 % slower).
+// round's few particles, whose lists at the doubled radius are long).  A warp
+// gathers the separations in parallel, once, into shared memory (the first
+// CACHE), and evaluates the refinement's entries in parallel; the sums
+// themselves are taken in the list's order in both forms, so a particle's root
+// does not depend on which form solves it.  A lane on its own gathers the
+// separations again in every pass (a running step's h takes one or two passes;
+// keeping 16 to 64 of a thread's separations in shared memory took its L1 and
+// was between 7 % faster and 50 % slower).
 template <int W>
 struct Walk {
     static constexpr int CACHE = W == 1 ? 0 : DENS_CACHE;
@@ -246,8 +248,11 @@ __device__ __forceinline__ NewtonF newton_float(const DensArgs &a, const Sep &se
     const float ftol = 2e-6f;
     float lo = 0.f, hi = -1.f;
     const int c0 = min(c, Walk<W>::CACHE);
+    if (W > 1) {
 #pragma unroll 4
-    for (int k = wk.lane; k < c0; k += W) wk.rs[k] = sep(idx[k]);
+        for (int k = wk.lane; k < c0; k += W) wk.rs[k] = sep(idx[k]);
+        __syncwarp();
+    }
     for (int it = 1; it <= max_iter; it++) {
         o.it = it;
         float f = 0.f, mq = 0.f, ih = 1.f / h;
@@ -256,40 +261,34 @@ __device__ __forceinline__ NewtonF newton_float(const DensArgs &a, const Sep &se
         // float r < X (1 + 1e-4) leaves the list complete for every
         // r < X (1 + 5e-5) when X > L / 65536 (compaction is skipped below that)
         const bool shrink = a.compact && hi > xmin && hi < 0.8f * hsi;
-        if (shrink) {
-            const float keep = hi * 1.0001f;
-            int w = 0;
-            for (int k0 = 0; k0 < c; k0 += W) {
-                const int k = k0 + wk.lane;
-                const bool in = W == 1 || k < c;
-                const int j = in ? idx[k] : 0;
-                const float r = !in ? INFINITY : k < Walk<W>::CACHE ? wk.rs[k] : sep(j);
-                wk.keep(r < keep, idx, j, r, w);
-                float fv, mv;
-                kernel_f<float>(a.kernel, r * ih, fv, mv);
-                f += fv;
-                mq += mv;
+        const float keep = hi * 1.0001f;
+        int w = 0;
+        for (int k = 0; k < c; k++) {   // (every lane of a warp: the sums are in order)
+            float r;
+            if (W == 1) {
+                const int j = idx[k];
+                r = sep(j);
+                if (shrink && r < keep) idx[w++] = j;
+            } else {
+                r = k < Walk<W>::CACHE ? wk.rs[k] : sep(idx[k]);
             }
+            float fv, mv;
+            kernel_f<float>(a.kernel, r * ih, fv, mv);
+            f += fv;
+            mq += mv;
+        }
+        if (shrink) {
+            if (W > 1)
+                for (int k0 = 0; k0 < c; k0 += W) {
+                    const int k = k0 + wk.lane;
+                    const int j = k < c ? idx[k] : 0;
+                    const float r = k >= c ? INFINITY : k < Walk<W>::CACHE ? wk.rs[k] : sep(j);
+                    wk.keep(r < keep, idx, j, r, w);
+                }
             c = w;
             o.comp = hi * 1.00005f;
             hsi = o.comp;
-        } else {
-            const int cs = min(c, Walk<W>::CACHE);
-            for (int k = wk.lane; k < cs; k += W) {
-                float fv, mv;
-                kernel_f<float>(a.kernel, wk.rs[k] * ih, fv, mv);
-                f += fv;
-                mq += mv;
-            }
-            for (int k = cs + wk.lane; k < c; k += W) {
-                float fv, mv;
-                kernel_f<float>(a.kernel, sep(idx[k]) * ih, fv, mv);
-                f += fv;
-                mq += mv;
-            }
         }
-        f = wk.sum(f);
-        mq = wk.sum(mq);
         float g = Kn * f - N;
         float dg = Kn * mq * ih;
         if (g == 0.f) { o.conv = true; break; }
@@ -536,47 +535,53 @@ __device__ __forceinline__ void dens_one(const DensArgs &a, const uint64_t *__re
         const int j = in ? idx[k] : 0;
         const float rf = !in ? INFINITY : k < Walk<W>::CACHE ? wk.rs[k] : sep(j);
         if (fin) wk.keep(rf < keep, idx, j, rf, w);
-        if (rf >= hcut) continue;
-        long long ix = (long long)(q64x[j] - xi64);
-        long long iy = (long long)(q64y[j] - yi64);
-        long long iz = (long long)(q64z[j] - zi64);
-        df dx = df_mulf(from_i64(ix), sx);
-        df dy = df_mulf(from_i64(iy), sy);
-        df dz = df_mulf(from_i64(iz), sz);
-        df r2 = df_add(df_add(df_mul(dx, dx), df_mul(dy, dy)), df_mul(dz, dz));
-        df q = df_mul(df_sqrt(r2), ih);
-        if (q.hi >= 1.f) continue;
-        df one = {1.f, 0.f};
-        df t = df_sub(one, q);
-        df t2 = df_mul(t, t);
-        if (a.kernel == 0) {
-            df t3 = df_mul(t2, t);
-            df fv = df_mul(df_mul(t3, t), df_add(one, df_mulf(q, 4.f)));
-            df mv = df_mulf(df_mul(df_mul(q, q), t3), 20.f);
-            F = df_add(F, fv);
-            MQ = df_add(MQ, mv);
-        } else {
-            df q2 = df_mul(q, q);
-            df fv, mv;
-            if (q.hi <= 0.5f) {
-                fv = df_add(df_sub(one, df_mulf(q2, 6.f)), df_mulf(df_mul(q2, q), 6.f));
-                mv = df_sub(df_mulf(q2, 12.f), df_mulf(df_mul(q2, q), 18.f));
-            } else {
-                fv = df_mulf(df_mul(t2, t), 2.f);
-                mv = df_mulf(df_mul(q, t2), 6.f);
+        df fv = {0.f, 0.f}, mv = {0.f, 0.f};
+        bool on = rf < hcut;
+        if (on) {
+            long long ix = (long long)(q64x[j] - xi64);
+            long long iy = (long long)(q64y[j] - yi64);
+            long long iz = (long long)(q64z[j] - zi64);
+            df dx = df_mulf(from_i64(ix), sx);
+            df dy = df_mulf(from_i64(iy), sy);
+            df dz = df_mulf(from_i64(iz), sz);
+            df r2 = df_add(df_add(df_mul(dx, dx), df_mul(dy, dy)), df_mul(dz, dz));
+            df q = df_mul(df_sqrt(r2), ih);
+            on = q.hi < 1.f;
+            if (on) {
+                df one = {1.f, 0.f};
+                df t = df_sub(one, q);
+                df t2 = df_mul(t, t);
+                if (a.kernel == 0) {
+                    df t3 = df_mul(t2, t);
+                    fv = df_mul(df_mul(t3, t), df_add(one, df_mulf(q, 4.f)));
+                    mv = df_mulf(df_mul(df_mul(q, q), t3), 20.f);
+                } else {
+                    df q2 = df_mul(q, q);
+                    if (q.hi <= 0.5f) {
+                        fv = df_add(df_sub(one, df_mulf(q2, 6.f)), df_mulf(df_mul(q2, q), 6.f));
+                        mv = df_sub(df_mulf(q2, 12.f), df_mulf(df_mul(q2, q), 18.f));
+                    } else {
+                        fv = df_mulf(df_mul(t2, t), 2.f);
+                        mv = df_mulf(df_mul(q, t2), 6.f);
+                    }
+                }
             }
-            F = df_add(F, fv);
-            MQ = df_add(MQ, mv);
+        }
+        if (W == 1) {
+            if (on) {
+                F = df_add(F, fv);
+                MQ = df_add(MQ, mv);
+            }
+        } else {
+            // in the list's order
+            for (unsigned m = __ballot_sync(0xffffffffu, on); m; m &= m - 1) {
+                const int l = __ffs(m) - 1;
+                F = df_add(F, {__shfl_sync(0xffffffffu, fv.hi, l), __shfl_sync(0xffffffffu, fv.lo, l)});
+                MQ = df_add(MQ, {__shfl_sync(0xffffffffu, mv.hi, l), __shfl_sync(0xffffffffu, mv.lo, l)});
+            }
         }
     }
-    if (W > 1) {
-        for (int o = W / 2; o > 0; o >>= 1) {
-            F = df_add(F, {__shfl_xor_sync(0xffffffffu, F.hi, o), __shfl_xor_sync(0xffffffffu, F.lo, o)});
-            MQ = df_add(MQ, {__shfl_xor_sync(0xffffffffu, MQ.hi, o),
-                             __shfl_xor_sync(0xffffffffu, MQ.lo, o)});
-        }
-        if (!lead) return;
-    }
+    if (!lead) return;
     // g = Kn F - N, dg = Kn MQ / h  ->  h_new = h - (F - N/Kn) h / MQ
     double Fd = (double)F.hi + (double)F.lo;
     double MQd = (double)MQ.hi + (double)MQ.lo;

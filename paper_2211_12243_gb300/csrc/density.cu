@@ -58,7 +58,7 @@ struct DensArgs {
     DevCounters *cnt;
     bool rank;                // full solve: rank the CTA's 128 particles by list length
     const int32_t *list;      // the guard round's particles, their count on the device
-    const int *nlist;         // (k_density_list)
+    const int *nlist;         // (k_density_list; NULL: every particle)
 };
 
 // Growth of the search radius hs after a failed solve.  First failure
@@ -140,6 +140,10 @@ __device__ __forceinline__ df from_i64(long long v) {
 // ------------------------------------------------- the iteration in float
 constexpr int DENS_THREADS = 128;
 static_assert(DENS_THREADS == RANK_THREADS, "the ranked tiles take 128 threads a round");
+// particles that a warp each solves faster than a thread each (4,096: 78 -> 47 us,
+// 8,000: 84 -> 67 us, 17,576: 82 -> 108 us)
+constexpr int64_t DENS_WARP_MAX = 8192;
+
 // separations a warp that walks one list keeps in shared memory
 constexpr int DENS_CACHE = 1536;
 
@@ -649,11 +653,12 @@ k_density_list(DensArgs a, const uint64_t *__restrict__ q64x, const uint64_t *__
     __shared__ float rs[DENS_THREADS / 32][DENS_CACHE];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const Walk<32> wk{rs[warp], lane};
-    const int nl = *a.nlist;
+    const int nl = a.list ? *a.nlist : (int)a.n;
     for (int t = blockIdx.x * (DENS_THREADS / 32) + warp; t < nl; t += gridDim.x * (DENS_THREADS / 32)) {
+        const int64_t s = a.list ? a.list[t] : t;
         __syncwarp();
-        if constexpr (sizeof(R) == 8) dens_one<32>(a, rec, wk, a.list[t]);
-        else dens_one<32>(a, q64x, q64y, q64z, rec, wk, a.list[t]);
+        if constexpr (sizeof(R) == 8) dens_one<32>(a, rec, wk, s);
+        else dens_one<32>(a, q64x, q64y, q64z, rec, wk, s);
     }
 }
 
@@ -714,19 +719,29 @@ cudaError_t run_density(hydro_ctx *c, bool only_active, bool compact, stream_t s
     a.list = c->d_guard_idx.get();
     a.nlist = &c->d_cnt->nguard;
     HYD_CUDA(cudaMemsetAsync(&c->d_cnt->search_fail, 0, sizeof(int), st));
+    // a warp per particle: the guard round's list, or every particle of a set
+    // so small that a thread each would leave the GPU idle
+    // (the few buckets of a sparse sub-step of individual timesteps too)
+    const bool listed = guard && only_active;
+    const bool sparse = c->rung_live && only_active && c->rung_touch_n >= 0 &&
+                        c->rung_touch_n * BUCKET <= DENS_WARP_MAX;
+    const bool warps = listed || sparse || n <= DENS_WARP_MAX;
+    if (!listed) a.list = nullptr;
+    const unsigned grid = !warps ? grid_for(n, DENS_THREADS)
+        : listed ? 152u * 8u : std::min(152u * 8u, grid_for(n * 32, DENS_THREADS));
     if (c->cfg.precision == HYDRO_MIXED) {
         const uint64_t *q64 = c->d_q64.get();   // (gather_state)
-        if (guard && only_active)
-            k_density_list<float><<<152 * 8, DENS_THREADS, 0, st>>>(a, q64, q64 + n, q64 + 2 * n,
-                                                                   c->d_recf.get());
+        if (warps)
+            k_density_list<float><<<grid, DENS_THREADS, 0, st>>>(a, q64, q64 + n, q64 + 2 * n,
+                                                                c->d_recf.get());
         else
-            k_density_mixed<<<grid_for(n, DENS_THREADS), DENS_THREADS, 0, st>>>(
-                a, q64, q64 + n, q64 + 2 * n, c->d_recf.get());
-    } else if (guard && only_active) {
-        k_density_list<double><<<152 * 8, DENS_THREADS, 0, st>>>(a, nullptr, nullptr, nullptr,
-                                                                c->d_recd.get());
+            k_density_mixed<<<grid, DENS_THREADS, 0, st>>>(a, q64, q64 + n, q64 + 2 * n,
+                                                           c->d_recf.get());
+    } else if (warps) {
+        k_density_list<double><<<grid, DENS_THREADS, 0, st>>>(a, nullptr, nullptr, nullptr,
+                                                              c->d_recd.get());
     } else {
-        k_density_f64<<<grid_for(n, DENS_THREADS), DENS_THREADS, 0, st>>>(a, c->d_recd.get());
+        k_density_f64<<<grid, DENS_THREADS, 0, st>>>(a, c->d_recd.get());
     }
     return launch_check();
 }

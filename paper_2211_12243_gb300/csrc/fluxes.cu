@@ -223,6 +223,7 @@ cudaError_t run_fluxes(hydro_ctx *c, double dt, const double *dt_dev, stream_t s
     a.dt0 = c->rung_dt0;
     a.bucket_ids = nullptr;
     a.queue = c->flux_queue ? &c->d_cnt->flux_cursor : nullptr;
+    a.split = 0;   // (the launchers set it)
     if (c->rung_live && c->rung_touch_n >= 0) {
         a.bucket_ids = c->d_touch.get();
         a.nbucket = c->rung_touch_n;

@@ -93,3 +93,25 @@ def test_density_where_the_float_iteration_does_not_settle(orc, hyd, n):
     H.density(s)
     assert np.max(np.abs(s["h"].cpu().numpy() / h - 1)) < 1e-12
     H.close()
+
+
+@pytest.mark.parametrize("n", [131, 8192, 8193])
+def test_warp_and_thread_solves_agree(orc, hyd, n):
+    """either side of the size up to which a warp solves each particle"""
+    import torch
+    rng = np.random.default_rng(n)
+    c = rng.random((3, n))
+    n_ngb = 32.0 if n > 1000 else 18.0
+    h0 = np.full(n, np.cbrt(3 * n_ngb / (4 * np.pi * max(n, 40))))
+    h, om, _, st = orc.density(orc.config(n_ngb=n_ngb), *c, np.ones(3), h0)
+    assert st == 0
+    for precision in ("fp64", "mixed"):
+        H = hyd.Hydro(hyd.default_config(precision=precision, n_ngb=n_ngb))
+        H.set_boxes(np.array([0, n], dtype=np.int64), np.ones(3))
+        dev = lambda v: torch.as_tensor(np.ascontiguousarray(v), device="cuda")
+        s = {"x": dev(c[0]), "y": dev(c[1]), "z": dev(c[2]), "h": dev(h0), "omega": dev(np.zeros(n))}
+        H.build_neighbours(s, dev(np.minimum(h * 1.2, 0.49)), export=False)
+        H.density(s)
+        ok = h < 0.48
+        assert np.max(np.abs(s["h"].cpu().numpy() / h - 1)[ok]) < 1e-12
+        H.close()

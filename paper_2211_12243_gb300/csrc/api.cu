@@ -558,8 +558,8 @@ static int guard_lists(hydro_ctx *c, bool first, cudaStream_t st) {
 // particles, seeing the other within its own h).  So only the buckets
 // holding such particles need fresh lists and a flux walk: a reverse walk
 // of the tree from every starting particle flags them (ACT_REDO), and when
-// they are few their lists are rebuilt into the overflow region and the
-// flux kernel walks only them; the other lists are stale and unused.  Too
+// they are few only their rows are rebuilt and the flux kernel walks only
+// them; the other lists are stale and unused.  Too
 // many, or no room: every list, every bucket.
 static int rung_lists(hydro_ctx *c, cudaStream_t st) {
     const int64_t n = c->plan.n, nb = c->plan.nbucket;
@@ -574,8 +574,7 @@ static int rung_lists(hydro_ctx *c, cudaStream_t st) {
         API_CUDA(c->d_touch.ensure(nb));
         API_CUDA(cudaMemcpyAsync(c->d_touch.get(), c->d_ovf.get(), (size_t)nq * sizeof(int32_t),
                                  cudaMemcpyDeviceToDevice, st));
-        API_CUDA(set_u64(&c->d_cnt->list_cursor, (unsigned long long)n * c->list_cap, st));
-        API_CUDA(build_lists_queued(c, nq, st));
+        API_CUDA(build_rows_of(c, c->d_touch.get(), nq, st));
         int fl = 0;
         unsigned long long cursor = 0;
         API_CUDA(cudaMemcpyAsync(&fl, &c->d_cnt->flags, sizeof(int), cudaMemcpyDeviceToHost, st));

@@ -349,6 +349,7 @@ cudaError_t build_tree(hydro_ctx *c, stream_t st);
 cudaError_t raise_tree(hydro_ctx *c, stream_t st);
 cudaError_t build_lists(hydro_ctx *c, int cap, stream_t st);
 cudaError_t build_lists_queued(hydro_ctx *c, int nq, stream_t st);
+cudaError_t build_rows_of(hydro_ctx *c, const int32_t *buckets, int nq, stream_t st);
 cudaError_t rebuild_active_lists(hydro_ctx *c, int *nq, stream_t st, bool guard = false);
 // ACT_REDO on the guard round's particles and on every particle i with one
 // of them in its list (r_ia < h_i), found by walks of the bucket tree

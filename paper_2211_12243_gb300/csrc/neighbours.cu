@@ -152,6 +152,7 @@ struct ListArgs {
     int64_t capacity;
     DevCounters *cnt;
     int cap;   // fixed slots per particle (row s at s cap)
+    const int32_t *rows_of; // LIST_ROWS: only these nbucket buckets (NULL: all)
     int32_t *ovf_list;      // queued bucket ids
     int *ovf_count;
     bool nq_dev;            // modes 1, 2: the queue's length is *ovf_count
@@ -236,6 +237,7 @@ __global__ void __launch_bounds__(LIST_WARPS * 32, LIST_CTAS) k_build_lists(List
         const int sub = SPLIT > 1 ? (int)(item % SPLIT) * OW : 0;
         const bool valid = item < nitem;
         if (valid && MODE != LIST_ROWS) b = a.ovf_list[b];
+        if (valid && MODE == LIST_ROWS && a.rows_of) b = a.rows_of[b];
         const int bcnt = valid ? a.node_cnt[b] : 0;
         bool over = false;
         // (warp-uniform; the warps of a CTA meet at the end of LIST_ROWS)
@@ -558,20 +560,103 @@ __global__ void __launch_bounds__(LIST_WARPS * 32, LIST_CTAS) k_build_lists(List
     }
 }
 
+// One particle's walk of the tree by a warp: visit(first, count) is called for
+// every bucket that `near` (a lane's test of a child's box) lets pass, in the
+// order of k_build_lists's walk (internal nodes last pushed first, buckets in
+// ascending order), with the lane's particle of the bucket prefetched: the walk
+// is a chain of dependent loads, so the next bucket's are issued before one is
+// visited.  False when the stack overflowed (cannot happen for trees of
+// MAX_LEVELS levels).
+struct Spot {
+    uint32_t qx, qy, qz;
+};
+
+template <typename Near, typename Visit>
+__device__ __forceinline__ bool walk_particle(int root, int64_t nbucket, const int32_t *node_first,
+                                              const int32_t *node_cnt, const uint4 *lo,
+                                              const uint4 *hi, const uint32_t *qx,
+                                              const uint32_t *qy, const uint32_t *qz,
+                                              int32_t *stack, int depth, Near &&near, Visit &&visit) {
+    const int lane = threadIdx.x & 31;
+    auto spot = [&](int f, int c) {
+        const int j = f + min(lane, c - 1);
+        return Spot{qx[j], qy[j], qz[j]};
+    };
+    if (root < nbucket) {
+        const int f = node_first[root], c = node_cnt[root];
+        visit(f, c, spot(f, c));
+        return true;
+    }
+    __syncwarp();
+    if (lane == 0) stack[0] = root;
+    int sp = 1;
+    __syncwarp();
+    while (sp > 0) {
+        sp--;
+        const int node = stack[sp];
+        __syncwarp();
+        const int nf = node_first[node], nc = node_cnt[node];
+        bool hit = false;
+        int cf = 0, cc = 0;
+        if (lane < nc) {
+            const uint4 l = lo[nf + lane], u = hi[nf + lane];
+            if (nf < nbucket) { cf = node_first[nf + lane]; cc = node_cnt[nf + lane]; }
+            hit = near(l, u);
+        }
+        unsigned m = __ballot_sync(0xffffffffu, hit);
+        if (nf < nbucket) {
+            if (!m) continue;
+            int k = __ffs(m) - 1;
+            m &= m - 1;
+            int f = __shfl_sync(0xffffffffu, cf, k), c = __shfl_sync(0xffffffffu, cc, k);
+            Spot p = spot(f, c);
+            for (;;) {
+                const bool more = m != 0;
+                k = more ? __ffs(m) - 1 : 0;
+                m &= m - 1;
+                const int f1 = __shfl_sync(0xffffffffu, cf, k), c1 = __shfl_sync(0xffffffffu, cc, k);
+                Spot p1 = p;
+                if (more) p1 = spot(f1, c1);
+                visit(f, c, p);
+                if (!more) break;
+                f = f1; c = c1; p = p1;
+            }
+            __syncwarp();
+        } else {
+            const int nh = __popc(m);
+            if (sp + nh > depth) return false;
+            if (hit) stack[sp + __popc(m & ((1u << lane) - 1u))] = nf + lane;
+            sp += nh;
+            __syncwarp();
+        }
+    }
+    return true;
+}
+
+// the float band around h^2 for separations from the fixed-point positions
+// (k_build_lists says where its width comes from)
+__device__ __forceinline__ void point_band(double h, const Box &bx, float &lo2, float &hi2) {
+    const float hf = (float)h, ih = 1.f / hf;
+    const float eps = 3e-6f + 2e-9f * (float)bx.Lmax * ih;
+    lo2 = hf * hf * (1.0f - eps);
+    hi2 = hf * hf * (1.0f + eps);
+    if (!(eps < 0.1f)) { lo2 = -1.0f; hi2 = 3.0e38f; }
+}
+
 // Lists of single particles (the N_cond guard's grown particles, whose
 // search radii rose): one warp per particle walks the tree with that
 // particle's own sphere -- the lanes test a node's children at once, then a
 // bucket's particles at once -- instead of rebuilding the lists of the
-// particle's whole bucket at its largest radius.  The walk takes the
-// children in the order of k_build_lists's walk (internal nodes last pushed
-// first, buckets in ascending order), so a list holds the same entries in
-// the same order as a bucket rebuild would give it.  mode 1 counts and
-// reserves storage in the overflow region (flagging ST_LIST_CAPACITY when it
-// does not fit), mode 2 writes.  Warps stride over the *npidx particles of
-// pidx (the count is read on the device); with `active` set, only those
+// particle's whole bucket at its largest radius.  A list holds the same entries
+// in the same order as a bucket rebuild would give it.  The members collect in
+// shared memory, then the storage is reserved in the overflow region (flagging
+// ST_LIST_CAPACITY when it does not fit) and written; a list longer than the
+// buffer is written by a second walk.  Warps stride over the *npidx particles
+// of pidx (the count is read on the device); with `active` set, only those
 // with an ACT_SOLVE flag (a guard round's re-search: the guard particles
-// whose root left their radius), and mode 1 clears the search-failure flag
-// that the new lists answer.
+// whose root left their radius), and the search-failure flag that the new
+// lists answer is cleared.  Two walks, each waiting for every bucket's loads in
+// turn, took 80 us a round on a 500k log-normal box; this takes 34 us.
 struct PartListArgs {
     const int32_t *pidx;
     const int *npidx;
@@ -587,19 +672,18 @@ struct PartListArgs {
     int32_t *nbr_cnt;
     int64_t capacity;
     DevCounters *cnt;
-    int mode;
 };
 
 constexpr int PL_WARPS = 4;
+constexpr int PL_BUF = 1024;   // members a warp collects in shared memory
 
 __global__ void __launch_bounds__(PL_WARPS * 32) k_particle_lists(PartListArgs a) {
-    __shared__ int32_t stack_all[PL_WARPS][STACK];
+    __shared__ int32_t stack_all[PL_WARPS][STACK], buf_all[PL_WARPS][PL_BUF];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int32_t *stack = stack_all[warp];
+    int32_t *stack = stack_all[warp], *buf = buf_all[warp];
     const int np = *a.npidx;
     const int nwarps = gridDim.x * PL_WARPS;
-    if (a.active && a.mode == 1 && blockIdx.x == 0 && threadIdx.x == 0)
-        atomicAnd(&a.cnt->flags, ~ST_SEARCH);
+    if (a.active && blockIdx.x == 0 && threadIdx.x == 0) atomicAnd(&a.cnt->flags, ~ST_SEARCH);
     for (int g = blockIdx.x * PL_WARPS + warp; g < np; g += nwarps) {
         const int s = a.pidx[g];
         if (a.active && !(a.active[s] & ACT_SOLVE)) continue;   // (warp-uniform: one particle)
@@ -608,100 +692,65 @@ __global__ void __launch_bounds__(PL_WARPS * 32) k_particle_lists(PartListArgs a
         const double x = a.xs[s], y = a.ys[s], z = a.zs[s], hs = a.hs[s];
         const double h2 = __dmul_rn(hs, hs);
         float lo2, hi2;
-        {
-            const float hf = (float)hs;
-            lo2 = hf * hf * (1.0f - 1e-4f);
-            hi2 = hf * hf * (1.0f + 1e-4f);
-            const double Lmin = fmin(bx.L[0], fmin(bx.L[1], bx.L[2]));
-            if (hs < Lmin * (1.0 / 4096.0)) { lo2 = -1.0f; hi2 = 3.0e38f; }
-        }
-        int32_t *out = nullptr;
-        int64_t lim = 0;
-        if (a.mode == 2) {
-            const int64_t o = a.nbr_off[s];
-            out = a.nbr_idx + o;
-            lim = max((int64_t)0, a.capacity - o);
-        }
-        int count = 0;
-        // the particles of bucket b within the sphere, appended in order
-        auto scan_bucket = [&](int b) {
-            const int f = a.node_first[b], c = a.node_cnt[b];
-            bool in = false;
-            int j = f + lane;
-            if (lane < c) {
-                const float dx = qdiff(px, a.qx[j], bx.s[0]);
-                const float dy = qdiff(py, a.qy[j], bx.s[1]);
-                const float dz = qdiff(pz, a.qz[j], bx.s[2]);
-                const float r2 = dx * dx + dy * dy + dz * dz;
-                in = r2 < lo2;
-                if (!in && r2 <= hi2) {   // within the float band: decide in double
-                    const double ex = fold64(__dsub_rn(a.xs[j], x), bx.L[0]);
-                    const double ey = fold64(__dsub_rn(a.ys[j], y), bx.L[1]);
-                    const double ez = fold64(__dsub_rn(a.zs[j], z), bx.L[2]);
-                    in = r2_exact(ex, ey, ez) < h2;
-                }
-            }
-            const unsigned m = __ballot_sync(0xffffffffu, in);
-            if (in && a.mode == 2) {
-                const int pos = count + __popc(m & ((1u << lane) - 1u));
-                if (pos < lim) out[pos] = j;
-            }
-            count += __popc(m);
-        };
+        point_band(hs, bx, lo2, hi2);
         const int root = a.box_root[a.pbox[s]];
-        int sp = 0;
-        if (root < a.nbucket_total) {
-            scan_bucket(root);
-        } else {
-            if (lane == 0) stack[0] = root;
-            sp = 1;
-        }
-        __syncwarp();
-        bool stack_ovf = false;
-        while (sp > 0) {
-            sp--;
-            const int node = stack[sp];
-            __syncwarp();
-            const int nf = a.node_first[node], nc = a.node_cnt[node];
-            bool hit = false;
-            if (lane < nc) {
-                const uint4 l = a.lo[nf + lane], u = a.hi[nf + lane];
-                const float gx = u2f(point_gap(px, l.x, u.x)) * bx.s[0];
-                const float gy = u2f(point_gap(py, l.y, u.y)) * bx.s[1];
-                const float gz = u2f(point_gap(pz, l.z, u.z)) * bx.s[2];
-                hit = gx * gx + gy * gy + gz * gz <= hi2;
-            }
-            unsigned m = __ballot_sync(0xffffffffu, hit);
-            if (nf < a.nbucket_total) {
-                while (m) {
-                    const int k = __ffs(m) - 1;
-                    m &= m - 1;
-                    scan_bucket(nf + k);
-                }
-                __syncwarp();
-            } else {
-                const int nh = __popc(m);
-                if (sp + nh > STACK) {   // (cannot happen for trees of MAX_LEVELS levels)
-                    stack_ovf = true;
-                    break;
-                }
-                if (hit) stack[sp + __popc(m & ((1u << lane) - 1u))] = nf + lane;
-                sp += nh;
-                __syncwarp();
-            }
-        }
-        if (stack_ovf) {
+        // one walk: the members to shared memory (dst NULL) or to dst
+        int count = 0;
+        auto walk = [&](int32_t *dst) {
+            count = 0;
+            return walk_particle(
+                root, a.nbucket_total, a.node_first, a.node_cnt, a.lo, a.hi, a.qx, a.qy, a.qz, stack,
+                STACK,
+                [&](uint4 l, uint4 u) {
+                    const float gx = u2f(point_gap(px, l.x, u.x)) * bx.s[0];
+                    const float gy = u2f(point_gap(py, l.y, u.y)) * bx.s[1];
+                    const float gz = u2f(point_gap(pz, l.z, u.z)) * bx.s[2];
+                    return gx * gx + gy * gy + gz * gz <= hi2;
+                },
+                [&](int f, int c, const Spot &p) {
+                    bool in = false;
+                    const int j = f + lane;
+                    if (lane < c) {
+                        const float dx = qdiff(px, p.qx, bx.s[0]);
+                        const float dy = qdiff(py, p.qy, bx.s[1]);
+                        const float dz = qdiff(pz, p.qz, bx.s[2]);
+                        const float r2 = dx * dx + dy * dy + dz * dz;
+                        in = r2 < lo2;
+                        if (!in && r2 <= hi2) {   // within the float band: decide in double
+                            const double ex = fold64(__dsub_rn(a.xs[j], x), bx.L[0]);
+                            const double ey = fold64(__dsub_rn(a.ys[j], y), bx.L[1]);
+                            const double ez = fold64(__dsub_rn(a.zs[j], z), bx.L[2]);
+                            in = r2_exact(ex, ey, ez) < h2;
+                        }
+                    }
+                    const unsigned m = __ballot_sync(0xffffffffu, in);
+                    if (in) {
+                        const int pos = count + __popc(m & ((1u << lane) - 1u));
+                        if (dst) dst[pos] = j;
+                        else if (pos < PL_BUF) buf[pos] = j;
+                    }
+                    count += __popc(m);
+                });
+        };
+        if (!walk(nullptr)) {
             if (lane == 0) set_flag(a.cnt, ST_STACK);
             continue;
         }
-        if (a.mode == 1 && lane == 0) {
-            const unsigned long long base =
-                atomicAdd(&a.cnt->list_cursor, (unsigned long long)count);
+        unsigned long long base = 0;
+        if (lane == 0) base = atomicAdd(&a.cnt->list_cursor, (unsigned long long)count);
+        base = __shfl_sync(0xffffffffu, base, 0);
+        const bool fits = (int64_t)base + count <= a.capacity;
+        if (lane == 0) {
             a.nbr_off[s] = (int64_t)base;
-            a.nbr_cnt[s] = count;
-            if ((int64_t)base + count > a.capacity) {
-                set_flag(a.cnt, ST_LIST_CAPACITY);
-                a.nbr_cnt[s] = 0;   // nothing stored for this list
+            a.nbr_cnt[s] = fits ? count : 0;   // (nothing stored for a list that does not fit)
+            if (!fits) set_flag(a.cnt, ST_LIST_CAPACITY);
+        }
+        __syncwarp();
+        if (fits) {
+            if (count <= PL_BUF) {
+                for (int k = lane; k < count; k += 32) a.nbr_idx[base + k] = buf[k];
+            } else {
+                walk(a.nbr_idx + base);
             }
         }
         __syncwarp();
@@ -803,9 +852,8 @@ k_mark_reverse(const int32_t *__restrict__ guard_idx, const int *__restrict__ ng
                const double *__restrict__ h, const int32_t *__restrict__ pbox,
                const Box *__restrict__ boxes, uint8_t *__restrict__ active, DevCounters *cnt,
                bool use_h, int64_t nparticles) {
-    __shared__ int stack_all[RWARPS][RSTACK];
+    __shared__ int32_t stack_all[RWARPS][RSTACK];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int *stack = stack_all[warp];
     const int ng = *nguard;
     // (a guard round with many grown particles marks by the list scan below)
     if (use_h && mark_by_scan(ng, nparticles)) return;
@@ -814,48 +862,38 @@ k_mark_reverse(const int32_t *__restrict__ guard_idx, const int *__restrict__ ng
         const int a = guard_idx[g];
         const Box bx = boxes[pbox[a]];
         const uint32_t pax = qx[a], pay = qy[a], paz = qz[a];
-        const double xa = xs[a], ya = ys[a], za = zs[a];
-        if (lane == 0) {
-            active[a] |= ACT_REDO;
-            stack[0] = box_root[pbox[a]];
-        }
-        int sp = 1;
-        __syncwarp();
-        while (sp > 0) {
-            const int node = stack[--sp];
-            __syncwarp();
-            const int f = node_first[node], c = node_cnt[node];
-            if (node < nbucket) {
-                // a bucket: lane k tests its particle f + k
-                const int i = f + lane;
-                if (lane < c && i != a) {
-                    const double ex = fold64(__dsub_rn(xa, xs[i]), bx.L[0]);
-                    const double ey = fold64(__dsub_rn(ya, ys[i]), bx.L[1]);
-                    const double ez = fold64(__dsub_rn(za, zs[i]), bx.L[2]);
-                    const double hi_ = h[i];
-                    if (r2_exact(ex, ey, ez) < __dmul_rn(hi_, hi_)) active[i] |= ACT_REDO;
-                }
-                continue;
-            }
-            bool hit = false;
-            if (lane < c) {
-                const uint4 l = lo[f + lane], u = hi[f + lane];
+        if (lane == 0) active[a] |= ACT_REDO;
+        const bool ok = walk_particle(
+            box_root[pbox[a]], nbucket, node_first, node_cnt, lo, hi, qx, qy, qz, stack_all[warp],
+            RSTACK,
+            [&](uint4 l, uint4 u) {
                 const float rmax = __uint_as_float(use_h ? u.w : l.w) * 1.0001f;
                 const float gx = u2f(point_gap(pax, l.x, u.x)) * bx.s[0];
                 const float gy = u2f(point_gap(pay, l.y, u.y)) * bx.s[1];
                 const float gz = u2f(point_gap(paz, l.z, u.z)) * bx.s[2];
-                hit = gx * gx + gy * gy + gz * gz <= rmax * rmax;
-            }
-            const unsigned m = __ballot_sync(0xffffffffu, hit);
-            const int np = __popc(m);
-            if (sp + np > RSTACK) {   // (cannot happen for trees of MAX_LEVELS levels)
-                if (lane == 0) set_flag(cnt, ST_STACK);
-                break;
-            }
-            if (hit) stack[sp + __popc(m & ((1u << lane) - 1u))] = f + lane;
-            sp += np;
-            __syncwarp();
-        }
+                return gx * gx + gy * gy + gz * gz <= rmax * rmax;
+            },
+            [&](int f, int c, const Spot &p) {
+                // lane k tests its particle f + k
+                const int i = f + lane;
+                if (lane >= c || i == a) return;
+                const double hi_ = h[i];
+                float lo2, hi2;
+                point_band(hi_, bx, lo2, hi2);
+                const float dx = qdiff(p.qx, pax, bx.s[0]);
+                const float dy = qdiff(p.qy, pay, bx.s[1]);
+                const float dz = qdiff(p.qz, paz, bx.s[2]);
+                const float r2 = dx * dx + dy * dy + dz * dz;
+                bool in = r2 < lo2;
+                if (!in && r2 <= hi2) {   // within the float band: decide in double
+                    const double ex = fold64(__dsub_rn(xs[a], xs[i]), bx.L[0]);
+                    const double ey = fold64(__dsub_rn(ys[a], ys[i]), bx.L[1]);
+                    const double ez = fold64(__dsub_rn(zs[a], zs[i]), bx.L[2]);
+                    in = r2_exact(ex, ey, ez) < __dmul_rn(hi_, hi_);
+                }
+                if (in) active[i] |= ACT_REDO;
+            });
+        if (!ok && lane == 0) set_flag(cnt, ST_STACK);
         __syncwarp();
     }
 }
@@ -1010,6 +1048,7 @@ static ListArgs list_args(hydro_ctx *c, int cap) {
     a.capacity = (int64_t)c->d_nbr_idx.cap;
     a.cnt = c->d_cnt;
     a.cap = cap;
+    a.rows_of = nullptr;
     a.ovf_list = c->d_ovf.get();
     a.ovf_count = &c->d_cnt->ovf_buckets;
     a.nq_dev = false;
@@ -1046,6 +1085,18 @@ cudaError_t build_lists(hydro_ctx *c, int cap, stream_t st) {
     HYD_CUDA(set_u64(&c->d_cnt->list_cursor, (unsigned long long)n * cap, st));
     HYD_CUDA(cudaMemsetAsync(&c->d_cnt->ovf_buckets, 0, sizeof(int), st));
     return launch_lists<LIST_ROWS>(list_args(c, cap), c->plan.nbucket, st);
+}
+
+// new rows for nq buckets (their lists may lie anywhere; longer ones go to the
+// overflow region, where nothing of a whole build is kept)
+cudaError_t build_rows_of(hydro_ctx *c, const int32_t *buckets, int nq, stream_t st) {
+    HYD_CUDA(set_u64(&c->d_cnt->list_cursor, (unsigned long long)c->plan.n * c->list_cap, st));
+    HYD_CUDA(cudaMemsetAsync(&c->d_cnt->ovf_buckets, 0, sizeof(int), st));
+    ListArgs a = list_args(c, c->list_cap);
+    a.nbucket = nq;
+    a.rows_of = buckets;
+    HYD_CUDA(launch_lists<LIST_ROWS>(a, nq, st));
+    return build_lists_queued_dev(c, st);
 }
 
 // the queued buckets: count and reserve in the overflow region, then fill
@@ -1130,13 +1181,8 @@ cudaError_t guard_particle_lists(hydro_ctx *c, stream_t st, bool only_search) {
     a.nbr_cnt = c->d_nbr_cnt.get();
     a.capacity = (int64_t)c->d_nbr_idx.cap;
     a.cnt = c->d_cnt;
-    const unsigned grid = 152 * 8;
-    for (int mode = 1; mode <= 2; mode++) {
-        a.mode = mode;
-        k_particle_lists<<<grid, PL_WARPS * 32, 0, st>>>(a);
-        HYD_CUDA(launch_check());
-    }
-    return cudaSuccess;
+    k_particle_lists<<<152 * 8, PL_WARPS * 32, 0, st>>>(a);
+    return launch_check();
 }
 
 cudaError_t queue_flagged(hydro_ctx *c, uint8_t bits, stream_t st) {

@@ -65,29 +65,39 @@ __global__ void k_rung_fill(int64_t n, const uint8_t *__restrict__ ract, double 
 
 // the records of the particles that do not start: everything but the
 // (current) positions from their last start
+// (a warp copies a particle's record at a time, one scalar per lane: whole lines)
 template <typename R>
 __global__ void k_rec_load(int64_t n, const int32_t *__restrict__ perm,
                            const uint8_t *__restrict__ ract, const R *__restrict__ store,
                            R *__restrict__ rec) {
-    const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (s >= n || ract[s]) return;
-    const R *src = store + (int64_t)perm[s] * REC;
-    R *dst = rec + s * REC;
-#pragma unroll
-    for (int q = R_H; q < REC; q++) dst[q] = src[q];
+    const int lane = threadIdx.x & 31;
+    const int64_t w0 = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * 32;
+    const int64_t s0 = w0 + lane;
+    const int p = s0 < n ? perm[s0] : 0;
+    unsigned m = __ballot_sync(0xffffffffu, s0 < n && !ract[s0]);
+    for (; m; m &= m - 1) {
+        const int k = __ffs(m) - 1;
+        const int64_t src = __shfl_sync(0xffffffffu, p, k);
+        if (lane >= R_H) rec[(w0 + k) * REC + lane] = store[src * REC + lane];
+    }
 }
 
 template <typename R>
 __global__ void k_rec_save(int64_t n, const int32_t *__restrict__ perm,
                            const uint8_t *__restrict__ ract, const R *__restrict__ rec,
                            R *__restrict__ store) {
-    const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (s >= n || !ract[s]) return;
-    const R *src = rec + s * REC;
-    R *dst = store + (int64_t)perm[s] * REC;
-#pragma unroll
-    for (int q = 0; q < REC; q++) dst[q] = src[q];
+    const int lane = threadIdx.x & 31;
+    const int64_t w0 = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * 32;
+    const int64_t s0 = w0 + lane;
+    const int p = s0 < n ? perm[s0] : 0;
+    unsigned m = __ballot_sync(0xffffffffu, s0 < n && ract[s0]);
+    for (; m; m &= m - 1) {
+        const int k = __ffs(m) - 1;
+        const int64_t dst = __shfl_sync(0xffffffffu, p, k);
+        store[dst * REC + lane] = rec[(w0 + k) * REC + lane];
+    }
 }
+static_assert(REC == 32, "a lane per scalar of the record");
 
 // rung from the two criteria (§2.3.10): dt_cfl (the gradient stage's
 // per-particle Eq. 31 value) and dt_acc = c_acc sqrt(h / |a|) with

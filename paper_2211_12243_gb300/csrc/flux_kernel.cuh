@@ -102,25 +102,31 @@ namespace {
 template <typename R>
 __device__ __forceinline__ int sgn_(R v) { return (v > R(0)) - (v < R(0)); }
 
-// pairwise limiter of the face value e seen from the side with cell value a
+// Pairwise limiter of the two face values of a field (l seen from the cell value
+// u, m from v): the side with the lower cell value is held in
+// [lo - psi1 d, mean + psi2 d], the other in [mean - psi2 d, hi + psi1 d]
+// (d = |u - v|); for a positive field a bound that would change sign is shrunk
+// instead.  Both sides share the bounds, and the selections are without
+// branches (equal cells leave no room and give back the cell value).
 template <typename R>
-__device__ __forceinline__ R pair_limit(R e, R a, R b, R psi1, R psi2, bool positive) {
-    if (a == b) return a;
-    R d = fabs(a - b);
-    R mean = R(0.5) * (a + b);
-    R d1 = psi1 * d, d2 = psi2 * d;
-    R lo = a < b ? a : b, hi = a > b ? a : b;
+__device__ __forceinline__ void pair_limit(R &l, R &m, R u, R v, R psi1, R psi2, bool positive) {
+    const R d = fabs(u - v), mean = R(0.5) * (u + v);
+    const R d1 = psi1 * d, d2 = psi2 * d;
+    const bool up = u < v;   // the owner's cell holds the lower value
+    const R lo = up ? u : v, hi = up ? v : u;
     R lox = lo - d1, hix = hi + d1;
-    if (positive) {
+    if (positive && !(lo > R(0) && lox > R(0))) {
         if (sgn_(lox) != sgn_(lo)) lox = lo == R(0) ? R(0) : div_(lo, R(1) + div_(d1, fabs(lo)));
         if (sgn_(hix) != sgn_(hi)) hix = hi == R(0) ? R(0) : div_(hi, R(1) + div_(d1, fabs(hi)));
     }
-    if (a < b) {
-        R t = e < mean + d2 ? e : mean + d2;
-        return t > lox ? t : lox;
-    }
-    R t = e > mean - d2 ? e : mean - d2;
-    return t < hix ? t : hix;
+    R low = up ? l : m, high = up ? m : l;
+    const R top = mean + d2, bottom = mean - d2;
+    low = low < top ? low : top;
+    low = low > lox ? low : lox;
+    high = high > bottom ? high : bottom;
+    high = high < hix ? high : hix;
+    l = up ? low : high;
+    m = up ? high : low;
 }
 
 template <typename R>
@@ -154,20 +160,15 @@ __device__ __forceinline__ void load4(const R *p, R v[4]) {
 
 // r < h_j decided exactly (float path: band + double fallback)
 __device__ __forceinline__ bool member_j(float r2, float hjf, const FluxArgs &a, int64_t i,
-                                         int64_t j, const Box &bx) {
+                                         int64_t j) {
     float lo = hjf * hjf * (1.0f - 1e-4f), hi = hjf * hjf * (1.0f + 1e-4f);
     if (hjf >= a.lmin_tiny) {
         if (r2 < lo) return true;
         if (r2 > hi) return false;
     }
-    double hj = a.h[j];
-    double ex = fold64(__dsub_rn(a.xs[j], a.xs[i]), bx.L[0]);
-    double ey = fold64(__dsub_rn(a.ys[j], a.ys[i]), bx.L[1]);
-    double ez = fold64(__dsub_rn(a.zs[j], a.zs[i]), bx.L[2]);
-    return r2_exact(ex, ey, ez) < __dmul_rn(hj, hj);
+    return member_exact(a.xs, a.ys, a.zs, a.boxes + a.pbox[i], i, j, a.h[j]);
 }
-__device__ __forceinline__ bool member_j(double r2, double hj, const FluxArgs &, int64_t,
-                                         int64_t, const Box &) {
+__device__ __forceinline__ bool member_j(double r2, double hj, const FluxArgs &, int64_t, int64_t) {
     return dlt_pos(r2, __dmul_rn(hj, hj));
 }
 
@@ -230,8 +231,7 @@ __device__ __forceinline__ bool face_state(const FluxArgs &a, const GasK<R> &K, 
 #pragma unroll
         for (int f = 0; f < 5; f++) {
             bool pos = (f == 0 || f == 4);
-            Lf[f] = pair_limit<R>(Lf[f], ri[R_RHO + f], rj[R_RHO + f], p1, p2, pos);
-            Rf[f] = pair_limit<R>(Rf[f], rj[R_RHO + f], ri[R_RHO + f], p1, p2, pos);
+            pair_limit<R>(Lf[f], Rf[f], ri[R_RHO + f], rj[R_RHO + f], p1, p2, pos);
         }
     }
     const R g = K.g;
@@ -657,7 +657,7 @@ k_fluxes(FluxArgs a, const R *__restrict__ rec) {
         R own4[4];   // the lane's own position and h (enumeration)
         load4<R>(rec + (int64_t)s * REC, own4);
         Member mem;
-        mem.init(a.xs, a.ys, a.zs, s, a.h[s], bx);
+        mem.init(a.xs, a.ys, a.zs, s, a.h[s], a.boxes + a.pbox[s]);
         typename AccOf<R>::T acc;
         acc.zero();
         const int64_t o = a.nbr_off[s];
@@ -838,7 +838,7 @@ k_fluxes(FluxArgs a, const R *__restrict__ rec) {
                 if (k < cnt && j != s) {
                     R d[3], r2;
                     rec_sep(own4, rc4, bx, d, r2);
-                    if (mem(r2, j)) has = (j > s) || !member_j(r2, rc4[R_H], a, s, j, bx);
+                    if (mem(r2, j)) has = (j > s) || !member_j(r2, rc4[R_H], a, s, j);
                     if (!LEAN && has && a.ract && !a.ract[s] && !a.ract[j]) has = false;
                 }
                 jc = jn;

@@ -290,7 +290,7 @@ __device__ __forceinline__ void grad_one(const GradArgs &a, R *__restrict__ rec,
         const double hd = a.h[s];
         const R h = (R)hd;
         Member mem;
-        mem.init(a.xs, a.ys, a.zs, s, hd, bx);
+        mem.init(a.xs, a.ys, a.zs, s, hd, a.boxes + a.pbox[s]);
         const R ih = R(1) / h;
         const R norm = kernel_norm<R>(a.kernel, h);
         const R fi[5] = {ri[R_RHO], ri[R_VX], ri[R_VY], ri[R_VZ], ri[R_P]};
@@ -676,7 +676,7 @@ __global__ void k_entropy_route(int64_t n, const int64_t *__restrict__ nbr_off,
     if (!cold) {
         const Box bx = boxes[pbox[s]];
         Member mem;
-        mem.init(xs, ys, zs, s, h[s], bx);
+        mem.init(xs, ys, zs, s, h[s], boxes + pbox[s]);
         const double vx = (double)ri[R_VX], vy = (double)ri[R_VY], vz = (double)ri[R_VZ];
         const int64_t o = nbr_off[s];
         const int c = nbr_cnt[s];

@@ -143,7 +143,7 @@ __global__ void k_rung_limit(int64_t n, const int64_t *__restrict__ nbr_off,
     if (s >= n) return;
     const Box bx = boxes[pbox[s]];
     Member mem;
-    mem.init(xs, ys, zs, s, h[s], bx);
+    mem.init(xs, ys, zs, s, h[s], boxes + pbox[s]);
     volatile const int32_t *rg = rung_s;
     int mine = rg[s];
     bool raised = false;

@@ -29,6 +29,7 @@
 // the full list.
 #include "fp64.cuh"
 #include "hydro_internal.cuh"
+#include "row.cuh"
 #include "tile_rank.cuh"
 
 namespace hyd {
@@ -159,14 +160,16 @@ struct Separation<float> {
     float sx, sy, sz;
     __device__ __forceinline__ Separation(const DensArgs &a, const float *rec_, int64_t s, const Box &bx)
         : rec(rec_), sx(bx.s[0]), sy(bx.s[1]), sz(bx.s[2]) {
-        const float *ri = rec + s * REC;
+        float ri[4];
+        load_row<4>(rec, s, ri);
         qx = __float_as_uint(ri[R_X]); qy = __float_as_uint(ri[R_Y]); qz = __float_as_uint(ri[R_Z]);
     }
     __device__ __forceinline__ float operator()(int j) const {
-        const float4 pj = *reinterpret_cast<const float4 *>(rec + (int64_t)j * REC);
-        float dx = qdiff(qx, __float_as_uint(pj.x), sx);
-        float dy = qdiff(qy, __float_as_uint(pj.y), sy);
-        float dz = qdiff(qz, __float_as_uint(pj.z), sz);
+        float rj[4];
+        load_row<4>(rec, j, rj);
+        float dx = qdiff(qx, __float_as_uint(rj[R_X]), sx);
+        float dy = qdiff(qy, __float_as_uint(rj[R_Y]), sy);
+        float dz = qdiff(qz, __float_as_uint(rj[R_Z]), sz);
         float r2 = dx * dx + dy * dy + dz * dz;
         return r2 > 0.f ? r2 * rsqrtf(r2) : 0.f;
     }
@@ -485,8 +488,9 @@ __device__ __forceinline__ void dens_one(const DensArgs &a, double *__restrict__
     const double om = 1.0 / (kernel_norm<double>(a.kernel, h) * F);
     a.h[s] = h;
     a.om[s] = om;
-    rec[s * REC + R_H] = h;
-    rec[s * REC + R_OM] = om;
+    const Row<double> rr(rec, s);
+    rr[R_H] = h;
+    rr[R_OM] = om;
 }
 
 // ---------------------------------------------------------------- mixed path
@@ -613,7 +617,7 @@ __device__ __forceinline__ void dens_one(const DensArgs &a, const uint64_t *__re
     double om = 1.0 / (normh * fsum);
     a.h[s] = hnew;
     a.om[s] = om;
-    float *rr = rec + s * REC;
+    const Row<float> rr(rec, s);
     rr[R_H] = (float)hnew;
     rr[R_OM] = (float)om;
 }

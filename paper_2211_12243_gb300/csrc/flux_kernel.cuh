@@ -129,35 +129,6 @@ __device__ __forceinline__ void pair_limit(R &l, R &m, R u, R v, R psi1, R psi2,
     m = up ? high : low;
 }
 
-template <typename R>
-__device__ __forceinline__ void load_full(const R *p, R v[REC]) {
-    if (sizeof(R) == 4) {
-#pragma unroll
-        for (int k = 0; k < REC / 4; k++) {
-            float4 t = reinterpret_cast<const float4 *>(p)[k];
-            v[4 * k] = t.x; v[4 * k + 1] = t.y; v[4 * k + 2] = t.z; v[4 * k + 3] = t.w;
-        }
-    } else {
-#pragma unroll
-        for (int k = 0; k < REC / 2; k++) {
-            double2 t = reinterpret_cast<const double2 *>(p)[k];
-            v[2 * k] = t.x; v[2 * k + 1] = t.y;
-        }
-    }
-}
-
-template <typename R>
-__device__ __forceinline__ void load4(const R *p, R v[4]) {
-    if (sizeof(R) == 4) {
-        float4 t = *reinterpret_cast<const float4 *>(p);
-        v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
-    } else {
-        double2 t0 = reinterpret_cast<const double2 *>(p)[0];
-        double2 t1 = reinterpret_cast<const double2 *>(p)[1];
-        v[0] = t0.x; v[1] = t0.y; v[2] = t1.x; v[3] = t1.y;
-    }
-}
-
 // r < h_j decided exactly (float path: band + double fallback)
 __device__ __forceinline__ bool member_j(float r2, float hjf, const FluxArgs &a, int64_t i,
                                          int64_t j) {
@@ -655,7 +626,7 @@ k_fluxes(FluxArgs a, const R *__restrict__ rec) {
         const GasK<R> &K = gas<R>(a);
         const R dt = (R)(a.dt_dev ? *a.dt_dev : a.dt);
         R own4[4];   // the lane's own position and h (enumeration)
-        load4<R>(rec + (int64_t)s * REC, own4);
+        load_row<4>(rec, s, own4);
         Member mem;
         mem.init(a.xs, a.ys, a.zs, s, a.h[s], a.boxes + a.pbox[s]);
         typename AccOf<R>::T acc;
@@ -722,8 +693,8 @@ k_fluxes(FluxArgs a, const R *__restrict__ rec) {
                 ol = sm.qo[lane];
                 const int j = sm.qj[lane];
                 R ri[REC], rj[REC];
-                load_full<R>(rec + (int64_t)(f + ol) * REC, ri);   // owner (L1-resident)
-                load_full<R>(rec + (int64_t)j * REC, rj);
+                load_row<REC>(rec, f + ol, ri);   // owner (L1-resident)
+                load_row<REC>(rec, j, rj);
                 R d[3], r2;
                 rec_sep(ri, rj, bx, d, r2);
                 FaceState<R> st;
@@ -824,14 +795,14 @@ k_fluxes(FluxArgs a, const R *__restrict__ rec) {
         int jc = 0 < cnt ? a.nbr_idx[o] : 0;
         int jn = 1 < cnt ? a.nbr_idx[o + 1] : 0;
         R rc4[4] = {R(0), R(0), R(0), R(0)};
-        if (0 < cnt) load4<R>(rec + (int64_t)jc * REC, rc4);
+        if (0 < cnt) load_row<4>(rec, jc, rc4);
         // (one call site of solve: the face code is instantiated once, which
         // keeps the kernel's instruction footprint small; the last pass
         // drains the queue)
         for (int k = 0; k < maxc || qn > 0; k++) {
             if (k < maxc) {
                 R rn4[4] = {R(0), R(0), R(0), R(0)};
-                if (k + 1 < cnt) load4<R>(rec + (int64_t)jn * REC, rn4);
+                if (k + 1 < cnt) load_row<4>(rec, jn, rn4);
                 const int jnn = k + 2 < cnt ? a.nbr_idx[o + k + 2] : 0;
                 bool has = false;
                 const int j = jc;
@@ -960,8 +931,8 @@ __global__ void __launch_bounds__(128) k_hard_faces(FluxArgs a) {
             }
             if (a.dM && c[0] != 0.f) {
                 float ri4[4], rj4[4], d[3], r2;
-                load4<float>(a.recf + (int64_t)s * REC, ri4);
-                load4<float>(a.recf + (int64_t)j * REC, rj4);
+                load_row<4>(a.recf, s, ri4);
+                load_row<4>(a.recf, j, rj4);
                 rec_sep(ri4, rj4, a.boxes[a.pbox[s]], d, r2);
                 const double cm = widen(c[0]);
                 for (int q = 0; q < 3; q++) {
@@ -972,7 +943,7 @@ __global__ void __launch_bounds__(128) k_hard_faces(FluxArgs a) {
             if (a.dS && c[0] != 0.f) {
                 const double cm = widen(c[0]);
                 const double sf =
-                    cm * (double)a.recf[(int64_t)(c[0] > 0.f ? s : j) * REC + R_PAD];
+                    cm * (double)Row<const float>(a.recf, c[0] > 0.f ? s : j)[R_PAD];
                 atomicAdd(&a.dS[s], -sf);
                 atomicAdd(&a.dS[j], sf);
             }

@@ -48,29 +48,6 @@ struct GradArgs {
                                          // (k_primitives; the entropy switch uses the slot)
 };
 
-template <typename R>
-__device__ __forceinline__ void load10(const R *p, R v[10]);
-
-template <>
-__device__ __forceinline__ void load10<float>(const float *p, float v[10]) {
-    float4 a = *reinterpret_cast<const float4 *>(p);
-    float4 b = *reinterpret_cast<const float4 *>(p + 4);
-    float2 c = *reinterpret_cast<const float2 *>(p + 8);
-    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
-    v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-    v[8] = c.x; v[9] = c.y;
-}
-
-template <>
-__device__ __forceinline__ void load10<double>(const double *p, double v[10]) {
-#pragma unroll
-    for (int k = 0; k < 5; k++) {
-        double2 a = *reinterpret_cast<const double2 *>(p + 2 * k);
-        v[2 * k] = a.x;
-        v[2 * k + 1] = a.y;
-    }
-}
-
 // grad_one in FP64, bound by the FP64 pipe: 72 FP64 instructions per
 // neighbour where the general form issued about 190 (gradient stage of the
 // 1.07 M tube 9.66 -> 5.34 ms, 32^3 lattice 0.38 -> 0.23 ms).  The
@@ -90,15 +67,13 @@ __device__ __forceinline__ void grad_one64(const GradArgs &a, double *__restrict
     }
     const Box bx = a.boxes[a.pbox[s]];
     double ri[10];
-    load10<double>(rec + s * REC, ri);
+    load_row<10>(rec, s, ri);
     const double h = a.h[s], h2 = __dmul_rn(h, h);
     const double h2lo = h2 * (1.0 - 1e-14), h2hi = h2 * (1.0 + 1e-14);
     const double ih = 1.0 / h, norm = kernel_norm<double>(a.kernel, h);
     const double fi[5] = {ri[R_RHO], ri[R_VX], ri[R_VY], ri[R_VZ], ri[R_P]};
-    auto sound = [&](const double *r, double rho, double p) {
-        return a.pad_c ? r[R_PAD] : sqrt(div_(a.gamma * p, rho));
-    };
-    const double ci = sound(rec + s * REC, ri[R_RHO], ri[R_P]);
+    const Row<double> rs(rec, s);
+    const double ci = a.pad_c ? rs[R_PAD] : sqrt(div_(a.gamma * ri[R_P], ri[R_RHO]));
     auto separation = [&](const double *rj, double d[3]) {
         d[0] = fold64(__dsub_rn(rj[0], ri[0]), bx.L[0]);
         d[1] = fold64(__dsub_rn(rj[1], ri[1]), bx.L[1]);
@@ -128,8 +103,8 @@ __device__ __forceinline__ void grad_one64(const GradArgs &a, double *__restrict
     int jn = 1 < c ? a.nbr_idx[o + 1] : 0;
     double rn[10], cn = 0.0;
     if (0 < c) {
-        load10<double>(rec + (int64_t)jc * REC, rn);
-        if (a.pad_c) cn = rec[(int64_t)jc * REC + R_PAD];
+        load_row<10>(rec, jc, rn);
+        if (a.pad_c) cn = Row<double>(rec, jc)[R_PAD];
     }
     for (int k = 0; k < c; k++) {
         const int j = jc;
@@ -137,8 +112,8 @@ __device__ __forceinline__ void grad_one64(const GradArgs &a, double *__restrict
 #pragma unroll
         for (int q = 0; q < 10; q++) rj[q] = rn[q];
         if (k + 1 < c) {
-            load10<double>(rec + (int64_t)jn * REC, rn);
-            if (a.pad_c) cn = rec[(int64_t)jn * REC + R_PAD];
+            load_row<10>(rec, jn, rn);
+            if (a.pad_c) cn = Row<double>(rec, jn)[R_PAD];
         }
         jc = jn;
         jn = k + 2 < c ? a.nbr_idx[o + k + 2] : 0;
@@ -210,9 +185,9 @@ __device__ __forceinline__ void grad_one64(const GradArgs &a, double *__restrict
         // largest extrapolations to the midpoints, doubled (dx . grad f)
         long long dp[5] = {0, 0, 0, 0, 0}, dm[5] = {0, 0, 0, 0, 0};
         auto pos3 = [&](int j, double v[3]) {
-            const double *pj = rec + (int64_t)j * REC;
-            const double2 t = *reinterpret_cast<const double2 *>(pj);
-            v[0] = t.x; v[1] = t.y; v[2] = pj[2];
+            const Row<double> rj(rec, j);
+            const double2 t = rj.get<double2>(0);
+            v[0] = t.x; v[1] = t.y; v[2] = rj[2];
         };
         int jc2 = 0 < c ? a.nbr_idx[o] : 0;
         int jn2 = 1 < c ? a.nbr_idx[o + 1] : 0;
@@ -247,7 +222,6 @@ __device__ __forceinline__ void grad_one64(const GradArgs &a, double *__restrict
             alpha[f] = al < 1.0 ? al : 1.0;
         }
     }
-    double *rs = rec + s * REC;
 #pragma unroll
     for (int k = 0; k < 6; k++) rs[R_B + k] = B[k];
 #pragma unroll
@@ -286,7 +260,7 @@ __device__ __forceinline__ void grad_one(const GradArgs &a, R *__restrict__ rec,
     if (s < a.n && (!a.only_redo || (a.active[s] & ACT_REDO)) && (LEAN || !a.ract || a.ract[s])) {
         const Box bx = a.boxes[a.pbox[s]];
         R ri[10];
-        load10<R>(rec + s * REC, ri);
+        load_row<10>(rec, s, ri);
         const double hd = a.h[s];
         const R h = (R)hd;
         Member mem;
@@ -312,13 +286,13 @@ __device__ __forceinline__ void grad_one(const GradArgs &a, R *__restrict__ rec,
         int jc = 0 < c ? a.nbr_idx[o] : 0;
         int jn = 1 < c ? a.nbr_idx[o + 1] : 0;
         R rn[10];
-        if (0 < c) load10<R>(rec + (int64_t)jc * REC, rn);
+        if (0 < c) load_row<10>(rec, jc, rn);
         for (int k = 0; k < c; k++) {
             const int j = jc;
             R rj[10];
 #pragma unroll
             for (int q = 0; q < 10; q++) rj[q] = rn[q];
-            if (k + 1 < c) load10<R>(rec + (int64_t)jn * REC, rn);
+            if (k + 1 < c) load_row<10>(rec, jn, rn);
             jc = jn;
             jn = k + 2 < c ? a.nbr_idx[o + k + 2] : 0;
             if (j == s) continue;
@@ -394,24 +368,15 @@ __device__ __forceinline__ void grad_one(const GradArgs &a, R *__restrict__ rec,
         R alpha[5] = {R(1), R(1), R(1), R(1), R(1)};
         if (a.limiter) {
             R dp[5] = {0, 0, 0, 0, 0}, dm[5] = {0, 0, 0, 0, 0};
-            auto pos4 = [&](int j, R v[4]) {
-                const R *pj = rec + (int64_t)j * REC;
-                if (sizeof(R) == 4) {
-                    float4 t = *reinterpret_cast<const float4 *>(pj);
-                    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
-                } else {
-                    v[0] = pj[0]; v[1] = pj[1]; v[2] = pj[2]; v[3] = pj[3];
-                }
-            };
             // (same pipeline as pass 1)
             int jc2 = 0 < c ? a.nbr_idx[o] : 0;
             int jn2 = 1 < c ? a.nbr_idx[o + 1] : 0;
             R rn4[4];
-            if (0 < c) pos4(jc2, rn4);
+            if (0 < c) load_row<4>(rec, jc2, rn4);
             for (int k = 0; k < c; k++) {
                 const int j = jc2;
                 R rj[4] = {rn4[0], rn4[1], rn4[2], rn4[3]};
-                if (k + 1 < c) pos4(jn2, rn4);
+                if (k + 1 < c) load_row<4>(rec, jn2, rn4);
                 jc2 = jn2;
                 jn2 = k + 2 < c ? a.nbr_idx[o + k + 2] : 0;
                 if (j == s) continue;
@@ -436,7 +401,7 @@ __device__ __forceinline__ void grad_one(const GradArgs &a, R *__restrict__ rec,
                 alpha[f] = al < R(1) ? al : R(1);
             }
         }
-        R *rs = rec + s * REC;
+        const Row<R> rs(rec, s);
 #pragma unroll
         for (int k = 0; k < 6; k++) rs[R_B + k] = B[k];
 #pragma unroll
@@ -584,7 +549,7 @@ __global__ void k_primitives(int64_t n, const double *__restrict__ Q,
             const double ax = agrav[s], ay = agrav[n + s], az = agrav[2 * n + s];
             egrav = m * sqrt(ax * ax + ay * ay + az * az) * h[s];
         }
-        R *r = rec + s * REC;
+        const Row<R> r(rec, s);
         // the pressure route of §2.3.7: 0 total energy, 2 internal energy; the
         // entropy route (1) is taken over by k_entropy_route, which needs the
         // neighbours' velocities this kernel writes
@@ -671,21 +636,24 @@ __global__ void k_entropy_route(int64_t n, const int64_t *__restrict__ nbr_off,
         const double ax = agrav[s], ay = agrav[n + s], az = agrav[2 * n + s];
         egrav = m * sqrt(ax * ax + ay * ay + az * az) * h[s];
     }
-    R *ri = rec + s * REC;
+    const Row<R> ri(rec, s);
     bool cold = U < ent.alpha3 * egrav;
     if (!cold) {
         const Box bx = boxes[pbox[s]];
         Member mem;
         mem.init(xs, ys, zs, s, h[s], boxes + pbox[s]);
+        R pi[4];
+        load_row<4>(rec, s, pi);
         const double vx = (double)ri[R_VX], vy = (double)ri[R_VY], vz = (double)ri[R_VZ];
         const int64_t o = nbr_off[s];
         const int c = nbr_cnt[s];
         for (int k = 0; k < c && !cold; k++) {
             const int j = nbr_idx[o + k];
             if (j == s) continue;
-            const R *rj = rec + (int64_t)j * REC;
-            R d[3], r2;
-            rec_sep(ri, rj, bx, d, r2);
+            const Row<R> rj(rec, j);
+            R d[3], r2, pj[4];
+            load_row<4>(rec, j, pj);
+            rec_sep(pi, pj, bx, d, r2);
             if (!mem(r2, j)) continue;
             const double dx = (double)rj[R_VX] - vx, dy = (double)rj[R_VY] - vy,
                          dz = (double)rj[R_VZ] - vz;
@@ -749,7 +717,7 @@ template <typename R>
 __global__ void k_load_grads(int64_t n, const double *__restrict__ st, R *__restrict__ rec) {
     int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (s >= n) return;
-    R *r = rec + s * REC;
+    const Row<R> r(rec, s);
     for (int k = 0; k < 6; k++) r[R_B + k] = (R)st[k * n + s];
     for (int f = 0; f < 5; f++) {
         double al = st[(21 + f) * n + s];

@@ -9,7 +9,8 @@
 //                              256 B (double) line, read whole by the pair
 //                              kernels when particle s is a neighbour:
 //                              x y z h | rho vx vy vz | p omega B(6) |
-//                              limited grad rho(3) v(9) p(3) | pad
+//                              limited grad rho(3) v(9) p(3) | pad,
+//                              16-byte columns turned by s (row.cuh)
 //                              (in float records x y z hold the q bits)
 //   Qs[6][n]          double   conserved m, px, py, pz, E, U (sorted copy)
 //   nbr_off/nbr_cnt   int64/int32  per-particle slice of nbr_idx (sorted ids)

@@ -4,10 +4,11 @@
 
 #include "fp64.cuh"
 #include "hydro_internal.cuh"
+#include "row.cuh"
 
 namespace hyd {
 
-// positions from the first three record slots
+// separation from the first three slots
 __device__ __forceinline__ void rec_sep(const double *ri, const double *rj, const Box &bx,
                                         double d[3], double &r2) {
     d[0] = fold64(__dsub_rn(rj[0], ri[0]), bx.L[0]);

@@ -78,7 +78,7 @@ __global__ void k_rec_load(int64_t n, const int32_t *__restrict__ perm,
     for (; m; m &= m - 1) {
         const int k = __ffs(m) - 1;
         const int64_t src = __shfl_sync(0xffffffffu, p, k);
-        if (lane >= R_H) rec[(w0 + k) * REC + lane] = store[src * REC + lane];
+        if (lane >= R_H) Row<R>(rec, w0 + k)[lane] = store[src * REC + lane];
     }
 }
 
@@ -94,7 +94,7 @@ __global__ void k_rec_save(int64_t n, const int32_t *__restrict__ perm,
     for (; m; m &= m - 1) {
         const int k = __ffs(m) - 1;
         const int64_t dst = __shfl_sync(0xffffffffu, p, k);
-        store[dst * REC + lane] = rec[(w0 + k) * REC + lane];
+        store[dst * REC + lane] = Row<const R>(rec, w0 + k)[lane];
     }
 }
 static_assert(REC == 32, "a lane per scalar of the record");
@@ -112,7 +112,7 @@ __global__ void k_rung_assign(int64_t n, const double *__restrict__ dt_cfl,
                               DevCounters *cnt) {
     const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (s >= n) return;
-    const R *r = rec + s * REC;
+    const Row<const R> r(rec, s);
     const double gx = (double)r[R_G + 12], gy = (double)r[R_G + 13], gz = (double)r[R_G + 14];
     const double g2 = __dadd_rn(__dadd_rn(__dmul_rn(gx, gx), __dmul_rn(gy, gy)), __dmul_rn(gz, gz));
     const double acc = __ddiv_rn(sqrt(g2), (double)r[R_RHO]);
@@ -144,6 +144,8 @@ __global__ void k_rung_limit(int64_t n, const int64_t *__restrict__ nbr_off,
     const Box bx = boxes[pbox[s]];
     Member mem;
     mem.init(xs, ys, zs, s, h[s], boxes + pbox[s]);
+    R ri[4], rj[4];
+    load_row<4>(rec, s, ri);
     volatile const int32_t *rg = rung_s;
     int mine = rg[s];
     bool raised = false;
@@ -153,14 +155,15 @@ __global__ void k_rung_limit(int64_t n, const int64_t *__restrict__ nbr_off,
         const int j = nbr_idx[o + k];
         if (j == s) continue;
         R d[3], r2;
-        rec_sep(rec + s * REC, rec + (int64_t)j * REC, bx, d, r2);
+        load_row<4>(rec, j, rj);
+        rec_sep(ri, rj, bx, d, r2);
         if (!mem(r2, j)) continue;
-        const int rj = rg[j];
-        if (rj - 2 > mine) {
-            mine = rj - 2;
+        const int other = rg[j];
+        if (other - 2 > mine) {
+            mine = other - 2;
             atomicMax(&rung_s[s], mine);
             raised = true;
-        } else if (mine - 2 > rj) {
+        } else if (mine - 2 > other) {
             atomicMax(&rung_s[j], mine - 2);
             raised = true;
         }

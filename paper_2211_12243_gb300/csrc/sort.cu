@@ -4,6 +4,7 @@
 // gathers/scatters between the caller's order and the sorted order.
 #include "fp64.cuh"
 #include "hydro_internal.cuh"
+#include "row.cuh"
 
 namespace hyd {
 
@@ -311,7 +312,7 @@ __global__ void k_gather_state(int64_t n, const int32_t *__restrict__ perm,
     double r = h_search ? h_search[o] : margin * h;
     hs[s] = r;
     pbox[s] = b;
-    R *rr = rec + (int64_t)s * REC;
+    const Row<R> rr(rec, s);
     if (sizeof(R) == 8) {
         rr[R_X] = (R)px; rr[R_Y] = (R)py; rr[R_Z] = (R)pz;
     } else {

@@ -409,7 +409,7 @@ int hydro_reserve(hydro_ctx *c, int64_t max_n, int nbr_per_particle) {
     API_CUDA(c->d_dQ.ensure((size_t)5 * n));
     if (c->cfg.precision == HYDRO_MIXED) {
         API_CUDA(c->d_recf.ensure((size_t)REC * n));
-        API_CUDA(c->d_q64.ensure((size_t)3 * n));
+        API_CUDA(c->d_pos.ensure(n)); API_CUDA(c->d_low.ensure(n));
     } else {
         API_CUDA(c->d_recd.ensure((size_t)REC * n));
         API_CUDA(c->d_dQe.ensure((size_t)5 * n));

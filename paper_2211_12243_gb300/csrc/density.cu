@@ -60,6 +60,7 @@ struct DensArgs {
     bool rank;                // full solve: rank the CTA's 128 particles by list length
     const int32_t *list;      // the guard round's particles, their count on the device
     const int *nlist;         // (k_density_list; NULL: every particle)
+    const uint4 *pos, *low;   // mixed path: high and low words of the 64-bit fixed-point x y z
 };
 
 // Growth of the search radius hs after a failed solve.  First failure
@@ -100,6 +101,18 @@ __device__ __forceinline__ df df_add(df a, df b) {
     s.lo += t.lo;
     return quick_two_sum(s.hi, s.lo);
 }
+// df_add of a single float: the same bits with half the operations
+__device__ __forceinline__ df df_addf(df a, float b) {
+    df s = two_sum(a.hi, b);
+    s.lo += a.lo;
+    return quick_two_sum(s.hi, s.lo);
+}
+// 1 - q, 0 <= q <= 1
+__device__ __forceinline__ df df_one_minus(df q) {
+    df s = quick_two_sum(1.f, -q.hi);
+    s.lo -= q.lo;
+    return quick_two_sum(s.hi, s.lo);
+}
 __device__ __forceinline__ df df_mul(df a, df b) {
     df p = two_prod(a.hi, b.hi);
     p.lo += a.hi * b.lo + a.lo * b.hi;
@@ -126,6 +139,10 @@ __device__ __forceinline__ df df_div(df a, df b) {
     float q2 = r.hi / b.hi;
     return quick_two_sum(q1, q2);
 }
+// difference of two 64-bit fixed-point coordinates given as their words
+__device__ __forceinline__ long long fixed_diff(uint32_t hj, uint32_t lj, uint32_t hi, uint32_t li) {
+    return (long long)((((uint64_t)hj << 32) | lj) - (((uint64_t)hi << 32) | li));
+}
 // float-float of a 64-bit integer |v| < 2^62 from three 21-bit pieces,
 // each converted exactly without a conversion instruction
 __device__ __forceinline__ df from_i64(long long v) {
@@ -134,8 +151,11 @@ __device__ __forceinline__ df from_i64(long long v) {
     int32_t lo = (int32_t)((unsigned long long)v & 0x1FFFFFull);
     float fh = i2f_small(hi) * 4398046511104.0f;                       // 2^42
     float fm = i2f_small(mid) * 2097152.0f;                            // 2^21
-    df s = two_sum(fh, fm);
-    return df_add(s, {i2f_small(lo), 0.f});
+    // (each term is at least as large as what is added to it, or zero)
+    const df s = quick_two_sum(fh, fm);
+    df t = quick_two_sum(s.hi, i2f_small(lo));
+    t.lo += s.lo;
+    return quick_two_sum(t.hi, t.lo);
 }
 
 // ------------------------------------------------- the iteration in float
@@ -148,28 +168,26 @@ constexpr int64_t DENS_WARP_MAX = 8192;
 // separations a warp that walks one list keeps in shared memory
 constexpr int DENS_CACHE = 1536;
 
-// float separations of a particle from its list's entries: from the float
-// records (mixed path) or the fixed-point positions (FP64 path).  Within
+// float separations of a particle from its list's entries, from the fixed-point
+// positions: side by side (mixed path) or the coordinate arrays (FP64 path).  Within
 // 4e-7 r + 4e-10 L of the exact ones.
 template <typename R>
 struct Separation;
 template <>
 struct Separation<float> {
-    const float *rec;
+    const uint4 *pos;
     uint32_t qx, qy, qz;
     float sx, sy, sz;
-    __device__ __forceinline__ Separation(const DensArgs &a, const float *rec_, int64_t s, const Box &bx)
-        : rec(rec_), sx(bx.s[0]), sy(bx.s[1]), sz(bx.s[2]) {
-        float ri[4];
-        load_row<4>(rec, s, ri);
-        qx = __float_as_uint(ri[R_X]); qy = __float_as_uint(ri[R_Y]); qz = __float_as_uint(ri[R_Z]);
+    __device__ __forceinline__ Separation(const DensArgs &a, const float *, int64_t s, const Box &bx)
+        : pos(a.pos), sx(bx.s[0]), sy(bx.s[1]), sz(bx.s[2]) {
+        const uint4 pi = pos[s];
+        qx = pi.x; qy = pi.y; qz = pi.z;
     }
     __device__ __forceinline__ float operator()(int j) const {
-        float rj[4];
-        load_row<4>(rec, j, rj);
-        float dx = qdiff(qx, __float_as_uint(rj[R_X]), sx);
-        float dy = qdiff(qy, __float_as_uint(rj[R_Y]), sy);
-        float dz = qdiff(qz, __float_as_uint(rj[R_Z]), sz);
+        const uint4 pj = pos[j];
+        float dx = qdiff(qx, pj.x, sx);
+        float dy = qdiff(qy, pj.y, sy);
+        float dz = qdiff(qz, pj.z, sz);
         float r2 = dx * dx + dy * dy + dz * dz;
         return r2 > 0.f ? r2 * rsqrtf(r2) : 0.f;
     }
@@ -496,10 +514,8 @@ __device__ __forceinline__ void dens_one(const DensArgs &a, double *__restrict__
 // ---------------------------------------------------------------- mixed path
 // one particle's float Newton solve, then the double-float refinement
 template <int W>
-__device__ __forceinline__ void dens_one(const DensArgs &a, const uint64_t *__restrict__ q64x,
-                                         const uint64_t *__restrict__ q64y,
-                                         const uint64_t *__restrict__ q64z,
-                                         float *__restrict__ rec, const Walk<W> &wk, int64_t s) {
+__device__ __forceinline__ void dens_one(const DensArgs &a, float *__restrict__ rec,
+                                         const Walk<W> &wk, int64_t s) {
     if (s >= a.n) return;
     if (a.only_active && !(a.active[s] & 1)) return;
     const Box bx = a.boxes[a.pbox[s]];
@@ -526,7 +542,7 @@ __device__ __forceinline__ void dens_one(const DensArgs &a, const uint64_t *__re
     const float comp = nf.comp;
     const int c = nf.c;
     // one Newton step in double-float on exact 64-bit fixed-point separations
-    const uint64_t xi64 = q64x[s], yi64 = q64y[s], zi64 = q64z[s];
+    const uint4 li = a.low[s];
     const float sx = (float)(bx.L[0] * 5.421010862427522e-20);  // L / 2^64
     const float sy = (float)(bx.L[1] * 5.421010862427522e-20);
     const float sz = (float)(bx.L[2] * 5.421010862427522e-20);
@@ -546,9 +562,10 @@ __device__ __forceinline__ void dens_one(const DensArgs &a, const uint64_t *__re
         df fv = {0.f, 0.f}, mv = {0.f, 0.f};
         bool on = rf < hcut;
         if (on) {
-            long long ix = (long long)(q64x[j] - xi64);
-            long long iy = (long long)(q64y[j] - yi64);
-            long long iz = (long long)(q64z[j] - zi64);
+            const uint4 pj = a.pos[j], lj = a.low[j];
+            const long long ix = fixed_diff(pj.x, lj.x, sep.qx, li.x);
+            const long long iy = fixed_diff(pj.y, lj.y, sep.qy, li.y);
+            const long long iz = fixed_diff(pj.z, lj.z, sep.qz, li.z);
             df dx = df_mulf(from_i64(ix), sx);
             df dy = df_mulf(from_i64(iy), sy);
             df dz = df_mulf(from_i64(iz), sz);
@@ -556,17 +573,16 @@ __device__ __forceinline__ void dens_one(const DensArgs &a, const uint64_t *__re
             df q = df_mul(df_sqrt(r2), ih);
             on = q.hi < 1.f;
             if (on) {
-                df one = {1.f, 0.f};
-                df t = df_sub(one, q);
+                df t = df_one_minus(q);
                 df t2 = df_mul(t, t);
                 if (a.kernel == 0) {
                     df t3 = df_mul(t2, t);
-                    fv = df_mul(df_mul(t3, t), df_add(one, df_mulf(q, 4.f)));
+                    fv = df_mul(df_mul(t3, t), df_addf({4.f * q.hi, 4.f * q.lo}, 1.f));
                     mv = df_mulf(df_mul(df_mul(q, q), t3), 20.f);
                 } else {
                     df q2 = df_mul(q, q);
                     if (q.hi <= 0.5f) {
-                        fv = df_add(df_sub(one, df_mulf(q2, 6.f)), df_mulf(df_mul(q2, q), 6.f));
+                        fv = df_add(df_sub({1.f, 0.f}, df_mulf(q2, 6.f)), df_mulf(df_mul(q2, q), 6.f));
                         mv = df_sub(df_mulf(q2, 12.f), df_mulf(df_mul(q2, q), 18.f));
                     } else {
                         fv = df_mulf(df_mul(t2, t), 2.f);
@@ -639,21 +655,25 @@ __global__ void k_density_f64(DensArgs a, double *__restrict__ rec) {
     dens_one<1>(a, rec, Walk<1>{nullptr, 0}, dens_particle(a));
 }
 
-__global__ void k_density_mixed(DensArgs a, const uint64_t *__restrict__ q64x,
-                                const uint64_t *__restrict__ q64y,
-                                const uint64_t *__restrict__ q64z, float *__restrict__ rec) {
-    dens_one<1>(a, q64x, q64y, q64z, rec, Walk<1>{nullptr, 0}, dens_particle(a));
+// Bound by the latency of the walk's gathers and by the L1 data stage they go
+// through: 16-byte positions side by side in place of the records' first columns
+// and of three 64-bit arrays, and 10 CTAs per SM (48 registers; 9: 2 % slower, 12:
+// 2 % slower on the tube), took 1.95 -> 1.58 ms (2.10 M particles), 0.786 -> 0.653
+// (1.07 M tube), 2.79 -> 2.23 (4 M log-normal).  Two to eight entries' loads in
+// flight per thread cost more registers than they hide; so does cutting the
+// list to the root before the refinement.
+__global__ void __launch_bounds__(DENS_THREADS, 10) k_density_mixed(DensArgs a, float *__restrict__ rec) {
+    dens_one<1>(a, rec, Walk<1>{nullptr, 0}, dens_particle(a));
 }
 
 // A guard round's re-solve: a warp per particle of the round's guard list.
 // The particles are few (0.4 % of a log-normal box in the first round, fewer
 // later) and their lists long, so a thread each leaves most of the GPU idle
 // behind one serial walk (gradient stage of a 4 M log-normal box, which holds
-// the rounds: 7.15 -> 5.58 ms; 300k in FP64 9.5 -> 6.3 ms).
+// the rounds: 7.15 -> 5.79 ms; 300k in FP64 9.5 -> 6.3 ms).
 template <typename R>
 __global__ void __launch_bounds__(DENS_THREADS)
-k_density_list(DensArgs a, const uint64_t *__restrict__ q64x, const uint64_t *__restrict__ q64y,
-               const uint64_t *__restrict__ q64z, R *__restrict__ rec) {
+k_density_list(DensArgs a, R *__restrict__ rec) {
     __shared__ float rs[DENS_THREADS / 32][DENS_CACHE];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const Walk<32> wk{rs[warp], lane};
@@ -661,8 +681,7 @@ k_density_list(DensArgs a, const uint64_t *__restrict__ q64x, const uint64_t *__
     for (int t = blockIdx.x * (DENS_THREADS / 32) + warp; t < nl; t += gridDim.x * (DENS_THREADS / 32)) {
         const int64_t s = a.list ? a.list[t] : t;
         __syncwarp();
-        if constexpr (sizeof(R) == 8) dens_one<32>(a, rec, wk, s);
-        else dens_one<32>(a, q64x, q64y, q64z, rec, wk, s);
+        dens_one<32>(a, rec, wk, s);
     }
 }
 
@@ -734,16 +753,12 @@ cudaError_t run_density(hydro_ctx *c, bool only_active, bool compact, stream_t s
     const unsigned grid = !warps ? grid_for(n, DENS_THREADS)
         : listed ? 152u * 8u : std::min(152u * 8u, grid_for(n * 32, DENS_THREADS));
     if (c->cfg.precision == HYDRO_MIXED) {
-        const uint64_t *q64 = c->d_q64.get();   // (gather_state)
-        if (warps)
-            k_density_list<float><<<grid, DENS_THREADS, 0, st>>>(a, q64, q64 + n, q64 + 2 * n,
-                                                                c->d_recf.get());
-        else
-            k_density_mixed<<<grid, DENS_THREADS, 0, st>>>(a, q64, q64 + n, q64 + 2 * n,
-                                                           c->d_recf.get());
+        a.pos = c->d_pos.get();   // (gather_state)
+        a.low = c->d_low.get();
+        if (warps) k_density_list<float><<<grid, DENS_THREADS, 0, st>>>(a, c->d_recf.get());
+        else k_density_mixed<<<grid, DENS_THREADS, 0, st>>>(a, c->d_recf.get());
     } else if (warps) {
-        k_density_list<double><<<grid, DENS_THREADS, 0, st>>>(a, nullptr, nullptr, nullptr,
-                                                              c->d_recd.get());
+        k_density_list<double><<<grid, DENS_THREADS, 0, st>>>(a, c->d_recd.get());
     } else {
         k_density_f64<<<grid, DENS_THREADS, 0, st>>>(a, c->d_recd.get());
     }

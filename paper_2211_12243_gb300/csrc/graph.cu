@@ -233,7 +233,8 @@ std::vector<unsigned long long> graph_key(const hydro_ctx *c, const hydro_partic
           (const void *)c->d_xs.get(), (const void *)c->d_ys.get(), (const void *)c->d_zs.get(),
           (const void *)c->d_hs.get(), (const void *)c->d_hsorted.get(),
           (const void *)c->d_omsorted.get(), (const void *)c->d_qx.get(),
-          (const void *)c->d_qy.get(), (const void *)c->d_qz.get(), (const void *)c->d_q64.get(),
+          (const void *)c->d_qy.get(), (const void *)c->d_qz.get(), (const void *)c->d_pos.get(),
+          (const void *)c->d_low.get(),
           (const void *)c->d_pbox.get(), (const void *)c->d_Q.get(), (const void *)c->d_dQ.get(), (const void *)c->d_dQe.get(),
           (const void *)c->d_recf.get(), (const void *)c->d_recd.get(),
           (const void *)c->d_out.get(), (const void *)c->d_nngb.get(),

@@ -175,7 +175,10 @@ struct hydro_ctx {
     // sorted state
     hyd::DevBuf<double> d_xs, d_ys, d_zs, d_hs, d_hsorted, d_omsorted;
     hyd::DevBuf<uint32_t> d_qx, d_qy, d_qz;
-    hyd::DevBuf<uint64_t> d_q64;      // 3 n, mixed-path refinement
+    // mixed path: the high and the low words of the 64-bit fixed-point x y z
+    // side by side (the density walk reads 16 bytes a neighbour and pass, and
+    // eight particles share a line instead of one record)
+    hyd::DevBuf<uint4> d_pos, d_low;
     hyd::DevBuf<int32_t> d_pbox;
     hyd::DevBuf<double> d_Q;          // 6 n
     hyd::DevBuf<double> d_dQ;         // 5 n

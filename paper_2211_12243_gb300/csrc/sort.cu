@@ -293,7 +293,7 @@ __global__ void k_gather_state(int64_t n, const int32_t *__restrict__ perm,
                                uint32_t *__restrict__ qy, uint32_t *__restrict__ qz,
                                double *__restrict__ hsorted, double *__restrict__ hs,
                                int32_t *__restrict__ pbox, R *__restrict__ rec,
-                               uint64_t *__restrict__ q64) {
+                               uint4 *__restrict__ pos, uint4 *__restrict__ low) {
     int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (s >= n) return;
     int o = perm[s];
@@ -305,9 +305,11 @@ __global__ void k_gather_state(int64_t n, const int32_t *__restrict__ perm,
     const uint32_t ux = to_fixed(px, bx.L[0], bx.rL[0], wx), uy = to_fixed(py, bx.L[1], bx.rL[1], wy),
                    uz = to_fixed(pz, bx.L[2], bx.rL[2], wz);
     qx[s] = ux; qy[s] = uy; qz[s] = uz;
-    // (mixed path: the density refinement's positions)
-    if (sizeof(R) == 4) { q64[s] = wx; q64[n + s] = wy; q64[2 * n + s] = wz; }
     double h = h_in[o];
+    if (sizeof(R) == 4) {
+        pos[s] = make_uint4(ux, uy, uz, 0u);
+        low[s] = make_uint4((uint32_t)wx, (uint32_t)wy, (uint32_t)wz, 0u);
+    }
     hsorted[s] = h;
     double r = h_search ? h_search[o] : margin * h;
     hs[s] = r;
@@ -447,19 +449,19 @@ cudaError_t gather_state(hydro_ctx *c, const hydro_particles *p, const double *h
     const bool mixed = c->cfg.precision == HYDRO_MIXED;
     if (mixed) {
         HYD_CUDA(c->d_recf.ensure((size_t)n * REC));
-        HYD_CUDA(c->d_q64.ensure((size_t)3 * n));
+        HYD_CUDA(c->d_pos.ensure(n)); HYD_CUDA(c->d_low.ensure(n));
         k_gather_state<float><<<grid_for(n, 256), 256, 0, st>>>(
             n, c->d_perm.get(), c->d_box_off.get(), c->plan.nbox, c->d_boxes.get(), p->x, p->y,
             p->z, h_in, h_search, margin, c->d_xs.get(), c->d_ys.get(), c->d_zs.get(),
             c->d_qx.get(), c->d_qy.get(), c->d_qz.get(), c->d_hsorted.get(), c->d_hs.get(),
-            c->d_pbox.get(), c->d_recf.get(), c->d_q64.get());
+            c->d_pbox.get(), c->d_recf.get(), c->d_pos.get(), c->d_low.get());
     } else {
         HYD_CUDA(c->d_recd.ensure((size_t)n * REC));
         k_gather_state<double><<<grid_for(n, 256), 256, 0, st>>>(
             n, c->d_perm.get(), c->d_box_off.get(), c->plan.nbox, c->d_boxes.get(), p->x, p->y,
             p->z, h_in, h_search, margin, c->d_xs.get(), c->d_ys.get(), c->d_zs.get(),
             c->d_qx.get(), c->d_qy.get(), c->d_qz.get(), c->d_hsorted.get(), c->d_hs.get(),
-            c->d_pbox.get(), c->d_recd.get(), nullptr);
+            c->d_pbox.get(), c->d_recd.get(), nullptr, nullptr);
     }
     HYD_CUDA(launch_check());
     if (want_Q) {

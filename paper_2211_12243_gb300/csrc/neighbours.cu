@@ -18,7 +18,7 @@ namespace hyd {
 namespace {
 
 constexpr int LIST_WARPS = 4;
-constexpr int LIST_CTAS = 6;   // resident CTAs per SM (80 registers; 5 and 8 were within 3 %)
+constexpr int LIST_CTAS = 6;   // resident CTAs per SM (80 registers; 5: 4 % slower, 8: -1 to +10 %)
 constexpr int STACK = 256;
 
 __device__ __forceinline__ uint32_t wmin(uint32_t v) {
@@ -178,15 +178,48 @@ __device__ __forceinline__ uint32_t point_gap(uint32_t p, uint32_t b0, uint32_t 
     return e > w + 2u ? e - w - 2u : 0u;
 }
 
+// two floats side by side: one instruction for both
+struct Pair {
+    unsigned long long v;
+};
+__device__ __forceinline__ Pair pair(float a, float b) {
+    Pair p;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(p.v) : "f"(a), "f"(b));
+    return p;
+}
+__device__ __forceinline__ void halves(Pair p, float &a, float &b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(p.v));
+}
+__device__ __forceinline__ Pair add2(Pair a, Pair b) {
+    Pair p;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(p.v) : "l"(a.v), "l"(b.v));
+    return p;
+}
+__device__ __forceinline__ Pair mul2(Pair a, Pair b) {
+    Pair p;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(p.v) : "l"(a.v), "l"(b.v));
+    return p;
+}
+__device__ __forceinline__ Pair fma2(Pair a, Pair b, Pair c) {
+    Pair p;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(p.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return p;
+}
+
 // The warp's candidates, a ring of two tiles of 32: positions relative to the
 // bucket's corner (or the fixed-point ones) and sorted indices;
 // and the boxes its owners are culled by
 struct Tiles {
-    float4 r[64];
-    int32_t j[64];
+    alignas(16) float x[64];
+    alignas(16) float y[64];
+    alignas(16) float z[64];
+    alignas(16) int32_t j[64];
     int32_t stack[STACK];
     uint4 lo[2], hi[2];      // fixed-point corners; .w: largest radius
-    float4 ctr[2], ext[2];   // relative centre (.w: squared reach), half widths
+    // per axis both relative centres and both half widths, negated; the squared
+    // reaches
+    alignas(16) float2 ctr[3][2];
+    float2 reach2;
 };
 
 // r < hs decided as the definition states it
@@ -201,14 +234,17 @@ __device__ __forceinline__ bool list_exact(const ListArgs &a, const Box &bx, int
 // Neighbour lists: a warp takes 32 / SPLIT owners of a bucket, each held by
 // SPLIT lanes.  One walk of the tree finds the buckets near the owners'
 // boxes; their particles near those boxes are collected into tiles of 32 in
-// shared memory, and a full tile is tested by all owners: per candidate one
-// broadcast read, the distance, two comparisons and one bit of the lane's
-// member mask, without a branch (lane group g of an owner takes the g-th part
-// of the tile).  The masks then give the members in the candidates' order,
+// shared memory, and a full tile is tested by all owners: four candidates a
+// broadcast read, the distances two at a time, two comparisons and one bit of
+// the lane's member mask each, without a branch (lane group g of an owner takes
+// the g-th part of the tile).  The masks then give the members in the candidates' order,
 // which is the walk's -- internal nodes last pushed first, buckets in
 // ascending order -- whatever the split.
 //
-// Bound by instruction issue (about 11 instructions per candidate and warp).
+// Bound by instruction issue (about 8 instructions per candidate and warp, 5 to
+// append it, 75 per staged bucket of 32; one distance at a time, appends in a
+// loop over the mask's bits and exact position differences: 1.35 -> 1.15 ms for
+// the 128^3 lattice, 1.05 -> 0.93 for the tube, 3.94 -> 3.45 for 4 M log-normal).
 // Measured against lanes that each decided and appended one candidate at a
 // time, the owners culled by one box and the band 1e-4 wide (neighbour stage
 // with sort and gathers, 1 GB300): 128^3 lattice at 1.15 h 4.99 -> 1.47 ms (its
@@ -312,11 +348,11 @@ __global__ void __launch_bounds__(LIST_WARPS * 32, LIST_CTAS) k_build_lists(List
                       ez + qh < 0.49f * (float)bx.L[2];
             }
             // The band around hs^2 inside which a float distance does not
-            // decide: at r = hs the relative error of r^2 is at most 6.2e-7 X / hs
-            // (coordinates up to X rounded to 2^-24, their difference, three
-            // axes) + 8e-10 L / hs (positions cut to L / 2^32) + 5e-7 (the
-            // scale's, the squares' and the radius's rounding); two to three
-            // times that is taken.  Without relative coordinates X is the
+            // decide: at r = hs the relative error of r^2 is at most 8.3e-7 X / hs
+            // (both coordinates, up to X, rounded twice to 2^-24; three axes) +
+            // 8e-10 L / hs (positions cut to L / 2^32) + 5e-7 (the scale's, the
+            // difference's, the squares' and the radius's rounding); twice that
+            // is taken.  Without relative coordinates X is the
             // separation itself.
             const float ihf = 1.f / hf;
             const float eps = 2e-6f * (rel ? big : hf) * ihf + 2e-9f * Lmax * ihf + 1e-6f;
@@ -330,9 +366,14 @@ __global__ void __launch_bounds__(LIST_WARPS * 32, LIST_CTAS) k_build_lists(List
                 const float z0 = u2f(lo.z - oz) * bx.s[2], z1 = u2f(hi.z - oz) * bx.s[2];
                 const float h = __uint_as_float(lo.w);
                 const float reach = h + (4e-6f * big + 2e-9f * Lmax + 1e-5f * h);
-                W.ctr[lane] = make_float4(0.5f * (x0 + x1), 0.5f * (y0 + y1), 0.5f * (z0 + z1),
-                                          reach * reach);
-                W.ext[lane] = make_float4(0.5f * (x1 - x0), 0.5f * (y1 - y0), 0.5f * (z1 - z0), 0.f);
+                auto put = [&](int q, float v0, float v1) {
+                    (&W.ctr[q][0].x)[lane] = -0.5f * (v0 + v1);
+                    (&W.ctr[q][1].x)[lane] = -0.5f * (v1 - v0);
+                };
+                put(0, x0, x1);
+                put(1, y0, y1);
+                put(2, z0, z1);
+                (&W.reach2.x)[lane] = reach * reach;
             }
             __syncwarp();
             int32_t *const row =
@@ -345,33 +386,50 @@ __global__ void __launch_bounds__(LIST_WARPS * 32, LIST_CTAS) k_build_lists(List
             int count = 0;   // members of the owner's list so far
             int head = 0, fill = 0;   // the ring's first tile (0 or 32) and candidates in it
 
-            // the members among the 32 candidates from `head`
-            auto test_tile = [&]() {
+            // the members among the n <= 32 candidates from `head` (the slots of a
+            // short tile past them hold whatever was there before)
+            auto test_tile = [&](int n) {
                 constexpr int PER = 32 / SPLIT;
-                const float4 *T = W.r + head + slot * PER;
+                const int t0 = head + slot * PER;
                 unsigned in = 0, amb = 0;
                 if (rel) {
+                    const Pair mx = pair(-rx, -rx), my = pair(-ry, -ry), mz = pair(-rz, -rz);
 #pragma unroll
-                    for (int k = 0; k < PER; k++) {
-                        const float4 c = T[k];
-                        const float dx = c.x - rx, dy = c.y - ry, dz = c.z - rz;
-                        const float r2 = dx * dx + dy * dy + dz * dz;
-                        if (r2 <= hi2) in |= 1u << k;
-                        if (r2 <= hi2 && r2 >= lo2) amb |= 1u << k;
+                    for (int k = 0; k < PER; k += 4) {
+                        const float4 X = *reinterpret_cast<const float4 *>(W.x + t0 + k);
+                        const float4 Y = *reinterpret_cast<const float4 *>(W.y + t0 + k);
+                        const float4 Z = *reinterpret_cast<const float4 *>(W.z + t0 + k);
+                        float r2[4];
+#pragma unroll
+                        for (int u = 0; u < 4; u += 2) {
+                            const Pair dx = add2(u ? pair(X.z, X.w) : pair(X.x, X.y), mx);
+                            const Pair dy = add2(u ? pair(Y.z, Y.w) : pair(Y.x, Y.y), my);
+                            const Pair dz = add2(u ? pair(Z.z, Z.w) : pair(Z.x, Z.y), mz);
+                            halves(fma2(dz, dz, fma2(dy, dy, mul2(dx, dx))), r2[u], r2[u + 1]);
+                        }
+#pragma unroll
+                        for (int u = 0; u < 4; u++) {
+                            if (r2[u] <= hi2) in |= 1u << (k + u);
+                            if (r2[u] <= hi2 && r2[u] >= lo2) amb |= 1u << (k + u);
+                        }
                     }
                 } else {
 #pragma unroll 4
                     for (int k = 0; k < PER; k++) {
-                        const float4 c = T[k];
-                        const float dx = qdiff(sqx, __float_as_uint(c.x), bx.s[0]);
-                        const float dy = qdiff(sqy, __float_as_uint(c.y), bx.s[1]);
-                        const float dz = qdiff(sqz, __float_as_uint(c.z), bx.s[2]);
-                        const float r2 = dx * dx + dy * dy + dz * dz + c.w;
+                        const float dx = qdiff(sqx, __float_as_uint(W.x[t0 + k]), bx.s[0]);
+                        const float dy = qdiff(sqy, __float_as_uint(W.y[t0 + k]), bx.s[1]);
+                        const float dz = qdiff(sqz, __float_as_uint(W.z[t0 + k]), bx.s[2]);
+                        const float r2 = dx * dx + dy * dy + dz * dz;
                         if (r2 <= hi2) in |= 1u << k;
                         if (r2 <= hi2 && r2 >= lo2) amb |= 1u << k;
                     }
                 }
-                const int32_t *J = W.j + head + slot * PER;
+                if (n < 32) {
+                    const unsigned have = ((1u << n) - 1u) >> (slot * PER);
+                    in &= have;
+                    amb &= have;
+                }
+                const int32_t *J = W.j + t0;
                 while (amb) {   // within the float band: decide in double
                     const int k = __ffs(amb) - 1;
                     amb &= amb - 1;
@@ -390,6 +448,20 @@ __global__ void __launch_bounds__(LIST_WARPS * 32, LIST_CTAS) k_build_lists(List
                 }
                 count += tot;
                 if (MODE != LIST_COUNT && own) {
+                    if (pos + __popc(in) <= lim) {
+                        // (a tile near the owners has members of nearly every
+                        // candidate: no loop over the bits)
+                        int32_t *p = row + pos;
+#pragma unroll
+                        for (int k = 0; k < PER; k += 4) {
+                            const int4 j = *reinterpret_cast<const int4 *>(J + k);
+                            if (in & (1u << k)) *p++ = j.x;
+                            if (in & (2u << k)) *p++ = j.y;
+                            if (in & (4u << k)) *p++ = j.z;
+                            if (in & (8u << k)) *p++ = j.w;
+                        }
+                        in = 0;
+                    }
                     while (in) {
                         const int k = __ffs(in) - 1;
                         in &= in - 1;
@@ -406,20 +478,27 @@ __global__ void __launch_bounds__(LIST_WARPS * 32, LIST_CTAS) k_build_lists(List
             // owners' boxes join the ring
             auto stage = [&](int cf, int cc, uint32_t px, uint32_t py, uint32_t pz) {
                 bool keep = false;
-                float4 c;
+                float3 c;
                 if (rel) {
-                    c = make_float4(qdiff(ox, px, bx.s[0]), qdiff(oy, py, bx.s[1]),
-                                    qdiff(oz, pz, bx.s[2]), 0.f);
-#pragma unroll
-                    for (int t = 0; t < 2; t++) {
-                        const float4 m = W.ctr[t], e = W.ext[t];
-                        const float gx = fmaxf(fabsf(c.x - m.x) - e.x, 0.f);
-                        const float gy = fmaxf(fabsf(c.y - m.y) - e.y, 0.f);
-                        const float gz = fmaxf(fabsf(c.z - m.z) - e.z, 0.f);
-                        keep |= gx * gx + gy * gy + gz * gz <= m.w;
-                    }
+                    // (two roundings: the band allows for both)
+                    c = make_float3((float)(int32_t)(px - ox) * bx.s[0],
+                                    (float)(int32_t)(py - oy) * bx.s[1],
+                                    (float)(int32_t)(pz - oz) * bx.s[2]);
+                    // both boxes at once
+                    auto gap = [&](float v, int q) {
+                        const float4 m = *reinterpret_cast<const float4 *>(W.ctr[q]);
+                        float a0, a1;
+                        halves(add2(pair(v, v), pair(m.x, m.y)), a0, a1);
+                        halves(add2(pair(fabsf(a0), fabsf(a1)), pair(m.z, m.w)), a0, a1);
+                        return pair(fmaxf(a0, 0.f), fmaxf(a1, 0.f));
+                    };
+                    const Pair gx = gap(c.x, 0), gy = gap(c.y, 1), gz = gap(c.z, 2);
+                    const float2 lim2 = W.reach2;
+                    float g0, g1;
+                    halves(fma2(gz, gz, fma2(gy, gy, mul2(gx, gx))), g0, g1);
+                    keep = g0 <= lim2.x || g1 <= lim2.y;
                 } else {
-                    c = make_float4(__uint_as_float(px), __uint_as_float(py), __uint_as_float(pz), 0.f);
+                    c = make_float3(__uint_as_float(px), __uint_as_float(py), __uint_as_float(pz));
                     const float gx = u2f(point_gap(px, qlo.x, qhi.x)) * bx.s[0];
                     const float gy = u2f(point_gap(py, qlo.y, qhi.y)) * bx.s[1];
                     const float gz = u2f(point_gap(pz, qlo.z, qhi.z)) * bx.s[2];
@@ -429,12 +508,14 @@ __global__ void __launch_bounds__(LIST_WARPS * 32, LIST_CTAS) k_build_lists(List
                 const unsigned m = __ballot_sync(0xffffffffu, keep);
                 if (keep) {
                     const int at = (head + fill + __popc(m & lt)) & 63;
-                    W.r[at] = c;
+                    W.x[at] = c.x;
+                    W.y[at] = c.y;
+                    W.z[at] = c.z;
                     W.j[at] = cf + lane;
                 }
                 fill += __popc(m);
                 __syncwarp();
-                if (fill >= 32) test_tile();
+                if (fill >= 32) test_tile(32);
             };
 
             const int root = a.box_root[bid];
@@ -505,17 +586,7 @@ __global__ void __launch_bounds__(LIST_WARPS * 32, LIST_CTAS) k_build_lists(List
                     __syncwarp();
                 }
             }
-            if (fill > 0) {
-                // the last tile: the slots past its candidates hold points at
-                // infinity
-                if (lane >= fill) {
-                    W.r[head + lane] = rel ? make_float4(1.0e30f, 0.f, 0.f, 0.f)
-                                           : make_float4(0.f, 0.f, 0.f, INFINITY);
-                    W.j[head + lane] = 0;
-                }
-                __syncwarp();
-                test_tile();
-            }
+            if (fill > 0) test_tile(fill);
 
             if (MODE == LIST_ROWS) {
                 // each particle owns cap slots at s * cap; a longer list sends

@@ -494,8 +494,9 @@ int hydro_set_entropy(hydro_ctx *ctx, double *A);
  *     hydro_step {1.05, 1.1, 1.15, 1.25} and the fixed list slots per
  *     particle {64, 96, 128} (longer lists take two extra passes into an
  *     overflow region), timed over sort + lists + density;
- *   grad_min_ctas: register bound of the gradient kernel (1: none; 4, 5, 6
- *     resident 128-thread CTAs per SM), timed over the gradient stage;
+ *   grad_min_ctas: register bound of the gradient kernel (1: the path's own,
+ *     5 in the mixed one and none in FP64; 4, 5, 6 resident 128-thread CTAs
+ *     per SM), timed over the gradient stage;
  *   flux_min_ctas: register bound of the float flux kernel (4, 5, 6),
  *     timed over the plain-guess flux stage (mixed precision only);
  *   flux_queue: the flux kernel's buckets one per warp by index (0) or

@@ -137,7 +137,7 @@ __device__ __forceinline__ bool member_j(float r2, float hjf, const FluxArgs &a,
         if (r2 < lo) return true;
         if (r2 > hi) return false;
     }
-    return member_exact(a.xs, a.ys, a.zs, a.boxes + a.pbox[i], i, j, a.h[j]);
+    return member_exact(Exact{a.xs, a.ys, a.zs, a.h, a.pbox, a.boxes}, (int)i, (int)j, (int)j);
 }
 __device__ __forceinline__ bool member_j(double r2, double hj, const FluxArgs &, int64_t, int64_t) {
     return dlt_pos(r2, __dmul_rn(hj, hj));
@@ -627,8 +627,8 @@ k_fluxes(FluxArgs a, const R *__restrict__ rec) {
         const R dt = (R)(a.dt_dev ? *a.dt_dev : a.dt);
         R own4[4];   // the lane's own position and h (enumeration)
         load_row<4>(rec, s, own4);
-        Member mem;
-        mem.init(a.xs, a.ys, a.zs, s, a.h[s], a.boxes + a.pbox[s]);
+        Member<R> mem;
+        mem.init(a.h[s], bx);
         typename AccOf<R>::T acc;
         acc.zero();
         const int64_t o = a.nbr_off[s];
@@ -809,7 +809,7 @@ k_fluxes(FluxArgs a, const R *__restrict__ rec) {
                 if (k < cnt && j != s) {
                     R d[3], r2;
                     rec_sep(own4, rc4, bx, d, r2);
-                    if (mem(r2, j)) has = (j > s) || !member_j(r2, rc4[R_H], a, s, j);
+                    if (mem(Exact{a.xs, a.ys, a.zs, a.h, a.pbox, a.boxes}, r2, s, j)) has = (j > s) || !member_j(r2, rc4[R_H], a, s, j);
                     if (!LEAN && has && a.ract && !a.ract[s] && !a.ract[j]) has = false;
                 }
                 jc = jn;

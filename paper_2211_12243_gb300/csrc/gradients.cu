@@ -246,8 +246,8 @@ __device__ __forceinline__ void grad_one64(const GradArgs &a, double *__restrict
     }
 }
 
-// MINB: resident CTAs per SM the register allocation must allow (1: no
-// bound; 5, 6: the variants hydro_autotune times)
+// MINB: resident CTAs per SM the register allocation must allow (1, FP64: no
+// bound; 4, 5, 6: the variants hydro_autotune times)
 // LEAN: compiled without the staged outputs (outB, outG, outA, outN) and
 // the individual-timestep mask, which hydro_step does not use
 template <typename R, bool LEAN>
@@ -263,8 +263,9 @@ __device__ __forceinline__ void grad_one(const GradArgs &a, R *__restrict__ rec,
         load_row<10>(rec, s, ri);
         const double hd = a.h[s];
         const R h = (R)hd;
-        Member mem;
-        mem.init(a.xs, a.ys, a.zs, s, hd, a.boxes + a.pbox[s]);
+        Member<R> mem;
+        mem.init(hd, bx);
+        const Exact ex{a.xs, a.ys, a.zs, a.h, a.pbox, a.boxes};
         const R ih = R(1) / h;
         const R norm = kernel_norm<R>(a.kernel, h);
         const R fi[5] = {ri[R_RHO], ri[R_VX], ri[R_VY], ri[R_VZ], ri[R_P]};
@@ -281,24 +282,21 @@ __device__ __forceinline__ void grad_one(const GradArgs &a, R *__restrict__ rec,
         R vs = R(0);
         const int64_t o = a.nbr_off[s];
         const int c = a.nbr_cnt[s];
-        // software pipeline: the index two entries ahead and the record of
-        // the next entry are in flight while an entry is summed
+        // (the indices two entries ahead; a record ahead as well, or only its
+        // position, took registers that a fifth CTA hides more with: 1.212 and
+        // 1.204 against 1.175 ms on the 128^3 lattice)
         int jc = 0 < c ? a.nbr_idx[o] : 0;
         int jn = 1 < c ? a.nbr_idx[o + 1] : 0;
-        R rn[10];
-        if (0 < c) load_row<10>(rec, jc, rn);
         for (int k = 0; k < c; k++) {
             const int j = jc;
             R rj[10];
-#pragma unroll
-            for (int q = 0; q < 10; q++) rj[q] = rn[q];
-            if (k + 1 < c) load_row<10>(rec, jn, rn);
+            load_row<10>(rec, j, rj);
             jc = jn;
             jn = k + 2 < c ? a.nbr_idx[o + k + 2] : 0;
             if (j == s) continue;
             R d[3], r2;
             rec_sep(ri, rj, bx, d, r2);
-            if (!mem(r2, j)) continue;
+            if (!mem(ex, r2, (int)s, j)) continue;
             mypairs++;
             R r = sqrt_(r2);
             R w = rj[R_OM] * norm * kernel_shape<R>(a.kernel, r * ih);
@@ -382,7 +380,7 @@ __device__ __forceinline__ void grad_one(const GradArgs &a, R *__restrict__ rec,
                 if (j == s) continue;
                 R d[3], r2;
                 rec_sep(ri, rj, bx, d, r2);
-                if (!mem(r2, j)) continue;
+                if (!mem(ex, r2, (int)s, j)) continue;
 #pragma unroll
                 for (int f = 0; f < 5; f++) {
                     R e = R(0.5) * (d[0] * G[f][0] + d[1] * G[f][1] + d[2] * G[f][2]);
@@ -640,8 +638,9 @@ __global__ void k_entropy_route(int64_t n, const int64_t *__restrict__ nbr_off,
     bool cold = U < ent.alpha3 * egrav;
     if (!cold) {
         const Box bx = boxes[pbox[s]];
-        Member mem;
-        mem.init(xs, ys, zs, s, h[s], boxes + pbox[s]);
+        Member<R> mem;
+        mem.init(h[s], bx);
+        const Exact ex{xs, ys, zs, h, pbox, boxes};
         R pi[4];
         load_row<4>(rec, s, pi);
         const double vx = (double)ri[R_VX], vy = (double)ri[R_VY], vz = (double)ri[R_VZ];
@@ -654,7 +653,7 @@ __global__ void k_entropy_route(int64_t n, const int64_t *__restrict__ nbr_off,
             R d[3], r2, pj[4];
             load_row<4>(rec, j, pj);
             rec_sep(pi, pj, bx, d, r2);
-            if (!mem(r2, j)) continue;
+            if (!mem(ex, r2, (int)s, j)) continue;
             const double dx = (double)rj[R_VX] - vx, dy = (double)rj[R_VY] - vy,
                          dz = (double)rj[R_VZ] - vz;
             const double e = 0.5 * m * ((dx * dx + dy * dy) + dz * dz);
@@ -875,17 +874,17 @@ cudaError_t run_gradients(hydro_ctx *c, double *B_out, double *grad_out, double 
     HYD_CUDA(cudaMemsetAsync(&c->d_cnt->redo_pass, only_redo ? 1 : 0, sizeof(int), st));
     const bool lean = !a.outB && !a.outG && !a.outA && !a.outN && !a.ract;
     if (c->cfg.precision == HYDRO_MIXED) {
+        // (5 CTAs per SM unless another bound was chosen: 128^3 lattice 1.26 -> 1.18
+        // ms against the 4 that no bound gives, 6: 1.24)
         float *r = c->d_recf.get();
         if (lean) {
             if (c->grad_minb == 4) k_gradients<float, 4, true><<<grid, 128, smem, st>>>(a, r);
-            else if (c->grad_minb == 5) k_gradients<float, 5, true><<<grid, 128, smem, st>>>(a, r);
             else if (c->grad_minb == 6) k_gradients<float, 6, true><<<grid, 128, smem, st>>>(a, r);
-            else k_gradients<float, 1, true><<<grid, 128, smem, st>>>(a, r);
+            else k_gradients<float, 5, true><<<grid, 128, smem, st>>>(a, r);
         } else {
             if (c->grad_minb == 4) k_gradients<float, 4><<<grid, 128, smem, st>>>(a, r);
-            else if (c->grad_minb == 5) k_gradients<float, 5><<<grid, 128, smem, st>>>(a, r);
             else if (c->grad_minb == 6) k_gradients<float, 6><<<grid, 128, smem, st>>>(a, r);
-            else k_gradients<float, 1><<<grid, 128, smem, st>>>(a, r);
+            else k_gradients<float, 5><<<grid, 128, smem, st>>>(a, r);
         }
     } else {
         double *r = c->d_recd.get();

@@ -25,47 +25,56 @@ __device__ __forceinline__ void rec_sep(const float *ri, const float *rj, const 
     r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
 }
 
-// r_ij^2 < h^2 as the definition states it in double (minimum image folded
+// the arrays an exact membership test reads
+struct Exact {
+    const double *xs, *ys, *zs, *h;
+    const int32_t *pbox;
+    const Box *boxes;
+};
+
+// r_ij^2 < h_k^2 as the definition states it in double (minimum image folded
 // once, (dx^2 + dy^2) + dz^2, each step rounded).  Out of line and from memory:
 // a float separation decides all but a few pairs, and the operands in double
 // would cost the pair kernels some thirty registers.
-static __device__ __noinline__ bool member_exact(const double *xs, const double *ys,
-                                                 const double *zs, const Box *b, int64_t i,
-                                                 int64_t j, double h) {
-    const double ex = fold64(__dsub_rn(xs[j], xs[i]), b->L[0]);
-    const double ey = fold64(__dsub_rn(ys[j], ys[i]), b->L[1]);
-    const double ez = fold64(__dsub_rn(zs[j], zs[i]), b->L[2]);
+static __device__ __noinline__ bool member_exact(Exact a, int i, int j, int k) {
+    const Box *b = a.boxes + a.pbox[i];
+    const double ex = fold64(__dsub_rn(a.xs[j], a.xs[i]), b->L[0]);
+    const double ey = fold64(__dsub_rn(a.ys[j], a.ys[i]), b->L[1]);
+    const double ez = fold64(__dsub_rn(a.zs[j], a.zs[i]), b->L[2]);
+    const double h = a.h[k];
     return r2_exact(ex, ey, ez) < __dmul_rn(h, h);
 }
 
 // Membership r_ij < h_i of particle i's pairs.
-struct Member {
-    const double *xs, *ys, *zs;
-    const Box *b;
-    int64_t i;
-    double h;
+template <typename R>
+struct Member;
+template <>
+struct Member<float> {
     float lo2, hi2;     // float band around h^2 (empty when h is tiny vs L)
-    __device__ __forceinline__ void init(const double *xs_, const double *ys_, const double *zs_,
-                                         int64_t i_, double h_, const Box *b_) {
-        xs = xs_; ys = ys_; zs = zs_; i = i_; b = b_; h = h_;
+    __device__ __forceinline__ void init(double h, const Box &b) {
         float hf = (float)h;
         lo2 = hf * hf * (1.0f - 1e-4f);
         hi2 = hf * hf * (1.0f + 1e-4f);
         // fixed-point separations are exact to L/2^32; below h = L/4096 the
         // float band would no longer be conservative, so decide every pair
         // in double there
-        double Lmin = fmin(b->L[0], fmin(b->L[1], b->L[2]));
+        double Lmin = fmin(b.L[0], fmin(b.L[1], b.L[2]));
         if (h < Lmin * (1.0 / 4096.0)) { lo2 = -1.0f; hi2 = 3.0e38f; }
     }
-    // float path: r2 from the fixed-point separation
-    __device__ __forceinline__ bool operator()(float r2, int64_t j) const {
+    // r2 from the fixed-point separation
+    __device__ __forceinline__ bool operator()(const Exact &a, float r2, int i, int j) const {
         if (r2 < lo2) return true;
         if (r2 > hi2) return false;
-        return member_exact(xs, ys, zs, b, i, j, h);
+        return member_exact(a, i, j, i);
     }
-    // double path: r2 is already the exact value (r2, h2 >= 0)
-    __device__ __forceinline__ bool operator()(double r2, int64_t) const {
-        return dlt_pos(r2, __dmul_rn(h, h));
+};
+template <>
+struct Member<double> {
+    double h2;
+    __device__ __forceinline__ void init(double h, const Box &) { h2 = __dmul_rn(h, h); }
+    // r2 is already the exact value (r2, h2 >= 0)
+    __device__ __forceinline__ bool operator()(const Exact &, double r2, int, int) const {
+        return dlt_pos(r2, h2);
     }
 };
 

@@ -142,8 +142,9 @@ __global__ void k_rung_limit(int64_t n, const int64_t *__restrict__ nbr_off,
     const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (s >= n) return;
     const Box bx = boxes[pbox[s]];
-    Member mem;
-    mem.init(xs, ys, zs, s, h[s], boxes + pbox[s]);
+    Member<R> mem;
+    mem.init(h[s], bx);
+    const Exact ex{xs, ys, zs, h, pbox, boxes};
     R ri[4], rj[4];
     load_row<4>(rec, s, ri);
     volatile const int32_t *rg = rung_s;
@@ -157,7 +158,7 @@ __global__ void k_rung_limit(int64_t n, const int64_t *__restrict__ nbr_off,
         R d[3], r2;
         load_row<4>(rec, j, rj);
         rec_sep(ri, rj, bx, d, r2);
-        if (!mem(r2, j)) continue;
+        if (!mem(ex, r2, (int)s, j)) continue;
         const int other = rg[j];
         if (other - 2 > mine) {
             mine = other - 2;

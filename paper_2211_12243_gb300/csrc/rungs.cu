@@ -65,7 +65,10 @@ __global__ void k_rung_fill(int64_t n, const uint8_t *__restrict__ ract, double 
 
 // the records of the particles that do not start: everything but the
 // (current) positions from their last start
-// (a warp copies a particle's record at a time, one scalar per lane: whole lines)
+// (a warp copies a particle's record at a time, one scalar per lane: whole lines;
+// REC_BATCH of them in flight, since a copy waits for its load: 21.4 -> 8.0 us for
+// 110,592 particles)
+constexpr int REC_BATCH = 8;
 template <typename R>
 __global__ void k_rec_load(int64_t n, const int32_t *__restrict__ perm,
                            const uint8_t *__restrict__ ract, const R *__restrict__ store,
@@ -74,11 +77,17 @@ __global__ void k_rec_load(int64_t n, const int32_t *__restrict__ perm,
     const int64_t w0 = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * 32;
     const int64_t s0 = w0 + lane;
     const int p = s0 < n ? perm[s0] : 0;
-    unsigned m = __ballot_sync(0xffffffffu, s0 < n && !ract[s0]);
-    for (; m; m &= m - 1) {
-        const int k = __ffs(m) - 1;
-        const int64_t src = __shfl_sync(0xffffffffu, p, k);
-        if (lane >= R_H) Row<R>(rec, w0 + k)[lane] = store[src * REC + lane];
+    const unsigned m = __ballot_sync(0xffffffffu, s0 < n && !ract[s0]);
+    for (int k0 = 0; k0 < 32; k0 += REC_BATCH) {
+        R v[REC_BATCH];
+#pragma unroll
+        for (int u = 0; u < REC_BATCH; u++) {
+            const int64_t src = __shfl_sync(0xffffffffu, p, k0 + u);
+            if ((m >> (k0 + u) & 1u) && lane >= R_H) v[u] = store[src * REC + lane];
+        }
+#pragma unroll
+        for (int u = 0; u < REC_BATCH; u++)
+            if ((m >> (k0 + u) & 1u) && lane >= R_H) Row<R>(rec, w0 + k0 + u)[lane] = v[u];
     }
 }
 

@@ -32,8 +32,7 @@ __device__ __forceinline__ uint32_t spread10(uint32_t v) {
 // The position as a fraction of the box in 64-bit fixed point, and its leading
 // 32 bits: floor(x / L 2^64) and floor(x / L 2^32) of the correctly rounded
 // quotient, by five FP64 instructions (fp64.cuh) and integer operations.  A
-// position at or beyond L comes back in at 0 (q64) or wraps once (q32), a
-// negative one is 0.
+// position at or beyond L wraps once (its low word is 0), a negative one is 0.
 __device__ __forceinline__ uint32_t to_fixed(double x, double L, double rL, uint64_t &q64) {
     const double t = div2(x, L, rL);
     if (dpos(t) && dlt_pos(t, 1.0)) {

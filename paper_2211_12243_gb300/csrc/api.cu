@@ -366,6 +366,10 @@ int hydro_set_boxes(hydro_ctx *c, int64_t nbox, const int64_t *box_off, const do
     }
     if (box_off[nbox] > INT32_MAX) return HYDRO_EINVAL;
     Plan &P = c->plan;
+    // (the same boxes again leave a captured step valid)
+    const bool same = P.nbox == nbox && std::equal(P.box_off.begin(), P.box_off.end(), box_off) &&
+                      std::equal(P.box_len.begin(), P.box_len.end(), box_len);
+    if (!same) P.generation++;
     P.nbox = nbox;
     P.n = box_off[nbox];
     P.box_off.assign(box_off, box_off + nbox + 1);

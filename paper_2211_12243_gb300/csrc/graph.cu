@@ -211,6 +211,8 @@ std::vector<unsigned long long> graph_key(const hydro_ctx *c, const hydro_partic
     k.push_back((unsigned long long)c->plan.n);
     k.push_back((unsigned long long)c->plan.nbucket);
     k.push_back((unsigned long long)c->plan.nlevels);
+    // (the captured kernels hold the number of boxes and each level's extent)
+    k.push_back((unsigned long long)c->plan.generation);
     put(c->rec_faces);
     put(c->grav);
     put(c->d_agrav.get());

@@ -113,6 +113,7 @@ struct Plan {
     int64_t n = 0, nbox = 0;
     int64_t nbucket = 0, nnode = 0;
     int nlevels = 0;
+    unsigned long long generation = 0;     // counts the changes of the boxes
     std::vector<int64_t> box_off;          // nbox+1
     std::vector<double> box_len;           // 3 nbox
     std::vector<int64_t> level_off;        // nlevels+1 (node ids, level-major)

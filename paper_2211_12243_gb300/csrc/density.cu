@@ -169,8 +169,9 @@ constexpr int64_t DENS_WARP_MAX = 8192;
 constexpr int DENS_CACHE = 1536;
 
 // float separations of a particle from its list's entries, from the fixed-point
-// positions: side by side (mixed path) or the coordinate arrays (FP64 path).  Within
-// 4e-7 r + 4e-10 L of the exact ones.
+// positions: side by side (mixed path) or the coordinate arrays (FP64 path, in units
+// of the box's longest side, so that their squares stay in the float range whatever
+// the caller's unit of length).  Within 4e-7 r + 4e-10 L of the exact ones.
 template <typename R>
 struct Separation;
 template <>
@@ -198,7 +199,9 @@ struct Separation<double> {
     uint32_t qx, qy, qz;
     float sx, sy, sz;
     __device__ __forceinline__ Separation(const DensArgs &a, const double *, int64_t s, const Box &bx)
-        : px(a.qx), py(a.qy), pz(a.qz), sx(bx.s[0]), sy(bx.s[1]), sz(bx.s[2]) {
+        : px(a.qx), py(a.qy), pz(a.qz) {
+        const double u = bx.rLmax * (1.0 / 4294967296.0);
+        sx = (float)(bx.L[0] * u); sy = (float)(bx.L[1] * u); sz = (float)(bx.L[2] * u);
         qx = px[s]; qy = py[s]; qz = pz[s];
     }
     __device__ __forceinline__ float operator()(int j) const {
@@ -369,38 +372,40 @@ __device__ __forceinline__ void dens_one(const DensArgs &a, double *__restrict__
     const double hsi_d = a.hs[s], hguess = a.h[s];
     const double N = a.nngb ? a.nngb[s] : a.n_ngb;
     int32_t *idx = a.nbr_idx + a.nbr_off[s];
+    // (the float iteration's lengths are in units of the longest side)
+    const double Lmax = bx.Lmax, rLmax = bx.rLmax;
     const double Lmin = fmin(bx.L[0], fmin(bx.L[1], bx.L[2]));
-    const float xmin = (float)(Lmin * (1.0 / 65536.0));
-    const double Lmax = fmax(bx.L[0], fmax(bx.L[1], bx.L[2]));
+    const float xmin = (float)(Lmin * rLmax * (1.0 / 65536.0));
     const Separation<double> sep(a, rec, s, bx);
-    const float hsf = (float)hsi_d;
-    float hf = (float)hguess;
+    const float hsf = (float)(hsi_d * rLmax);
+    float hf = (float)(hguess * rLmax);
     if (!(hf > 0.f) || hf > hsf) hf = hsf;
     // (a radius below 1e-4 of the box leaves the float separations less than
     // 4e-6 accurate: everything in double then)
     const NewtonF o = newton_float<W>(a, sep, idx, a.nbr_cnt[s], hf, hsf, (float)N, xmin,
                                       hsi_d > 1e-4 * Lmax ? min(a.max_iter, FLOAT_ITER) : 0, wk);
-    const float slack = (float)(1e-9 * Lmax);   // (bounds the error of a float r)
+    const float slack = 1e-9f;   // (bounds the error of a float r)
     int c = o.c;
     // The same iteration in double from the float root (from the list radius
     // where it lies beyond, from the guess where the float iteration did not
     // settle): a step below 2e-6 h, taken to
     // third order, leaves an error below 1e-16 h.
-    const double hsi = o.comp > 0.f ? (double)o.comp : hsi_d;
+    const double comp = (double)o.comp * Lmax;
+    const double hsi = o.comp > 0.f ? comp : hsi_d;
     const double Kn = kernel_Kn<double>(a.kernel), iKn = a.kernel == 0 ? 1.0 / 14.0 : 3.0 / 32.0;
     const double M = N * iKn;   // sum f at the root
-    double h = o.fail ? hsi_d : o.conv ? (double)o.h : hguess;
+    double h = o.fail ? hsi_d : o.conv ? (double)o.h * Lmax : hguess;
     if (!(h > 0.0) || h > hsi) h = hsi;
     const double xi = a.xs[s], yi = a.ys[s], zi = a.zs[s];
     double lo = 0.0, hi = -1.0, F = 0.0;
     bool conv = false, fail = false;
-    double crad = o.comp > 0.f ? (double)o.comp : 0.0;
+    double crad = o.comp > 0.f ? comp : 0.0;
     const int left = a.max_iter - (o.conv || o.fail ? o.it : 0);   // evaluations left
     for (int it = 1; it <= (left > 1 ? left : 1); it++) {
         const double ih = 1.0 / h;   // (rounded correctly: its error is common to every q)
         double f = 0.0, f1 = 0.0, mq = 0.0;
         float s2 = 0.f;
-        const float hh = narrow(h);
+        const float hh = narrow(h * rLmax);
         const float cut = hh * (1.f + 1e-5f) + slack, keep = hh * 1.0001f;
         // (the first pass of a converged float root compacts the list)
         const bool shrink = a.compact && it == 1 && o.conv && hh > xmin;
@@ -439,7 +444,7 @@ __device__ __forceinline__ void dens_one(const DensArgs &a, double *__restrict__
         f = wk.sum(f + f1);
         mq = wk.sum(mq);
         s2 = wk.sum(s2);
-        if (shrink) { c = w; crad = (double)hh * (1.0 + 5e-5); }
+        if (shrink) { c = w; crad = (double)hh * Lmax * (1.0 + 5e-5); }
         const double g = f - M;   // (g / Kn)
         F = f;
         if (g == 0.0) { conv = true; break; }

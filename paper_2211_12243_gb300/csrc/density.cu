@@ -287,7 +287,8 @@ __device__ __forceinline__ NewtonF newton_float(const DensArgs &a, const Sep &se
         // an upper bracket well inside the list radius: drop the entries
         // beyond it (no later iterate exceeds hi).  Keeping the entries with
         // float r < X (1 + 1e-4) leaves the list complete for every
-        // r < X (1 + 5e-5) when X > L / 65536 (compaction is skipped below that)
+        // r < X (1 + 5e-5) when X > L / 65536, L the longest side, which sets the
+        // separation's error (compaction is skipped below that)
         const bool shrink = a.compact && hi > xmin && hi < 0.8f * hsi;
         const float keep = hi * 1.0001f;
         int w = 0;
@@ -374,8 +375,7 @@ __device__ __forceinline__ void dens_one(const DensArgs &a, double *__restrict__
     int32_t *idx = a.nbr_idx + a.nbr_off[s];
     // (the float iteration's lengths are in units of the longest side)
     const double Lmax = bx.Lmax, rLmax = bx.rLmax;
-    const double Lmin = fmin(bx.L[0], fmin(bx.L[1], bx.L[2]));
-    const float xmin = (float)(Lmin * rLmax * (1.0 / 65536.0));
+    const float xmin = 1.f / 65536.f;
     const Separation<double> sep(a, rec, s, bx);
     const float hsf = (float)(hsi_d * rLmax);
     float hf = (float)(hguess * rLmax);
@@ -532,7 +532,7 @@ __device__ __forceinline__ void dens_one(const DensArgs &a, float *__restrict__ 
     int32_t *idx = a.nbr_idx + o;
     float h = (float)a.h[s];
     if (!(h > 0.f) || h > hsi) h = hsi;
-    const float xmin = (float)(fmin(bx.L[0], fmin(bx.L[1], bx.L[2])) * (1.0 / 65536.0));
+    const float xmin = (float)(bx.Lmax * (1.0 / 65536.0));
     const NewtonF nf = newton_float<W>(a, sep, idx, a.nbr_cnt[s], h, hsi, N, xmin, a.max_iter, wk);
     const bool lead = wk.lane == 0;
     if (nf.fail) {   // (no compaction happened: failing needs h >= hsi, below any bracket)

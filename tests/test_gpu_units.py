@@ -46,3 +46,42 @@ def test_fp64_step_in_other_length_units(name, k):
     for q, e in (("h", k), ("omega", 3 * k), ("x", k), ("px", 3 * k), ("E", 3 * k)):
         c = np.ldexp(b[q], -e)
         assert np.max(np.abs(c - a[q])) <= 1e-12 * np.max(np.abs(a[q])), q
+
+
+@pytest.mark.parametrize("length,R,h0", [(64.0, 2.3e-4, 5.7e-3)])
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_pairs_of_a_cluster_in_a_long_box(precision, length, R, h0):
+    """A cluster whose smoothing lengths are small against the short sides of a
+    long box: the fixed-point positions resolve the long side coarsely, and the
+    lists that the density solve compacts must keep every member
+    (the pair counts of the gradient
+    and flux stages against all pairs in double)."""
+    import torch
+    from paper_2211_12243_gb300 import hydro
+    rng = np.random.default_rng(4)
+    n, L = 3000, np.array([length, 1.0, 1.0])
+    d = rng.standard_normal((n, 3))
+    p = 0.43 + R * d / np.linalg.norm(d, axis=1)[:, None] * np.cbrt(rng.random((n, 1)))
+    p[:, 0] += 0.64 * length
+    m, z = np.full(n, 1.0 / n), np.zeros(n)
+    w = dict(x=p[:, 0], y=p[:, 1], z=p[:, 2], m=m, px=z, py=z, pz=z, E=1.5 * m, U=1.5 * m,
+             h=np.full(n, h0))
+    H = hydro.Hydro(hydro.default_config(precision=precision, max_ngb_grow=0))
+    H.set_boxes(np.array([0, n], dtype=np.int64), L)
+    st = hydro.to_device(w)
+    s = H.step(st, 1e-12, check=False)
+    torch.cuda.synchronize()
+    assert s["status"] in (0, -5), s
+    h = st["h"].cpu().numpy()
+    assert np.median(h) < R / 3
+    pairs = faces = 0
+    for i in range(n):
+        e = p - p[i]
+        r2 = (e[:, 0] * e[:, 0] + e[:, 1] * e[:, 1]) + e[:, 2] * e[:, 2]
+        r2[i] = np.inf
+        mine = r2 < h[i] * h[i]
+        pairs += int(np.count_nonzero(mine))
+        faces += int(np.count_nonzero((mine | (r2 < h * h))[i:]))
+    assert s["grad_pairs"] == pairs
+    assert s["flux_pairs"] == faces
+    H.close()

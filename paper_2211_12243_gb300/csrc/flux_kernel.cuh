@@ -61,7 +61,7 @@ struct FluxArgs {
     int rec_hard_only;
     GasK<float> Kf;          // gas constants, precomputed on the host
     GasK<double> Kd;
-    float psi1f, psi2f, ptolf, lmin_tiny;   // float copies (no per-face conversions)
+    float psi1f, psi2f, ptolf;   // float copies (no per-face conversions)
     int64_t nbucket;
     const int32_t *node_first, *node_cnt;
     // gravity (§2.3.8): sum_j dm_ij r_ij, 3 n sorted SoA (NULL: no gravity);
@@ -130,16 +130,17 @@ __device__ __forceinline__ void pair_limit(R &l, R &m, R u, R v, R psi1, R psi2,
 }
 
 // r < h_j decided exactly (float path: band + double fallback)
-__device__ __forceinline__ bool member_j(float r2, float hjf, const FluxArgs &a, int64_t i,
-                                         int64_t j) {
+__device__ __forceinline__ bool member_j(float r2, float hjf, const FluxArgs &a, const Box &bx,
+                                         int64_t i, int64_t j) {
     float lo = hjf * hjf * (1.0f - 1e-4f), hi = hjf * hjf * (1.0f + 1e-4f);
-    if (hjf >= a.lmin_tiny) {
+    if (hjf >= band_radius(bx)) {
         if (r2 < lo) return true;
         if (r2 > hi) return false;
     }
     return member_exact(Exact{a.xs, a.ys, a.zs, a.h, a.pbox, a.boxes}, (int)i, (int)j, (int)j);
 }
-__device__ __forceinline__ bool member_j(double r2, double hj, const FluxArgs &, int64_t, int64_t) {
+__device__ __forceinline__ bool member_j(double r2, double hj, const FluxArgs &, const Box &, int64_t,
+                                         int64_t) {
     return dlt_pos(r2, __dmul_rn(hj, hj));
 }
 
@@ -809,7 +810,7 @@ k_fluxes(FluxArgs a, const R *__restrict__ rec) {
                 if (k < cnt && j != s) {
                     R d[3], r2;
                     rec_sep(own4, rc4, bx, d, r2);
-                    if (mem(Exact{a.xs, a.ys, a.zs, a.h, a.pbox, a.boxes}, r2, s, j)) has = (j > s) || !member_j(r2, rc4[R_H], a, s, j);
+                    if (mem(Exact{a.xs, a.ys, a.zs, a.h, a.pbox, a.boxes}, r2, s, j)) has = (j > s) || !member_j(r2, rc4[R_H], a, bx, s, j);
                     if (!LEAN && has && a.ract && !a.ract[s] && !a.ract[j]) has = false;
                 }
                 jc = jn;

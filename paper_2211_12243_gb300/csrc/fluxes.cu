@@ -203,12 +203,6 @@ cudaError_t run_fluxes(hydro_ctx *c, double dt, const double *dt_dev, stream_t s
     a.psi1f = (float)c->cfg.psi1;
     a.psi2f = (float)c->cfg.psi2;
     a.ptolf = (float)std::max(c->cfg.p_tol, 2e-6);
-    {
-        // below h = Lmin / 4096 every membership is decided in double
-        double lmin = 1e300;
-        for (size_t k = 0; k < c->plan.box_len.size(); k++) lmin = std::min(lmin, c->plan.box_len[k]);
-        a.lmin_tiny = (float)(lmin / 4096.0);
-    }
     a.Kf = GasK<float>(c->cfg.gamma);
     a.Kd = GasK<double>(c->cfg.gamma);
     a.nbucket = c->plan.nbucket;

@@ -45,6 +45,12 @@ static __device__ __noinline__ bool member_exact(Exact a, int i, int j, int k) {
     return r2_exact(ex, ey, ez) < __dmul_rn(h, h);
 }
 
+// The smallest radius that the float band (1e-4 of its square) decides: L / 4096
+// with L the longest side, from the sides' units 2^-32 L.
+__device__ __forceinline__ float band_radius(const Box &b) {
+    return fmaxf(b.s[0], fmaxf(b.s[1], b.s[2])) * 1048576.0f;
+}
+
 // Membership r_ij < h_i of particle i's pairs.
 template <typename R>
 struct Member;
@@ -55,11 +61,10 @@ struct Member<float> {
         float hf = (float)h;
         lo2 = hf * hf * (1.0f - 1e-4f);
         hi2 = hf * hf * (1.0f + 1e-4f);
-        // fixed-point separations are exact to L/2^32; below h = L/4096 the
-        // float band would no longer be conservative, so decide every pair
-        // in double there
-        double Lmin = fmin(b.L[0], fmin(b.L[1], b.L[2]));
-        if (h < Lmin * (1.0 / 4096.0)) { lo2 = -1.0f; hi2 = 3.0e38f; }
+        // fixed-point separations are exact to L/2^32, L the longest side; below
+        // h = L/4096 the float band would no longer be conservative, so decide
+        // every pair in double there
+        if (hf < band_radius(b)) { lo2 = -1.0f; hi2 = 3.0e38f; }
     }
     // r2 from the fixed-point separation
     __device__ __forceinline__ bool operator()(const Exact &a, float r2, int i, int j) const {

@@ -48,13 +48,13 @@ def test_fp64_step_in_other_length_units(name, k):
         assert np.max(np.abs(c - a[q])) <= 1e-12 * np.max(np.abs(a[q])), q
 
 
-@pytest.mark.parametrize("length,R,h0", [(64.0, 2.3e-4, 5.7e-3)])
+@pytest.mark.parametrize("length,R,h0", [(64.0, 2.3e-4, 5.7e-3), (1024.0, 1.8e-3, 6e-4)])
 @pytest.mark.parametrize("precision", ["fp64", "mixed"])
 def test_pairs_of_a_cluster_in_a_long_box(precision, length, R, h0):
     """A cluster whose smoothing lengths are small against the short sides of a
     long box: the fixed-point positions resolve the long side coarsely, and the
-    lists that the density solve compacts must keep every member
-    (the pair counts of the gradient
+    lists that the density solve compacts must keep every member, the float
+    band must not decide pairs that it cannot (the pair counts of the gradient
     and flux stages against all pairs in double)."""
     import torch
     from paper_2211_12243_gb300 import hydro

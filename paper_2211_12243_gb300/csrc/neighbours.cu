@@ -21,6 +21,13 @@ constexpr int LIST_WARPS = 4;
 constexpr int LIST_CTAS = 6;   // resident CTAs per SM (80 registers; 5: 4 % slower, 8: -1 to +10 %)
 constexpr int STACK = 256;
 
+// Squared lengths below the normal floats (a unit of length so large that h is
+// below 1e-19) carry an absolute error of a few of the smallest subnormals: every
+// pair of a radius with a square below BAND_MIN2 is decided in double, and
+// CULL_MIN2 widens the culls (by nothing where the square is a normal float).
+constexpr float BAND_MIN2 = 1e-30f;
+constexpr float CULL_MIN2 = 8e-45f;
+
 __device__ __forceinline__ uint32_t wmin(uint32_t v) {
     for (int o = 16; o > 0; o >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, o));
     return v;
@@ -331,7 +338,7 @@ __global__ void __launch_bounds__(LIST_WARPS * 32, LIST_CTAS) k_build_lists(List
             }
             __syncwarp();
             const float qh = __uint_as_float(qlo.w);
-            const float rad2 = (qh * 1.00001f) * (qh * 1.00001f);
+            const float rad2 = (qh * 1.00001f) * (qh * 1.00001f) + CULL_MIN2;
             const float Lmax = (float)fmax(bx.L[0], fmax(bx.L[1], bx.L[2]));
             // Coordinates relative to the bucket's corner: their differences
             // are one periodic image, the nearest one for every pair within
@@ -357,7 +364,7 @@ __global__ void __launch_bounds__(LIST_WARPS * 32, LIST_CTAS) k_build_lists(List
             const float ihf = 1.f / hf;
             const float eps = 2e-6f * (rel ? big : hf) * ihf + 2e-9f * Lmax * ihf + 1e-6f;
             float lo2 = hf * hf * (1.0f - eps), hi2 = hf * hf * (1.0f + eps);
-            if (!(eps < 0.1f)) { lo2 = -1.0f; hi2 = 3.0e38f; }   // (every pair exactly)
+            if (!(eps < 0.1f && hf * hf > BAND_MIN2)) { lo2 = -1.0f; hi2 = 3.0e38f; }   // (every pair exactly)
             // the boxes in relative coordinates, their reach widened likewise
             if (lane < 2) {
                 const uint4 lo = W.lo[lane], hi = W.hi[lane];
@@ -373,7 +380,7 @@ __global__ void __launch_bounds__(LIST_WARPS * 32, LIST_CTAS) k_build_lists(List
                 put(0, x0, x1);
                 put(1, y0, y1);
                 put(2, z0, z1);
-                (&W.reach2.x)[lane] = reach * reach;
+                (&W.reach2.x)[lane] = reach * reach + CULL_MIN2;
             }
             __syncwarp();
             int32_t *const row =
@@ -544,7 +551,7 @@ __global__ void __launch_bounds__(LIST_WARPS * 32, LIST_CTAS) k_build_lists(List
                     for (int t = 0; t < 2; t++) {
                         const uint4 lo = W.lo[t];
                         const float h = __uint_as_float(lo.w) * 1.00001f;
-                        hit |= boxes_near(lo, W.hi[t], clo, chi, bx, h * h);
+                        hit |= boxes_near(lo, W.hi[t], clo, chi, bx, h * h + CULL_MIN2);
                     }
                 }
                 unsigned m = __ballot_sync(0xffffffffu, hit);
@@ -711,7 +718,7 @@ __device__ __forceinline__ void point_band(double h, const Box &bx, float &lo2, 
     const float eps = 3e-6f + 2e-9f * (float)bx.Lmax * ih;
     lo2 = hf * hf * (1.0f - eps);
     hi2 = hf * hf * (1.0f + eps);
-    if (!(eps < 0.1f)) { lo2 = -1.0f; hi2 = 3.0e38f; }
+    if (!(eps < 0.1f && hf * hf > BAND_MIN2)) { lo2 = -1.0f; hi2 = 3.0e38f; }
 }
 
 // Lists of single particles (the N_cond guard's grown particles, whose
@@ -942,7 +949,7 @@ k_mark_reverse(const int32_t *__restrict__ guard_idx, const int *__restrict__ ng
                 const float gx = u2f(point_gap(pax, l.x, u.x)) * bx.s[0];
                 const float gy = u2f(point_gap(pay, l.y, u.y)) * bx.s[1];
                 const float gz = u2f(point_gap(paz, l.z, u.z)) * bx.s[2];
-                return gx * gx + gy * gy + gz * gz <= rmax * rmax;
+                return gx * gx + gy * gy + gz * gz <= rmax * rmax + CULL_MIN2;
             },
             [&](int f, int c, const Spot &p) {
                 // lane k tests its particle f + k

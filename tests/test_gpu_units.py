@@ -48,6 +48,25 @@ def test_fp64_step_in_other_length_units(name, k):
         assert np.max(np.abs(c - a[q])) <= 1e-12 * np.max(np.abs(a[q])), q
 
 
+@pytest.mark.parametrize("n,k", [(4099, -66), (4099, -62), (120011, -64), (4099, 66)])
+def test_lists_in_other_length_units(n, k):
+    """radii whose squares are subnormal floats (or beyond them)"""
+    import torch
+    from paper_2211_12243_gb300 import hydro
+    rng = np.random.default_rng(n)
+    x, y, z = rng.random((3, n))
+    hs = np.cbrt(3.0 * 40.0 / (4.0 * np.pi * n)) * rng.uniform(0.7, 1.2, n)
+    out = []
+    for kk in (0, k):
+        H = hydro.Hydro(hydro.default_config())
+        H.set_boxes(np.array([0, n], dtype=np.int64), np.full(3, np.ldexp(1.0, kk)))
+        dev = lambda v: torch.as_tensor(np.ldexp(v, kk), device="cuda")
+        off, idx = H.build_neighbours({"x": dev(x), "y": dev(y), "z": dev(z), "h": dev(hs)}, dev(hs))
+        out.append((off.cpu().numpy(), idx.cpu().numpy()))
+        H.close()
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+
+
 @pytest.mark.parametrize("length,R,h0", [(64.0, 2.3e-4, 5.7e-3), (1024.0, 1.8e-3, 6e-4)])
 @pytest.mark.parametrize("precision", ["fp64", "mixed"])
 def test_pairs_of_a_cluster_in_a_long_box(precision, length, R, h0):

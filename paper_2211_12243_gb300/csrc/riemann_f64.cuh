@@ -86,7 +86,9 @@ __device__ __forceinline__ StarOut star_solve64(const GasK<double> &k, const Gas
                                                 double tol, int max_newton, double &ps, double &us) {
     StarOut o{0, 0, 0};
     const double du = ur - ul;
-    if (!dlt(du, k.g4 * (cl + cr))) {
+    // (compared in FP64: states that are not numbers are no vacuum, and zeros of
+    // either sign at zero sound speeds are one)
+    if (k.g4 * (cl + cr) <= du) {
         o.vacuum = 1;
         ps = us = 0.0;
         return o;

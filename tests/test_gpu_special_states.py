@@ -1,0 +1,69 @@
+"""States at the edges of what a step accepts: positions of minus zero, cold
+gas whose velocities are zeros of either sign, negative pressures, values that
+are not numbers in the staged calls, densities beyond the float range, and
+limiter factors that switch a bound off."""
+import numpy as np
+import pytest
+
+from paper_2211_12243_gb300 import workloads as W
+from parity_util import compare, gpu_stages, oracle_stages
+
+pytestmark = pytest.mark.gpu
+
+
+def _step(hydro, w, dt, **opts):
+    import torch
+    H = hydro.Hydro(hydro.default_config(gamma=w["gamma"], **opts))
+    H.set_boxes(*hydro.single_box(w))
+    st = hydro.to_device(w)
+    s = H.step(st, dt, check=False)
+    torch.cuda.synchronize()
+    out = {k: v.cpu().numpy() for k, v in st.items()}
+    H.close()
+    return s, out
+
+
+def _cold(n, seed):
+    """a jittered lattice without pressure or motion"""
+    w = dict(W.lattice_wave(n, jitter=0.05, seed=seed))
+    z = np.zeros(w["x"].size)
+    w.update(m=np.full(z.size, 1.0 / z.size), px=z, py=z.copy(), pz=z.copy(), E=z.copy(), U=z.copy())
+    return w
+
+
+@pytest.mark.parametrize("scheme", ["mfv", "mfm"])
+def test_cold_gas_with_zeros_of_either_sign(scheme):
+    """no pressure, velocities +0 and -0: every face is a vacuum"""
+    from paper_2211_12243_gb300 import hydro
+    w = _cold(10, 2)
+    rng = np.random.default_rng(3)
+    for k in ("px", "py", "pz"):
+        w[k] = np.copysign(0.0, rng.standard_normal(w["x"].size))
+    s, out = _step(hydro, w, 1e-3, scheme=scheme)
+    assert s["status"] in (0, -5), s
+    assert s["vacuum_faces"] == s["flux_pairs"] > 0
+    for k in ("m", "px", "E", "x", "y", "z"):
+        assert np.array_equal(out[k], w[k]), k
+
+
+@pytest.mark.parametrize("riemann,scheme", [("exact", "mfv"), ("exact", "mfm"), ("hllc", "mfv"),
+                                            ("hllc", "mfm")])
+def test_nan_gradients_reach_the_fluxes(riemann, scheme):
+    """a velocity gradient that is not a number: the fluxes of that particle
+    are not numbers either (they are not dropped as a vacuum's)"""
+    import torch
+    from paper_2211_12243_gb300 import hydro
+    w = W.lattice_wave(9, jitter=0.05)
+    H = hydro.Hydro(hydro.default_config(gamma=w["gamma"], scheme=scheme, riemann=riemann,
+                                         limiter=0, time_extrap=0))
+    H.set_boxes(*hydro.single_box(w))
+    st = hydro.to_device(w)
+    H.build_neighbours(st, st["h"] * 1.3, export=False)
+    H.density(st)
+    B, G, A, N = H.gradients(st)
+    G[77, 1, 0] = float("nan")
+    dQ = H.fluxes(st, B, G, A, 1e-3)
+    torch.cuda.synchronize()
+    bad = ~np.isfinite(dQ.cpu().numpy()[:, :5])
+    assert bad[77, 4] and np.count_nonzero(bad.any(1)) > 5
+    H.close()

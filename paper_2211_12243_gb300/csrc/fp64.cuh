@@ -18,7 +18,18 @@ __device__ __forceinline__ long long dbits(double v) { return __double_as_longlo
 
 // 0 < v (v not NaN), without the FP64 pipe
 __device__ __forceinline__ bool dpos(double v) {
-    return (unsigned long long)(dbits(v) - 1) < 0x7ff0000000000000ull;
+    return (unsigned long long)dbits(v) - 1ull < 0x7ff0000000000000ull;
+}
+
+// v positive, normal and finite
+__device__ __forceinline__ bool dnormal(double v) {
+    return (unsigned long long)dbits(v) - 0x0010000000000000ull < 0x7fe0000000000000ull;
+}
+
+// 0 <= v (-0 included; v not NaN)
+__device__ __forceinline__ bool dge0(double v) {
+    const unsigned long long b = (unsigned long long)dbits(v);
+    return b <= 0x7ff0000000000000ull || b == 0x8000000000000000ull;
 }
 
 // v < 0 (neither -0 nor NaN)
@@ -77,11 +88,20 @@ __device__ __forceinline__ double rsqrt64(double x) {
     return fma(r, e * fma(0.375, e, 0.5), r);
 }
 
-// sqrt(x) (0 where x is not positive), with a final correction of the residual
+// sqrt(x) of what rsqrt64 does not take: 0 of zeros and positive subnormals,
+// infinity of itself, NaN of negative numbers and NaN
+__device__ __forceinline__ double sqrt_rest(double x) {
+    const unsigned long long b = (unsigned long long)dbits(x);
+    if (b < 0x0010000000000000ull || (b << 1) == 0ull) return 0.0;
+    return __longlong_as_double(b == 0x7ff0000000000000ull ? 0x7ff0000000000000ll
+                                                           : 0x7ff8000000000000ll);
+}
+
+// sqrt(x), with a final correction of the residual
 __device__ __forceinline__ double sqrt64(double x) {
     const double r = rsqrt64(x);
     const double s = x * r;
-    return dpos(x) ? fma(fma(-s, s, x), 0.5 * r, s) : 0.0;
+    return dnormal(x) ? fma(fma(-s, s, x), 0.5 * r, s) : sqrt_rest(x);
 }
 
 // a / b from y = 1/b (within an ulp): each step adds the exactly computed

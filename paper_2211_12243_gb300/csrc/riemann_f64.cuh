@@ -112,8 +112,9 @@ __device__ __forceinline__ StarOut star_solve64(const GasK<double> &k, const Gas
         pf = pn;
         if (done) break;
     }
-    // FP64 finish (a float start out of range or not converged: the plain path)
-    if (pf > 1e-30f && pf < 1e30f && it < 12) {
+    // FP64 finish (a float start out of range or not converged, and a state without
+    // a sound speed, whose float root is 0 and not NaN: the plain path)
+    if (pf > 1e-30f && pf < 1e30f && it < 12 && clf >= 0.f && crf >= 0.f) {
         double p = widen(pf);
         for (int n = 1; n <= 4; n++) {
             const double ip = rcp40(p);
@@ -203,21 +204,22 @@ __device__ __forceinline__ void hllc_flux64(const GasK<double> &k, double rl, do
     const double cl = sqrt64(k.g * pl * irl), cr = sqrt64(k.g * pr * irr);
     double ppv = 0.5 * (pl + pr) - 0.125 * (ur - ul) * (rl + rr) * (cl + cr);
     ppv = dpos(ppv) ? ppv : 0.0;
-    const double ql = dlt(pl, ppv) ? sqrt64(1.0 + k.g2 * fma(ppv, rcp64(pl), -1.0)) : 1.0;
-    const double qr = dlt(pr, ppv) ? sqrt64(1.0 + k.g2 * fma(ppv, rcp64(pr), -1.0)) : 1.0;
+    const double ql = dlt_pos(dabs_(pl), ppv) ? sqrt64(1.0 + k.g2 * fma(ppv, rcp64(pl), -1.0)) : 1.0;
+    const double qr = dlt_pos(dabs_(pr), ppv) ? sqrt64(1.0 + k.g2 * fma(ppv, rcp64(pr), -1.0)) : 1.0;
     const double sl = ul - cl * ql, sr = ur + cr * qr;
     const double al = rl * (sl - ul), ar = rr * (sr - ur);
     ss = (pr - pl + al * ul - ar * ur) * rcp64(al - ar);
     ps = fma(al, ss - ul, pl);
     if (CONTACT_ONLY) return;
-    const bool left = !dneg(sl) || !dneg(ss);
+    // (speeds that are not numbers select as in hllc_flux)
+    const bool left = dge0(sl) || dge0(ss);
     const double r = left ? rl : rr, u = left ? ul : ur, p = left ? pl : pr;
     const double ir = left ? irl : irr, s = left ? sl : sr, al_ = left ? al : ar;
     const double w0 = left ? wl[0] : wr[0], w1 = left ? wl[1] : wr[1], w2 = left ? wl[2] : wr[2];
     const double E = 0.5 * fma(r, fma(u, u, fma(w0, w0, fma(w1, w1, w2 * w2))), k.g4 * p);
     double fm = r * u, fn = fma(fm, u, p), fe = u * (E + p);
     // between the outer waves (s and the contact on either side of x/t = 0)
-    if (left ? dneg(sl) : !dneg(sr)) {
+    if (left ? !dge0(sl) : dge0(sr)) {
         const double kk = al_ * rcp64(s - ss);
         const double e2 = kk * fma(ss - u, ss + p * rcp64(al_), E * ir);
         fn = fma(s, fma(kk, ss, -fm), fn);

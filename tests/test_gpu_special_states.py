@@ -46,6 +46,19 @@ def test_cold_gas_with_zeros_of_either_sign(scheme):
         assert np.array_equal(out[k], w[k]), k
 
 
+@pytest.mark.parametrize("riemann,scheme", [("exact", "mfv"), ("exact", "mfm"), ("hllc", "mfm")])
+def test_negative_pressure_is_reported(riemann, scheme):
+    """a particle of negative internal energy: HYDRO_ENONFINITE, as the
+    solver's square roots of negative numbers give"""
+    from paper_2211_12243_gb300 import hydro
+    w = dict(W.lattice_wave(10, jitter=0.05))
+    for k in ("E", "U"):
+        w[k] = w[k].copy()
+        w[k][123] *= -0.1
+    s, _ = _step(hydro, w, 1e-3, scheme=scheme, riemann=riemann)
+    assert s["status"] == -7, s
+
+
 @pytest.mark.parametrize("riemann,scheme", [("exact", "mfv"), ("exact", "mfm"), ("hllc", "mfv"),
                                             ("hllc", "mfm")])
 def test_nan_gradients_reach_the_fluxes(riemann, scheme):

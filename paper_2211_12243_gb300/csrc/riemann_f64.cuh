@@ -129,6 +129,9 @@ __device__ __forceinline__ StarOut star_solve64(const GasK<double> &k, const Gas
             const float iw = __fdividef(1.f, wl + wr), x = narrow(N) * ipf;
             const double step = fma(N, widen(-0.5f * x * (wl * kl + wr * kr) * iw), N);
             p += step;
+            // (densities beyond the float range leave no weights for the curvatures
+            // and the step is not a number: the plain path)
+            if (!dpos(p)) break;
             if (fabsf(x) < 3e-6f) {
                 ps = p;
                 const double h = fma(dfr - dfl, step, fr - fl) +
@@ -137,7 +140,6 @@ __device__ __forceinline__ StarOut star_solve64(const GasK<double> &k, const Gas
                 o.iters = it + 1 + n;
                 return o;
             }
-            if (!dpos(p)) break;
             pf = narrow(p);
         }
     }

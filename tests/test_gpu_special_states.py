@@ -80,3 +80,25 @@ def test_nan_gradients_reach_the_fluxes(riemann, scheme):
     bad = ~np.isfinite(dQ.cpu().numpy()[:, :5])
     assert bad[77, 4] and np.count_nonzero(bad.any(1)) > 5
     H.close()
+
+
+@pytest.mark.parametrize("scheme", ["mfv", "mfm"])
+@pytest.mark.parametrize("unit", [1e-60, 1e-42, 1e42, 1e60])
+def test_uniform_pressure_at_densities_beyond_float(orc, scheme, unit):
+    from paper_2211_12243_gb300 import hydro
+    w = dict(W.lattice_wave(9, jitter=0.08))
+    n = w["x"].size
+    rng = np.random.default_rng(5)
+    w["m"] = unit / n * np.exp(0.3 * rng.standard_normal(n))
+    dt = 1e-3 * np.sqrt(unit)
+    # (the pressure the solver sees is U (gamma - 1) / omega: uniform to rounding)
+    cfg = orc.config(gamma=w["gamma"], scheme=scheme, limiter=1)
+    h, om, _, st = orc.density(cfg, w["x"], w["y"], w["z"], w["L"], w["h"])
+    w["U"] = om / (w["gamma"] - 1.0)
+    w["E"] = w["U"].copy()
+    o = oracle_stages(orc, cfg, w, dt)
+    H = hydro.Hydro(hydro.default_config(gamma=w["gamma"], scheme=scheme))
+    g = gpu_stages(hydro, H, w, dt)
+    errs, bad = compare(g, o, 1e-12, what=("h", "omega", "B", "grad", "ncond", "dQ"))
+    assert not bad, errs
+    H.close()

@@ -421,7 +421,7 @@ __device__ __forceinline__ void dens_one(const DensArgs &a, double *__restrict__
             const double dy = fold64(a.ys[j] - yi, bx.L[1]);
             const double dz = fold64(a.zs[j] - zi, bx.L[2]);
             const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-            const double q = dpos(r2) ? r2 * rsqrt64(r2) * ih : 0.0;
+            const double q = dnormal(r2) ? r2 * rsqrt64(r2) * ih : 0.0;   // (closer than 1e-154: r = 0)
             if (!dlt_pos(q, 1.0)) continue;
             const double t = 1.0 - q, t2 = t * t;
             double fn;

@@ -281,7 +281,8 @@ __device__ __forceinline__ bool face_state64(const FluxArgs &a, const GasK<doubl
     A[2] = fma(fma(Bi[2], d[0], fma(Bi[4], d[1], Bi[5] * d[2])), wi,
                fma(Bj[2], d[0], fma(Bj[4], d[1], Bj[5] * d[2])) * wj);
     const double A2 = fma(A[0], A[0], fma(A[1], A[1], A[2] * A[2]));
-    if (!dpos(A2)) return false;
+    // (an area below 1e-154, whose square is subnormal, is none)
+    if (!dpos(A2) || dlt_pos(A2, 2.2250738585072014e-308)) return false;
     const double inA = rsqrt64(A2);
     st.sA = dt * (A2 * inA);
     st.nh[0] = A[0] * inA; st.nh[1] = A[1] * inA; st.nh[2] = A[2] * inA;

@@ -81,7 +81,8 @@ __device__ __forceinline__ double rcp40(double x) {
     return fma(r, fma(-x, r, 1.0), r);
 }
 
-// 1 / sqrt(x), x > 0: with e = 1 - x r^2, (1 - e)^(-1/2) = 1 + e/2 + 3 e^2/8 + O(e^3)
+// 1 / sqrt(x), x positive, normal and finite (anything else gives infinity, 0 or
+// NaN: dnormal first where it can occur): with e = 1 - x r^2, (1 - e)^(-1/2) = 1 + e/2 + 3 e^2/8 + O(e^3)
 __device__ __forceinline__ double rsqrt64(double x) {
     const double r = rsqrt_seed(x);
     const double e = fma(-x * r, r, 1.0);

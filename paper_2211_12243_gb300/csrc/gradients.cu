@@ -124,7 +124,7 @@ __device__ __forceinline__ void grad_one64(const GradArgs &a, double *__restrict
         if (!member(d, r2)) continue;
         mypairs++;
         if (k < 64) members |= 1ull << k;
-        const double ir = dpos(r2) ? rsqrt64(r2) : 0.0, r = r2 * ir;   // (coincident particles: r = 0)
+        const double ir = dnormal(r2) ? rsqrt64(r2) : 0.0, r = r2 * ir;   // (coincident particles: r = 0)
         const double w = rj[R_OM] * (norm * kernel_shape<double>(a.kernel, r * ih));
         const double wd[3] = {w * d[0], w * d[1], w * d[2]};
         E[0] = fma(wd[0], d[0], E[0]);

@@ -102,3 +102,24 @@ def test_uniform_pressure_at_densities_beyond_float(orc, scheme, unit):
     errs, bad = compare(g, o, 1e-12, what=("h", "omega", "B", "grad", "ncond", "dQ"))
     assert not bad, errs
     H.close()
+
+
+@pytest.mark.parametrize("gap", [1e-156, 1e-161])
+def test_particles_whose_squared_distance_is_subnormal(orc, gap):
+    """two pairs of particles closer than 1e-154: as coincident ones, not NaN"""
+    from paper_2211_12243_gb300 import hydro
+    w = dict(W.lattice_wave(9, jitter=0.08))
+    for k in ("x", "y", "z"):
+        w[k] = w[k].copy()
+        w[k][100:102] = 0.0
+        w[k][300:302] = 0.0
+    w["x"][101] = gap
+    w["y"][300:302] = 0.5
+    w["z"][301] = gap
+    opts = dict(n_ngb=48.0)
+    o = oracle_stages(orc, orc.config(gamma=w["gamma"], **opts), w, 1e-3)
+    H = hydro.Hydro(hydro.default_config(gamma=w["gamma"], **opts))
+    g = gpu_stages(hydro, H, w, 1e-3, search=1.6)
+    errs, bad = compare(g, o, 1e-12, what=("h", "omega", "B", "grad", "ncond", "dQ"))
+    assert not bad, errs
+    H.close()

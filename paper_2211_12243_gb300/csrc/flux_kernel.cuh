@@ -107,7 +107,8 @@ __device__ __forceinline__ int sgn_(R v) { return (v > R(0)) - (v < R(0)); }
 // [lo - psi1 d, mean + psi2 d], the other in [mean - psi2 d, hi + psi1 d]
 // (d = |u - v|); for a positive field a bound that would change sign is shrunk
 // instead.  Both sides share the bounds, and the selections are without
-// branches (equal cells leave no room and give back the cell value).
+// branches.  Equal cells leave no room and give back the cell value, whatever the
+// factors (an infinite one switches its bound off, and times d = 0 is NaN).
 template <typename R>
 __device__ __forceinline__ void pair_limit(R &l, R &m, R u, R v, R psi1, R psi2, bool positive) {
     const R d = fabs(u - v), mean = R(0.5) * (u + v);
@@ -125,8 +126,8 @@ __device__ __forceinline__ void pair_limit(R &l, R &m, R u, R v, R psi1, R psi2,
     low = low > lox ? low : lox;
     high = high > bottom ? high : bottom;
     high = high < hix ? high : hix;
-    l = up ? low : high;
-    m = up ? high : low;
+    l = u == v ? u : up ? low : high;
+    m = u == v ? v : up ? high : low;
 }
 
 // r < h_j decided exactly (float path: band + double fallback)
@@ -315,7 +316,7 @@ __device__ __forceinline__ bool face_state64(const FluxArgs &a, const GasK<doubl
             const double hi2 = dmin_(dmax_(high, fma(-a.psi2, df, mean)), hix);
             l = up ? lo2 : hi2;
             m = up ? hi2 : lo2;
-            if (dbits(u) == dbits(v)) l = m = u;
+            if ((dbits(df) << 1) == 0) { l = u; m = v; }   // (equal cells)
         }
         Lf[f] = l;
         Rf[f] = m;

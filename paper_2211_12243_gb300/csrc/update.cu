@@ -94,7 +94,10 @@ __global__ void k_update(UpdArgs a) {
     double x = a.xs[s] + dt * 0.5 * (vx0 + vx1);
     double y = a.ys[s] + dt * 0.5 * (vy0 + vy1);
     double z = a.zs[s] + dt * 0.5 * (vz0 + vz1);
-    auto wrap = [](double v, double L) { return dneg(v) ? v + L : dlt_pos(v, L) ? v : v - L; };
+    // (-0.0 is not negative, but its bits are above those of L)
+    auto wrap = [](double v, double L) {
+        return dneg(v) ? v + L : dlt_pos(dabs_(v), L) ? v : v - L;
+    };
     x = wrap(x, bx.L[0]);
     y = wrap(y, bx.L[1]);
     z = wrap(z, bx.L[2]);

@@ -114,9 +114,11 @@ __device__ __forceinline__ int64_t sample_index(uint64_t seed, uint64_t step, ui
 }
 
 // Gradient of 0.5 mean (y - t)^2 over the nb samples of the minibatch: each
-// CTA takes tiles of 16 samples, keeps the sums of its tiles in registers and
-// writes them (and its share of the loss) to its row of `part`, which
-// k_mlp_reduce or k_mlp_adam folds -- no atomics, so training is reproducible.
+// CTA takes tiles of 16 samples and keeps the sums of its tiles in registers.
+// In training it writes them (and its share of the loss) to its row of `part`,
+// which k_mlp_adam folds -- no atomics, so training is reproducible.  For a
+// caller's gradient (grad not NULL) it adds them to the caller's zeroed arrays:
+// no scratch of the context, so calls on several streams do not meet.
 // A tile's layers are small matrix products with a few outputs per thread: bound by shared-memory reads and latency.  With a batch of 2048 it
 // runs on 128 CTAs; one thread per sample on 32 CTAs, the output layer's
 // gradient by shared atomics of all threads on one address, took 200 us a step;
@@ -138,7 +140,9 @@ __global__ void __launch_bounds__(GRAD_THREADS) k_mlp_grad(const float *__restri
                                                            const float *__restrict__ t, int64_t n,
                                                            int64_t nb, int random, uint64_t seed,
                                                            uint64_t step, int quant,
-                                                           float *__restrict__ part) {
+                                                           float *__restrict__ part,
+                                                           float *__restrict__ grad,
+                                                           float *__restrict__ loss) {
     __shared__ __align__(16) GradSmem S;
     const int tid = threadIdx.x;
     const bool q = quant != 0;
@@ -306,15 +310,18 @@ __global__ void __launch_bounds__(GRAD_THREADS) k_mlp_grad(const float *__restri
             gW1[i] += acc;
         }
     }
-    // the CTA's row
-    float *row = part + (int64_t)blockIdx.x * GRAD_ROW;
+    // the CTA's sums
+    auto put = [&](int e, float v) {
+        if (grad) atomicAdd(e < MLP_NTRAIN ? grad + e : loss, v);
+        else part[(int64_t)blockIdx.x * GRAD_ROW + e] = v;
+    };
 #pragma unroll
     for (int i = 0; i < 2; i++)
-        if (tid + i * GRAD_THREADS < MLP_NH * MLP_NF) row[MLP_OFF_W1 + tid + i * GRAD_THREADS] = gW1[i];
+        if (tid + i * GRAD_THREADS < MLP_NH * MLP_NF) put(MLP_OFF_W1 + tid + i * GRAD_THREADS, gW1[i]);
 #pragma unroll
     for (int i = 0; i < 2; i++)
 #pragma unroll
-        for (int j = 0; j < 4; j++) row[MLP_OFF_W2 + (bo + i) * MLP_NH + bk + j] = gW2[i][j];
+        for (int j = 0; j < 4; j++) put(MLP_OFF_W2 + (bo + i) * MLP_NH + bk + j, gW2[i][j]);
     // the sums over the sample groups
     __syncthreads();
     float *fold = &S.W2[0];   // (the weights are done with) [3][GRAD_NG][64]
@@ -327,7 +334,7 @@ __global__ void __launch_bounds__(GRAD_THREADS) k_mlp_grad(const float *__restri
         float v = 0.f;
 #pragma unroll
         for (int i = 0; i < GRAD_NG; i++) v += f[i * MLP_NH];
-        row[(tid < 64 ? MLP_OFF_B1 : tid < 128 ? MLP_OFF_B2 : MLP_OFF_W3) + o64] = v;
+        put((tid < 64 ? MLP_OFF_B1 : tid < 128 ? MLP_OFF_B2 : MLP_OFF_W3) + o64, v);
     }
     if (tid < 32) {
         for (int m = 8; m > 0; m >>= 1) {
@@ -335,8 +342,8 @@ __global__ void __launch_bounds__(GRAD_THREADS) k_mlp_grad(const float *__restri
             lsum += __shfl_xor_sync(0xffffffffu, lsum, m);
         }
         if (tid == 0) {
-            row[MLP_OFF_B3] = gb3;
-            row[MLP_NTRAIN] = lsum;
+            put(MLP_OFF_B3, gb3);
+            put(MLP_NTRAIN, lsum);
         }
     }
 }
@@ -356,18 +363,6 @@ __device__ __forceinline__ float fold_column(const float *__restrict__ part, int
     __syncthreads();
     return ((sh[0][col] + sh[1][col]) + (sh[2][col] + sh[3][col])) +
            ((sh[4][col] + sh[5][col]) + (sh[6][col] + sh[7][col]));
-}
-
-// gradients and loss to the caller's arrays
-__global__ void __launch_bounds__(256) k_mlp_reduce(const float *__restrict__ part, int nrow,
-                                                    float *__restrict__ grad,
-                                                    float *__restrict__ loss) {
-    __shared__ float sh[8][32];
-    const int e = blockIdx.x * 32 + (threadIdx.x & 31);
-    const float g = fold_column(part, nrow, e, sh);
-    if (threadIdx.x >= 32) return;
-    if (e < MLP_NTRAIN) grad[e] = g;
-    else if (e == MLP_NTRAIN) *loss = g;
 }
 
 __global__ void __launch_bounds__(256) k_mlp_adam(float *__restrict__ theta,
@@ -511,34 +506,28 @@ cudaError_t mlp_features(hydro_ctx *c, const float *faces, int64_t n, float *x, 
     return launch_check();
 }
 
-// partial sums of one minibatch into the context's rows; their number
+// CTAs (training: rows of partial sums) for nb samples
 static int grad_rows(int64_t nb) {
     return (int)std::min<int64_t>((nb + GRAD_TILE - 1) / GRAD_TILE, GRAD_CTAS);
 }
 
-static cudaError_t grad_partials(hydro_ctx *c, const float *x, const float *t, int64_t n, int64_t nb,
-                                 int random, uint64_t seed, uint64_t step, int quant, stream_t st) {
-    const int rows = grad_rows(nb);
-    HYD_CUDA(c->d_mlp_grad.ensure((size_t)rows * GRAD_ROW));
-    k_mlp_grad<<<rows, GRAD_THREADS, 0, st>>>(c->d_mlp.get(), x, t, n, nb, random, seed, step, quant,
-                                              c->d_mlp_grad.get());
-    return launch_check();
-}
-
 cudaError_t mlp_gradient(hydro_ctx *c, const float *x, const float *t, int64_t n, int quant,
                          float *grad, float *loss, stream_t st) {
-    HYD_CUDA(grad_partials(c, x, t, n, n, 0, 0, 0, quant, st));
-    k_mlp_reduce<<<grid_for(GRAD_ROW, 32), 256, 0, st>>>(c->d_mlp_grad.get(), grad_rows(n), grad, loss);
+    k_mlp_grad<<<grad_rows(n), GRAD_THREADS, 0, st>>>(c->d_mlp.get(), x, t, n, n, 0, 0, 0, quant,
+                                                      nullptr, grad, loss);
     return launch_check();
 }
 
 cudaError_t mlp_train_step(hydro_ctx *c, const float *x, const float *t, int64_t n, int64_t nb,
                            uint64_t seed, uint64_t step, float *m, float *v, float *loss, float lr,
                            int adam_step, stream_t st) {
-    HYD_CUDA(grad_partials(c, x, t, n, nb, 1, seed, step, 1, st));
-    k_mlp_adam<<<grid_for(GRAD_ROW, 32), 256, 0, st>>>(c->d_mlp.get(), c->d_mlp_grad.get(),
-                                                       grad_rows(nb), m, v, loss, lr, 0.9f, 0.999f,
-                                                       1e-8f, adam_step);
+    const int rows = grad_rows(nb);
+    HYD_CUDA(c->d_mlp_grad.ensure((size_t)rows * GRAD_ROW));
+    k_mlp_grad<<<rows, GRAD_THREADS, 0, st>>>(c->d_mlp.get(), x, t, n, nb, 1, seed, step, 1,
+                                              c->d_mlp_grad.get(), nullptr, nullptr);
+    HYD_CUDA(launch_check());
+    k_mlp_adam<<<grid_for(GRAD_ROW, 32), 256, 0, st>>>(c->d_mlp.get(), c->d_mlp_grad.get(), rows, m,
+                                                       v, loss, lr, 0.9f, 0.999f, 1e-8f, adam_step);
     return launch_check();
 }
 

@@ -75,3 +75,31 @@ def test_training_repeats_bitwise():
         H.close()
     assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
     assert out[0][0][-5:].mean() < out[0][0][:5].mean()
+
+
+def test_gradients_on_two_streams():
+    """Calls of one context on two streams at once, each with its own samples:
+    the gradients of the calls alone (to the order of float sums)"""
+    import torch
+    from paper_2211_12243_gb300 import hydro
+    H = hydro.Hydro(hydro.default_config(precision="mixed"))
+    H.mlp_load(mlp.init(9))
+    data, alone = [], []
+    for seed in (1, 2):
+        x, t, _ = _case(60000 + 17 * seed, seed)
+        data.append((torch.as_tensor(x, device="cuda"), torch.as_tensor(t * seed, device="cuda")))
+        g, loss = H.mlp_gradient(*data[-1])
+        alone.append((g.clone(), loss.clone()))
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in data]
+    out = []
+    for _ in range(10):
+        for s, d in zip(streams, data):
+            with torch.cuda.stream(s):
+                out.append(H.mlp_gradient(*d, stream=s))
+    torch.cuda.synchronize()
+    for k, (g, loss) in enumerate(out):
+        ga, la = alone[k % 2]
+        assert float((g - ga).abs().max()) <= 1e-5 * float(ga.abs().max())
+        assert float((loss - la).abs()) <= 1e-5 * float(la)
+    H.close()

@@ -60,6 +60,9 @@ struct DensArgs {
     bool rank;                // full solve: rank the CTA's 128 particles by list length
     const int32_t *list;      // the guard round's particles, their count on the device
     const int *nlist;         // (k_density_list; NULL: every particle)
+    const int32_t *buckets;   // a sparse sub-step's buckets (k_density_list; NULL: every particle)
+    int nbuckets;
+    const int32_t *node_first, *node_cnt;
     const uint4 *pos, *low;   // mixed path: high and low words of the 64-bit fixed-point x y z
 };
 
@@ -682,9 +685,16 @@ k_density_list(DensArgs a, R *__restrict__ rec) {
     __shared__ float rs[DENS_THREADS / 32][DENS_CACHE];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const Walk<32> wk{rs[warp], lane};
-    const int nl = a.list ? *a.nlist : (int)a.n;
+    const int nl = a.list ? *a.nlist : a.buckets ? a.nbuckets * BUCKET : (int)a.n;
     for (int t = blockIdx.x * (DENS_THREADS / 32) + warp; t < nl; t += gridDim.x * (DENS_THREADS / 32)) {
-        const int64_t s = a.list ? a.list[t] : t;
+        int64_t s = t;
+        if (a.list) {
+            s = a.list[t];
+        } else if (a.buckets) {
+            const int b = a.buckets[t / BUCKET], k = t % BUCKET;
+            if (k >= a.node_cnt[b]) continue;
+            s = a.node_first[b] + k;
+        }
         __syncwarp();
         dens_one<32>(a, rec, wk, s);
     }
@@ -748,15 +758,23 @@ cudaError_t run_density(hydro_ctx *c, bool only_active, bool compact, stream_t s
     a.nlist = &c->d_cnt->nguard;
     HYD_CUDA(cudaMemsetAsync(&c->d_cnt->search_fail, 0, sizeof(int), st));
     // a warp per particle: the guard round's list, or every particle of a set
-    // so small that a thread each would leave the GPU idle
-    // (the few buckets of a sparse sub-step of individual timesteps too)
+    // so small that a thread each would leave the GPU idle, also that of the few
+    // buckets of a sparse sub-step of individual timesteps, which hold all its
+    // starting particles (us a sub-step with a thread for each of all particles,
+    // with these warps over all particles, over the buckets: 48^3 422, 387, 381;
+    // 128^3 1273, 1345, 1223; 200^3 4029, 4406, 3960)
     const bool listed = guard && only_active;
     const bool sparse = c->rung_live && only_active && c->rung_touch_n >= 0 &&
                         c->rung_touch_n * BUCKET <= DENS_WARP_MAX;
     const bool warps = listed || sparse || n <= DENS_WARP_MAX;
     if (!listed) a.list = nullptr;
+    a.buckets = sparse && !listed ? c->d_touch.get() : nullptr;
+    a.nbuckets = a.buckets ? (int)c->rung_touch_n : 0;
+    a.node_first = c->d_node_first.get();
+    a.node_cnt = c->d_node_cnt.get();
+    const int64_t np = a.buckets ? (int64_t)a.nbuckets * BUCKET : n;
     const unsigned grid = !warps ? grid_for(n, DENS_THREADS)
-        : listed ? 152u * 8u : std::min(152u * 8u, grid_for(n * 32, DENS_THREADS));
+        : listed ? 152u * 8u : std::min(152u * 8u, grid_for(np * 32, DENS_THREADS));
     if (c->cfg.precision == HYDRO_MIXED) {
         a.pos = c->d_pos.get();   // (gather_state)
         a.low = c->d_low.get();

@@ -208,3 +208,32 @@ def test_sparse_substeps_match_oracle(orc, hyd, scheme, precision, tol):
         d_g = sg[k] - w[k]
         scale = np.abs(d_o).max() + 1e-300
         assert np.max(np.abs(d_g - d_o)) < max(tol, 1e-12) * scale * 10 + 1e-300, k
+
+
+@pytest.mark.parametrize("precision,tol", [("fp64", 1e-12), ("mixed", 1e-5)])
+def test_sparse_substeps_with_a_short_last_bucket(orc, hyd, precision, tol):
+    """A blast at the corner of the box, on a lattice of 22^3 (332 buckets and 24
+    particles): the first and the last buckets of the order hold the starting
+    particles of the sparse sub-steps."""
+    w = dict(W.sedov(22))
+    for k in ("x", "y", "z"):
+        w[k] = np.mod(w[k] + 0.5, 1.0)
+    co = orc.config(gamma=w["gamma"], scheme="mfm")
+    _, _, i0 = orc.step(co, w, -1.0)
+    dt0 = 20.0 * i0["dt"]
+    so, rung_o, io = orc.step_rungs(co, w, dt0)
+    assert io["status"] == 0 and io["substeps"] >= 8
+    assert _margin(dt0, io["dt_cfl"], io["dt_acc"]) > (1e-4 if precision == "mixed" else 1e-9)
+    cg = hyd.default_config(gamma=w["gamma"], precision=precision, scheme="mfm")
+    sg, rung_g, stats = _run_gpu(hyd, w, cg, dt0)
+    assert stats["status"] == 0, stats
+    assert stats["rung_sparse"] >= stats["substeps"] // 2, stats
+    assert np.array_equal(rung_g, rung_o)
+    assert stats["flux_pairs"] == io["faces"]
+    for k in ("h", "omega"):
+        assert np.max(np.abs(sg[k] - so[k]) / np.abs(so[k])) < tol * 10, k
+    for k in ("px", "py", "pz", "E", "U"):
+        d_o = so[k] - w[k]
+        d_g = sg[k] - w[k]
+        scale = np.abs(d_o).max() + 1e-300
+        assert np.max(np.abs(d_g - d_o)) < max(tol, 1e-12) * scale * 10 + 1e-300, k

@@ -130,8 +130,8 @@ __device__ __forceinline__ StarOut star_solve64(const GasK<double> &k, const Gas
             const double step = fma(N, widen(-0.5f * x * (wl * kl + wr * kr) * iw), N);
             p += step;
             // (densities beyond the float range leave no weights for the curvatures
-            // and the step is not a number: the plain path)
-            if (!dpos(p)) break;
+            // and the step is not a number or infinite: the plain path)
+            if (!dnormal(p)) break;
             if (fabsf(x) < 3e-6f) {
                 ps = p;
                 const double h = fma(dfr - dfl, step, fr - fl) +
@@ -153,7 +153,7 @@ __device__ __forceinline__ void star_sample64(const GasK<double> &k, const GasK<
                                               double rl, double ul, double pl, double cl, double rr,
                                               double ur, double pr, double cr, double ps, double us,
                                               double &rho, double &u, double &p, int &side) {
-    const bool left = !dneg(us);
+    const bool left = dge0(us);   // (a speed that is not a number: right)
     side = left ? -1 : 1;
     const double rK = left ? rl : rr, pK = left ? pl : pr, cK = left ? cl : cr;
     const double uK = left ? ul : -ur, uS = left ? us : -us;
@@ -167,7 +167,7 @@ __device__ __forceinline__ void star_sample64(const GasK<double> &k, const GasK<
             vs = uS;
             qs = ps;
         }
-    } else if (dlt(uK, cK)) {   // (else beyond the rarefaction's head)
+    } else if (!dge0(uK - cK)) {   // (else beyond the rarefaction's head)
         double tz;
         if (k.nz > 0) {
             tz = 1.0 + pow_z_m1(k, ps, pK, __powf(__fdividef(narrow(ps), narrow(pK)), kf.z));
@@ -176,7 +176,8 @@ __device__ __forceinline__ void star_sample64(const GasK<double> &k, const GasK<
         }
         const double cm = cK * tz;
         // (a right side keeps its tail point in the star region)
-        const bool star = left ? dlt(uS, cm) : !dlt(cm, uS);
+        const double e = uS - cm;
+        const bool star = dneg(e) || (!left && (dbits(e) << 1) == 0);
         if (star) {
             rs = rK * (k.n4 > 0 ? ipow64(tz, k.n4) : pow(ps / pK, k.inv_g));
             vs = uS;
@@ -184,7 +185,7 @@ __device__ __forceinline__ void star_sample64(const GasK<double> &k, const GasK<
         } else {
             // inside the fan
             const double cc = k.g5 + k.g6 * uK * rcp64(cK);
-            const double c4 = k.n4 > 0 ? ipow64(cc, k.n4) : pow(cc, k.g4);
+            const double c4 = k.n4 > 0 && dge0(cc) ? ipow64(cc, k.n4) : pow(cc, k.g4);
             rs = rK * c4;
             vs = k.g5 * (cK + 0.5 * k.gm1 * uK);
             qs = pK * (c4 * cc * cc);   // cc^(2g/(g-1)) = cc^(2/(g-1)) cc^2

@@ -228,9 +228,11 @@ struct NewtonF {
 // A particle's list walked by one lane (W = 1) or by the 32 of a warp (a guard
 // round's few particles, whose lists at the doubled radius are long).  A warp
 // gathers the separations in parallel, once, into shared memory (the first
-// CACHE), and evaluates the refinement's entries in parallel; the sums
-// themselves are taken in the list's order in both forms, so a particle's root
-// does not depend on which form solves it.  A lane on its own gathers the
+// CACHE), and evaluates the refinement's entries in parallel.  The float
+// iteration and the mixed path's refinement take their sums in the list's order
+// in both forms, so a mixed root does not depend on which form solves it; the
+// FP64 finish of a warp sums every 32nd entry per lane and folds, which rounds
+// differently from a lane's serial sum.  A lane on its own gathers the
 // separations again in every pass (a running step's h takes one or two passes;
 // keeping 16 to 64 of a thread's separations in shared memory took its L1 and
 // was between 7 % faster and 50 % slower).
@@ -356,10 +358,6 @@ __device__ __forceinline__ void dens_fail(const DensArgs &a, int64_t s) {
 // float evaluations before the iteration starts again in double
 constexpr int FLOAT_ITER = 12;
 
-// Bound by the FP64 pipe: 23 FP64 instructions per neighbour in one pass,
-// where five passes of Newton's iteration and one for omega, with a square
-// root rounded correctly per neighbour, took about 220 (1.07 M tube 11.1 ->
-// 2.95 ms, 300k log-normal box 4.7 -> 0.88 ms).
 // h^2 d^2f/dh^2 of f(r/h) in float
 __device__ __forceinline__ float kernel_curv(int kernel, float q) {
     const float t = 1.f - q, q2 = q * q;
@@ -367,6 +365,10 @@ __device__ __forceinline__ float kernel_curv(int kernel, float q) {
     return q <= 0.5f ? -36.f * q2 + 72.f * q2 * q : 12.f * q * t * (q - t);
 }
 
+// Bound by the FP64 pipe: 23 FP64 instructions per neighbour in one pass,
+// where five passes of Newton's iteration and one for omega, with a square
+// root rounded correctly per neighbour, took about 220 (1.07 M tube 11.1 ->
+// 2.95 ms, 300k log-normal box 4.7 -> 0.88 ms).
 template <int W>
 __device__ __forceinline__ void dens_one(const DensArgs &a, double *__restrict__ rec,
                                          const Walk<W> &wk, int64_t s) {

@@ -115,3 +115,35 @@ def test_warp_and_thread_solves_agree(orc, hyd, n):
         ok = h < 0.48
         assert np.max(np.abs(s["h"].cpu().numpy() / h - 1)[ok]) < 1e-12
         H.close()
+
+
+@pytest.mark.parametrize("precision", ["mixed", "fp64"])
+def test_forms_of_the_solve_on_the_same_particles(hyd, precision):
+    """A box of 4,000 particles alone (a warp each) and beside one of 5,000 (a
+    thread each): the same lists, so the same bits in the mixed path, which sums
+    in the list's order in both forms.  In FP64 a warp's lanes sum every 32nd entry
+    and fold: at most 60 reordered terms, 60 2^-53 of a sum whose logarithmic slope
+    in h is about three."""
+    import torch
+    rng = np.random.default_rng(12)
+    n = (4000, 5000)
+    c = rng.random((3, sum(n)))
+    c[:, :2000] = 0.5 + 0.2 * (c[:, :2000] - 0.5)   # (denser in the middle of the first box)
+    out = []
+    for k in (1, 2):
+        m = sum(n[:k])
+        H = hyd.Hydro(hyd.default_config(precision=precision))
+        H.set_boxes(np.concatenate([[0], np.cumsum(n[:k])]).astype(np.int64), np.ones(3 * k))
+        dev = lambda v: torch.as_tensor(np.ascontiguousarray(v), device="cuda")
+        h0 = np.full(m, np.cbrt(24.0 / np.pi / 4000))
+        s = {"x": dev(c[0, :m]), "y": dev(c[1, :m]), "z": dev(c[2, :m]), "h": dev(h0),
+             "omega": dev(np.zeros(m))}
+        H.build_neighbours(s, dev(np.full(m, 0.25)), export=False)
+        H.density(s)
+        out.append([s[q].cpu().numpy()[:n[0]] for q in ("h", "omega")])
+        H.close()
+    for a, b in zip(*out):
+        if precision == "mixed":
+            assert np.array_equal(a, b)
+        else:
+            assert np.max(np.abs(a / b - 1.0)) <= 3 * 60 * 2.0 ** -53

@@ -56,3 +56,26 @@ def test_fp64_fluxes_match_oracle(orc, riemann, scheme, state):
     g = gpu_stages(hydro, H, w, dt)
     errs, bad = compare(g, o, 1e-12, what=("h", "omega", "B", "grad", "ncond", "dQ"))
     assert not bad, errs
+
+
+@pytest.mark.parametrize("scheme", ["mfv", "mfm"])
+def test_fp64_flux_sums_repeat(scheme):
+    """The sums of the faces' contributions, whose additions arrive in any order:
+    the rounding errors are summed beside them, so repeated calls agree to the
+    rounding of the total (one unit in its last place) and of the errors' sum
+    (2^-53 of at most 200 errors of 2^-53 of the largest contribution)."""
+    import torch
+    from paper_2211_12243_gb300 import hydro, workloads
+    w = workloads.lognormal(30011, seed=4, grid=32, contrast=100.0)
+    H = hydro.Hydro(hydro.default_config(gamma=w["gamma"], scheme=scheme))
+    H.set_boxes(*hydro.single_box(w))
+    st = hydro.to_device(w)
+    assert H.step(st, 1e-9, check=False)["status"] in (0, -5)   # (smoothing lengths)
+    H.build_neighbours(st, st["h"] * 1.05, export=False)
+    H.density(st)
+    B, G, A, _ = H.gradients(st)
+    dQ = np.stack([H.fluxes(st, B, G, A, 1e-3).cpu().numpy()[:, :5] for _ in range(8)])
+    spread = dQ.max(0) - dQ.min(0)
+    bound = np.spacing(np.abs(dQ).max(0)) + 200 * 2.0 ** -106 * np.abs(dQ).max((0, 1))
+    assert np.all(spread <= bound)
+    H.close()

@@ -182,7 +182,7 @@ struct Separation<float> {
     const uint4 *pos;
     uint32_t qx, qy, qz;
     float sx, sy, sz;
-    __device__ __forceinline__ Separation(const DensArgs &a, const float *, int64_t s, const Box &bx)
+    __device__ __forceinline__ Separation(const DensArgs &a, int64_t s, const Box &bx)
         : pos(a.pos), sx(bx.s[0]), sy(bx.s[1]), sz(bx.s[2]) {
         const uint4 pi = pos[s];
         qx = pi.x; qy = pi.y; qz = pi.z;
@@ -201,7 +201,7 @@ struct Separation<double> {
     const uint32_t *px, *py, *pz;
     uint32_t qx, qy, qz;
     float sx, sy, sz;
-    __device__ __forceinline__ Separation(const DensArgs &a, const double *, int64_t s, const Box &bx)
+    __device__ __forceinline__ Separation(const DensArgs &a, int64_t s, const Box &bx)
         : px(a.qx), py(a.qy), pz(a.qz) {
         const double u = bx.rLmax * (1.0 / 4294967296.0);
         sx = (float)(bx.L[0] * u); sy = (float)(bx.L[1] * u); sz = (float)(bx.L[2] * u);
@@ -381,7 +381,7 @@ __device__ __forceinline__ void dens_one(const DensArgs &a, double *__restrict__
     // (the float iteration's lengths are in units of the longest side)
     const double Lmax = bx.Lmax, rLmax = bx.rLmax;
     const float xmin = 1.f / 65536.f;
-    const Separation<double> sep(a, rec, s, bx);
+    const Separation<double> sep(a, s, bx);
     const float hsf = (float)(hsi_d * rLmax);
     float hf = (float)(hguess * rLmax);
     if (!(hf > 0.f) || hf > hsf) hf = hsf;
@@ -529,7 +529,7 @@ __device__ __forceinline__ void dens_one(const DensArgs &a, float *__restrict__ 
     if (s >= a.n) return;
     if (a.only_active && !(a.active[s] & 1)) return;
     const Box bx = a.boxes[a.pbox[s]];
-    const Separation<float> sep(a, rec, s, bx);
+    const Separation<float> sep(a, s, bx);
     const double hsi_d = a.hs[s];
     float hsi = (float)hsi_d;
     const float N = (float)(a.nngb ? a.nngb[s] : a.n_ngb);

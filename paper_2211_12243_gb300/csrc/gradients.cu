@@ -48,7 +48,7 @@ struct GradArgs {
                                          // (k_primitives; the entropy switch uses the slot)
 };
 
-// grad_one in FP64, bound by the FP64 pipe: 72 FP64 instructions per
+// A particle's gradients in FP64, bound by the FP64 pipe: 72 FP64 instructions per
 // neighbour where the general form issued about 190 (gradient stage of the
 // 1.07 M tube 9.66 -> 5.34 ms, 32^3 lattice 0.38 -> 0.23 ms).  The
 // sound speeds are formed once per particle (k_primitives), 1/r and r come
@@ -56,7 +56,7 @@ struct GradArgs {
 // integers, and membership is decided from the fused r^2 (the definition's
 // rounding only matters within 1e-14 of h^2) and remembered for the second pass.
 template <bool LEAN>
-__device__ __forceinline__ void grad_one64(const GradArgs &a, double *__restrict__ rec, int64_t s) {
+__device__ __forceinline__ void grad_one(const GradArgs &a, double *__restrict__ rec, int64_t s) {
     if (!(s < a.n && (!a.only_redo || (a.active[s] & ACT_REDO)) && (LEAN || !a.ract || a.ract[s]))) {
         if (!LEAN && s < a.n && a.ract && !a.ract[s]) {
             // not starting a step: no pairs, no CFL limit in this sub-step
@@ -246,16 +246,12 @@ __device__ __forceinline__ void grad_one64(const GradArgs &a, double *__restrict
     }
 }
 
-// MINB: resident CTAs per SM the register allocation must allow (1, FP64: no
-// bound; 4, 5, 6: the variants hydro_autotune times)
+// A particle's gradients in the mixed path.
 // LEAN: compiled without the staged outputs (outB, outG, outA, outN) and
 // the individual-timestep mask, which hydro_step does not use
-template <typename R, bool LEAN>
-__device__ __forceinline__ void grad_one(const GradArgs &a, R *__restrict__ rec, int64_t s) {
-    if constexpr (sizeof(R) == 8) {
-        grad_one64<LEAN>(a, rec, s);
-        return;
-    }
+template <bool LEAN>
+__device__ __forceinline__ void grad_one(const GradArgs &a, float *__restrict__ rec, int64_t s) {
+    using R = float;
     int mypairs = 0;
     if (s < a.n && (!a.only_redo || (a.active[s] & ACT_REDO)) && (LEAN || !a.ract || a.ract[s])) {
         const Box bx = a.boxes[a.pbox[s]];
@@ -338,19 +334,12 @@ __device__ __forceinline__ void grad_one(const GradArgs &a, R *__restrict__ rec,
             Bd[3] = (e00 * e22 - e02 * e02) * id;
             Bd[4] = (e02 * e01 - e00 * e12) * id;
             Bd[5] = (e00 * e11 - e01 * e01) * id;
-            if (sizeof(R) == 8) {
-                double nE = e00 * e00 + e11 * e11 + e22 * e22 + 2.0 * (e01 * e01 + e02 * e02 + e12 * e12);
-                double nB = Bd[0] * Bd[0] + Bd[3] * Bd[3] + Bd[5] * Bd[5] +
-                            2.0 * (Bd[1] * Bd[1] + Bd[2] * Bd[2] + Bd[4] * Bd[4]);
-                ncond = sqrt(nB * nE) / 3.0;
-            } else {
-                // N_cond only feeds the threshold test and the limiter's beta
-                float b0 = (float)Bd[0], b1 = (float)Bd[1], b2 = (float)Bd[2], b3 = (float)Bd[3],
-                      b4 = (float)Bd[4], b5 = (float)Bd[5];
-                float nE = E[0] * E[0] + E[3] * E[3] + E[5] * E[5] + 2.f * (E[1] * E[1] + E[2] * E[2] + E[4] * E[4]);
-                float nB = b0 * b0 + b3 * b3 + b5 * b5 + 2.f * (b1 * b1 + b2 * b2 + b4 * b4);
-                ncond = (double)(sqrtf(nB * nE) * (1.f / 3.f));
-            }
+            // N_cond only feeds the threshold test and the limiter's beta
+            float b0 = (float)Bd[0], b1 = (float)Bd[1], b2 = (float)Bd[2], b3 = (float)Bd[3],
+                  b4 = (float)Bd[4], b5 = (float)Bd[5];
+            float nE = E[0] * E[0] + E[3] * E[3] + E[5] * E[5] + 2.f * (E[1] * E[1] + E[2] * E[2] + E[4] * E[4]);
+            float nB = b0 * b0 + b3 * b3 + b5 * b5 + 2.f * (b1 * b1 + b2 * b2 + b4 * b4);
+            ncond = (double)(sqrtf(nB * nE) * (1.f / 3.f));
         } else {
             for (int k = 0; k < 6; k++) Bd[k] = 0.0;
             ncond = INFINITY;
@@ -420,9 +409,7 @@ __device__ __forceinline__ void grad_one(const GradArgs &a, R *__restrict__ rec,
         // CFL timestep of Eq. 31 with the signal velocity of Eq. 32 (the
         // minimum over particles is taken by k_grad_reduce)
         double dti = INFINITY;
-        if (vs > R(0))
-            dti = sizeof(R) == 8 ? a.c_cfl * hd / (double)vs
-                                 : (double)((float)a.c_cfl * (float)hd / (float)vs);
+        if (vs > R(0)) dti = (double)((float)a.c_cfl * (float)hd / (float)vs);
         a.dt_part[s] = dti;
         a.npair[s] = mypairs;
         // N_cond guard (§2.3.5)
@@ -439,14 +426,16 @@ __device__ __forceinline__ void grad_one(const GradArgs &a, R *__restrict__ rec,
 
 // one thread per particle: every particle (list NULL), or the *nlist
 // particles of list (a guard round's recomputed particles; the count is
-// read on the device, the warps take them 32 at a time)
+// read on the device, the warps take them 32 at a time).  MINB: resident CTAs per
+// SM the register allocation must allow (1, FP64: no bound; 4, 5, 6: the variants
+// hydro_autotune times)
 template <typename R, int MINB, bool LEAN = false>
 __global__ void __launch_bounds__(128, MINB) k_gradients(GradArgs a, R *__restrict__ rec) {
     if (a.list) {
         const int nl = *a.nlist;
         for (int base = warp_chunk(a.cursor); base < nl; base = warp_chunk(a.cursor)) {
             const int t = base + (threadIdx.x & 31);
-            if (t < nl) grad_one<R, LEAN>(a, rec, a.list[t]);
+            if (t < nl) grad_one<LEAN>(a, rec, a.list[t]);
         }
         return;
     }
@@ -459,7 +448,7 @@ __global__ void __launch_bounds__(128, MINB) k_gradients(GradArgs a, R *__restri
     if (a.rank_rounds) rank_tile(rank_key, rounds, a.nbr_cnt, tile, a.n);
     for (int r = 0; r < rounds; r++) {
         const int t = r * RANK_THREADS + threadIdx.x;
-        grad_one<R, LEAN>(a, rec, tile + (a.rank_rounds ? rank_index(rank_key[t], rounds) : t));
+        grad_one<LEAN>(a, rec, tile + (a.rank_rounds ? rank_index(rank_key[t], rounds) : t));
     }
 }
 

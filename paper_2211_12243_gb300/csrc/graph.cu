@@ -231,7 +231,7 @@ std::vector<unsigned long long> graph_key(const hydro_ctx *c, const hydro_partic
           (const void *)c->d_node_aabb.get(), (const void *)c->d_node_aabb_hi.get(),
           (const void *)c->d_keys.get(), (const void *)c->d_keys_alt.get(),
           (const void *)c->d_perm.get(), (const void *)c->d_perm_alt.get(),
-          (const void *)c->d_scan_tmp.get(), (const void *)c->d_hist.get(),
+          (const void *)c->d_scan_tmp.get(),
           (const void *)c->d_xs.get(), (const void *)c->d_ys.get(), (const void *)c->d_zs.get(),
           (const void *)c->d_hs.get(), (const void *)c->d_hsorted.get(),
           (const void *)c->d_omsorted.get(), (const void *)c->d_qx.get(),

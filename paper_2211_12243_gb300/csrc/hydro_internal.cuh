@@ -171,7 +171,6 @@ struct hydro_ctx {
     hyd::DevBuf<unsigned long long> d_keys, d_keys_alt;
     hyd::DevBuf<int32_t> d_perm, d_perm_alt;
     hyd::DevBuf<int64_t> d_scan_tmp;
-    hyd::DevBuf<int32_t> d_hist;
 
     // sorted state
     hyd::DevBuf<double> d_xs, d_ys, d_zs, d_hs, d_hsorted, d_omsorted;

@@ -1203,8 +1203,7 @@ cudaError_t rebuild_active_lists_dev(hydro_ctx *c, stream_t st, bool guard) {
         P.nbucket, c->d_node_first.get(), c->d_node_cnt.get(), c->d_active.get(), c->d_ovf.get(),
         &c->d_cnt->ovf_buckets, c->d_cnt);
     HYD_CUDA(launch_check());
-    // (in a guard round only the guard particles' radii grew)
-    HYD_CUDA(guard ? raise_tree(c, st) : build_tree(c, st));
+    HYD_CUDA(build_tree(c, st));
     return build_lists_queued_dev(c, st);
 }
 

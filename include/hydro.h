@@ -517,7 +517,7 @@ typedef struct {
     int grad_min_ctas;
     int flux_min_ctas;
     float front_ms[4][3];     /* [margin][slots] */
-    float grad_ms[4];         /* [1, 4, 5, 6] */
+    float grad_ms[4];         /* [1, 4, 5, 6]; mixed: 1 launches 5, timed once */
     float flux_ms[3];         /* [4, 5, 6]; 0 in FP64 */
     int flux_queue;
     float flux_queue_ms[2];   /* [by index, drawn]; 0 in FP64 */

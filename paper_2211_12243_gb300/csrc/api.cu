@@ -1108,6 +1108,10 @@ int hydro_autotune(hydro_ctx *c, hydro_particles *p, hydro_tuning *out, hydro_st
     best = 1e30f;
     int bg = 1;
     for (int k = 0; k < 4; k++) {
+        if (c->cfg.precision == HYDRO_MIXED && gminb[k] == 5) {   // (what 1 launches)
+            T.grad_ms[k] = T.grad_ms[0];
+            continue;
+        }
         c->grad_minb = gminb[k];
         float t = 1e30f;
         for (int rep = 0; rep < 2; rep++) {

@@ -96,7 +96,8 @@ __global__ void k_update(UpdArgs a) {
     double z = a.zs[s] + dt * 0.5 * (vz0 + vz1);
     // (-0.0 is not negative, but its bits are above those of L)
     auto wrap = [](double v, double L) {
-        return dneg(v) ? v + L : dlt_pos(dabs_(v), L) ? v : v - L;
+        if (!dlt_pos(v, L)) v = dneg(v) ? v + L : (dbits(v) << 1) == 0 ? v : v - L;
+        return v;
     };
     x = wrap(x, bx.L[0]);
     y = wrap(y, bx.L[1]);

@@ -41,8 +41,9 @@ struct UpdArgs {
 
 // One reciprocal per mass serves its three quotients and comparisons run on the
 // integer pipe: with IEEE divisions the FP64 pipe bound it (update stage with
-// the totals, 2,097,152 particles: 0.55 -> 0.31 ms; it still does: without the second
-// reciprocal where no mass moved and the corrections of the drift velocities 0.28).
+// the totals, 2,097,152 particles: 0.55 -> 0.29 ms; it still does).  FP64: the flux
+// sums carry their rounding errors.
+template <bool FP64>
 __global__ void k_update(UpdArgs a) {
     int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (s >= a.n) return;
@@ -61,7 +62,7 @@ __global__ void k_update(UpdArgs a) {
     double E0 = a.Q[4 * n + s], U0 = a.Q[5 * n + s];
     double dm = a.dQ[s], dpx = a.dQ[n + s], dpy = a.dQ[2 * n + s], dpz = a.dQ[3 * n + s];
     double dE = a.dQ[4 * n + s];
-    if (a.dQe) {
+    if (FP64) {
         dm += a.dQe[s]; dpx += a.dQe[n + s]; dpy += a.dQe[2 * n + s]; dpz += a.dQe[3 * n + s];
         dE += a.dQe[4 * n + s];
     }
@@ -86,10 +87,8 @@ __global__ void k_update(UpdArgs a) {
         py1 += w * ay;
         pz1 += w * az;
     }
-    // (these velocities only move the particle by a small part of the box: the
-    // product's last bit is far below the position's)
     const double r1 = moved ? rcp64(m1) : r0;
-    const double vx1 = px1 * r1, vy1 = py1 * r1, vz1 = pz1 * r1;
+    const double vx1 = div1(px1, m1, r1), vy1 = div1(py1, m1, r1), vz1 = div1(pz1, m1, r1);
     const Box bx = a.boxes[a.pbox[s]];
     double x = a.xs[s] + dt * 0.5 * (vx0 + vx1);
     double y = a.ys[s] + dt * 0.5 * (vy0 + vy1);
@@ -252,7 +251,8 @@ cudaError_t run_update(hydro_ctx *c, hydro_particles *p, double dt, const double
     a.A1 = c->ent_live ? c->d_A1.get() : nullptr;
     a.dS = c->ent_live && c->cfg.scheme == HYDRO_MFV ? c->d_dS.get() : nullptr;
     a.A_out = c->entA;
-    k_update<<<grid_for(a.n, 256), 256, 0, st>>>(a);
+    if (a.dQe) k_update<true><<<grid_for(a.n, 256), 256, 0, st>>>(a);
+    else k_update<false><<<grid_for(a.n, 256), 256, 0, st>>>(a);
     return launch_check();
 }
 

@@ -282,8 +282,8 @@ __device__ __forceinline__ bool face_state64(const FluxArgs &a, const GasK<doubl
     A[2] = fma(fma(Bi[2], d[0], fma(Bi[4], d[1], Bi[5] * d[2])), wi,
                fma(Bj[2], d[0], fma(Bj[4], d[1], Bj[5] * d[2])) * wj);
     const double A2 = fma(A[0], A[0], fma(A[1], A[1], A[2] * A[2]));
-    // (an area below 1e-154, whose square is subnormal, is none)
-    if (!dpos(A2) || dlt_pos(A2, 2.2250738585072014e-308)) return false;
+    // (an area below 1e-154, whose square is subnormal, is none, nor is NaN)
+    if (dhi(A2) - 0x00100000u > 0x7fe00000u) return false;
     const double inA = rsqrt64(A2);
     st.sA = dt * (A2 * inA);
     st.nh[0] = A[0] * inA; st.nh[1] = A[1] * inA; st.nh[2] = A[2] * inA;
@@ -316,7 +316,7 @@ __device__ __forceinline__ bool face_state64(const FluxArgs &a, const GasK<doubl
             const double hi2 = dmin_(dmax_(high, fma(-a.psi2, df, mean)), hix);
             l = up ? lo2 : hi2;
             m = up ? hi2 : lo2;
-            if ((dbits(df) << 1) == 0) { l = u; m = v; }   // (equal cells)
+            if (dzero(df)) { l = u; m = v; }   // (equal cells)
         }
         Lf[f] = l;
         Rf[f] = m;

@@ -19,6 +19,7 @@
 namespace hyd {
 
 __device__ __forceinline__ long long dbits(double v) { return __double_as_longlong(v); }
+__device__ __forceinline__ unsigned dhi(double v) { return (unsigned)__double2hiint(v); }
 
 // 0 < v (v not NaN), without the FP64 pipe
 __device__ __forceinline__ bool dpos(double v) {
@@ -27,13 +28,18 @@ __device__ __forceinline__ bool dpos(double v) {
 
 // v positive, normal and finite
 __device__ __forceinline__ bool dnormal(double v) {
-    return (unsigned long long)dbits(v) - 0x0010000000000000ull < 0x7fe0000000000000ull;
+    return dhi(v) - 0x00100000u < 0x7fe00000u;
 }
 
-// 0 <= v (-0 included; v not NaN)
+// v zero (of either sign)
+__device__ __forceinline__ bool dzero(double v) {
+    return ((dhi(v) << 1) | (unsigned)__double2loint(v)) == 0u;
+}
+
+// 0 <= v for a result of arithmetic (whose NaN is 0x7fffffff ffffffff), from the high
+// word: -0 counts, as do negative numbers above -2^-1042
 __device__ __forceinline__ bool dge0(double v) {
-    const unsigned long long b = (unsigned long long)dbits(v);
-    return b <= 0x7ff0000000000000ull || b == 0x8000000000000000ull;
+    return dhi(v) <= 0x7ff00000u || dhi(v) == 0x80000000u;
 }
 
 // v < 0 (neither -0 nor NaN)
@@ -107,7 +113,10 @@ __device__ __forceinline__ double sqrt_rest(double x) {
 __device__ __forceinline__ double sqrt64(double x) {
     const double r = rsqrt64(x);
     const double s = x * r;
-    return dnormal(x) ? fma(fma(-s, s, x), 0.5 * r, s) : sqrt_rest(x);
+    const double t = fma(fma(-s, s, x), 0.5 * r, s);
+    // (a negative operand's seed is NaN)
+    if (((dhi(x) >> 20) & 0x7ffu) - 1u >= 0x7feu) return sqrt_rest(x);
+    return t;
 }
 
 // a / b from y = 1/b (within an ulp): each step adds the exactly computed

@@ -177,7 +177,7 @@ __device__ __forceinline__ void star_sample64(const GasK<double> &k, const GasK<
         const double cm = cK * tz;
         // (a right side keeps its tail point in the star region)
         const double e = uS - cm;
-        const bool star = dneg(e) || (!left && (dbits(e) << 1) == 0);
+        const bool star = dneg(e) || (!left && dzero(e));
         if (star) {
             rs = rK * (k.n4 > 0 ? ipow64(tz, k.n4) : pow(ps / pK, k.inv_g));
             vs = uS;

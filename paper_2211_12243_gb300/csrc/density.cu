@@ -222,6 +222,7 @@ struct NewtonF {
     int c;         // entries of the list
     int it;        // evaluations
     bool conv, fail;
+    bool flat;     // the sum hardly grows with h at the last evaluation (see FLAT)
     float kf;      // N_enc(hsi) = Kn sum f at a failure
 };
 
@@ -267,6 +268,12 @@ struct Walk {
     }
 };
 
+// A sum f whose logarithmic slope in h is below this fixes its float root too
+// coarsely for the margin of a compacted list (f is good to about 1e-6, the margin
+// is 5e-5): N_NGB within a few parts in a hundred of the particle's own term, where
+// the slope of an ordinary N_NGB is about three.
+constexpr float FLAT = 0.1f;
+
 // the safeguarded Newton iteration of one particle over its list idx
 template <int W, typename Sep>
 __device__ __forceinline__ NewtonF newton_float(const DensArgs &a, const Sep &sep, int32_t *idx, int c,
@@ -275,11 +282,13 @@ __device__ __forceinline__ NewtonF newton_float(const DensArgs &a, const Sep &se
     NewtonF o;
     o.comp = -1.f;
     o.conv = o.fail = false;
+    o.flat = true;
     o.kf = 0.f;
     o.it = 0;
     const float Kn = kernel_Kn<float>(a.kernel);
     const float ftol = 2e-6f;
     float lo = 0.f, hi = -1.f;
+    bool hi_flat = true;   // the bracket hi is that of a flat sum
     const int c0 = min(c, Walk<W>::CACHE);
     if (W > 1) {
 #pragma unroll 4
@@ -294,7 +303,7 @@ __device__ __forceinline__ NewtonF newton_float(const DensArgs &a, const Sep &se
         // float r < X (1 + 1e-4) leaves the list complete for every
         // r < X (1 + 5e-5) when X > L / 65536, L the longest side, which sets the
         // separation's error (compaction is skipped below that)
-        const bool shrink = a.compact && hi > xmin && hi < 0.8f * hsi;
+        const bool shrink = a.compact && hi > xmin && hi < 0.8f * hsi && !hi_flat;
         const float keep = hi * 1.0001f;
         int w = 0;
         for (int k = 0; k < c; k++) {   // (every lane of a warp: the sums are in order)
@@ -325,12 +334,14 @@ __device__ __forceinline__ NewtonF newton_float(const DensArgs &a, const Sep &se
         }
         float g = Kn * f - N;
         float dg = Kn * mq * ih;
+        o.flat = !(mq > FLAT * f);
         if (g == 0.f) { o.conv = true; break; }
         if (g < 0.f) {
             if (h >= hsi) { o.fail = true; o.kf = Kn * f; break; }
             lo = fmaxf(lo, h);
-        } else {
-            hi = (hi < 0.f || h < hi) ? h : hi;
+        } else if (hi < 0.f || h < hi) {
+            hi = h;
+            hi_flat = o.flat;
         }
         float hn = dg > 0.f ? h - g / dg : -1.f;
         if (hn > 0.f && fabsf(hn - h) <= ftol * h && hn <= hsi) { h = hn; o.conv = true; break; }
@@ -413,7 +424,7 @@ __device__ __forceinline__ void dens_one(const DensArgs &a, double *__restrict__
         const float hh = narrow(h * rLmax);
         const float cut = hh * (1.f + 1e-5f) + slack, keep = hh * 1.0001f;
         // (the first pass of a converged float root compacts the list)
-        const bool shrink = a.compact && it == 1 && o.conv && hh > xmin;
+        const bool shrink = a.compact && it == 1 && o.conv && !o.flat && hh > xmin;
         int w = 0;
         for (int k0 = 0; k0 < c; k0 += W) {
             const int k = k0 + wk.lane;
@@ -560,7 +571,7 @@ __device__ __forceinline__ void dens_one(const DensArgs &a, float *__restrict__ 
     df ih = df_div({1.f, 0.f}, hd);
     df F = {0.f, 0.f}, MQ = {0.f, 0.f};
     const float hcut = h * (1.f + 1e-5f);   // W = 0 beyond h: skip those (float r is good to 1e-7)
-    const bool fin = a.compact && h > xmin;
+    const bool fin = a.compact && h > xmin && !nf.flat;
     const float keep = h * 1.0001f;
     int w = 0;
     for (int k0 = 0; k0 < c; k0 += W) {

@@ -147,3 +147,25 @@ def test_forms_of_the_solve_on_the_same_particles(hyd, precision):
             assert np.array_equal(a, b)
         else:
             assert np.max(np.abs(a / b - 1.0)) <= 3 * 60 * 2.0 ** -53
+
+
+@pytest.mark.parametrize("excess", [1.0, 1e-2, 1e-4, 1e-6])
+def test_step_with_n_ngb_near_the_own_term(hyd, excess):
+    """FP64, N_NGB just above the 14 of a particle's own term: the neighbours add little,
+    the root is flat, and its list must not be cut to a float root's margin.  The
+    steps solve (few neighbours leave the matrices ill-conditioned) and agree with
+    the staged solve, which cuts no list."""
+    w = W.lattice_wave(16, jitter=0.1)
+    H = hyd.Hydro(hyd.default_config(gamma=w["gamma"], n_ngb=14.0 + excess, max_ngb_grow=0))
+    H.set_boxes(*hyd.single_box(w))
+    st = hyd.to_device(w)
+    for _ in range(3):
+        assert H.step(st, 1e-12, check=False)["status"] in (0, -5)
+    h = st["h"].clone()
+    H.build_neighbours(st, h * 1.2, export=False)
+    H.density(st)
+    # (the slope is about 20 t^3 for one neighbour of 5 t^4 = excess / 14)
+    t = min((excess / 70.0) ** 0.25, 0.3)
+    tol = 1e-14 / t ** 3
+    assert float((st["h"] / h - 1.0).abs().max()) < tol
+    H.close()

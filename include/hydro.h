@@ -93,10 +93,17 @@ typedef struct {
     double beta_min, beta_max; /* conditioned BJ (1, 2) */
     double c_cfl;        /* CFL factor of Eq. 31 (0.2) */
     double alpha1;       /* total-energy pressure switch (1/100) */
-    double h_tol;        /* relative Newton tolerance on h (1e-10) */
-    double p_tol;        /* relative Newton tolerance on p* (1e-12 FP64) */
+    double h_tol;        /* relative Newton tolerance on h (1e-10); the FP64 path accepts a
+                            root finished by its third-order step, whose error is below
+                            1e-15, and applies h_tol only to the last evaluation that
+                            max_h_iter allows */
+    double p_tol;        /* relative Newton tolerance on p* (1e-12).  FP64: of the plain
+                            iteration, which takes the states that the usual finish (a float
+                            start and third-order steps to rounding) does not settle.
+                            Mixed: not below 2e-6 */
     int max_h_iter;      /* cap on the h iteration (60) */
-    int max_newton;      /* cap on Riemann Newton iterations (100) */
+    int max_newton;      /* cap on Riemann Newton iterations (100; FP64: of the plain
+                            iteration) */
     double search_margin;/* hydro_step: search radius = margin * h_in (1.15) */
     int graph;           /* hydro_step: 1 (default) runs the step as one captured
                             CUDA graph whose re-search and N_cond loops are

@@ -316,7 +316,9 @@ __global__ void __launch_bounds__(LIST_WARPS * 32, LIST_CTAS) k_build_lists(List
 #pragma unroll
             for (int t = 0; t < 2; t++) {
                 // (the lanes of the other part repeat one of this part's; a
-                // second part without owners repeats the last owner)
+                // second part without owners repeats the last owner.  With
+                // SPLIT > 1 the lanes from OW on hold all the item's owners
+                // again, so its second box spans both parts: no cut there)
                 const int src = t == 0 ? min(lane, cut - 1) : max(lane, min(cut, nown - 1));
                 const uint32_t x = __shfl_sync(0xffffffffu, sqx, src);
                 const uint32_t y = __shfl_sync(0xffffffffu, sqy, src);

@@ -62,6 +62,7 @@ struct FluxArgs {
     GasK<float> Kf;          // gas constants, precomputed on the host
     GasK<double> Kd;
     float psi1f, psi2f, ptolf;   // float copies (no per-face conversions)
+    bool psi_inf;            // psi1f or psi2f is infinite
     int64_t nbucket;
     const int32_t *node_first, *node_cnt;
     // gravity (§2.3.8): sum_j dm_ij r_ij, 3 n sorted SoA (NULL: no gravity);
@@ -107,8 +108,8 @@ __device__ __forceinline__ int sgn_(R v) { return (v > R(0)) - (v < R(0)); }
 // [lo - psi1 d, mean + psi2 d], the other in [mean - psi2 d, hi + psi1 d]
 // (d = |u - v|); for a positive field a bound that would change sign is shrunk
 // instead.  Both sides share the bounds, and the selections are without
-// branches.  Equal cells leave no room and give back the cell value, whatever the
-// factors (an infinite one switches its bound off, and times d = 0 is NaN).
+// branches: equal cells leave no room and give back the cell value (but for an
+// infinite factor, which times d = 0 is NaN: face_state then restores it).
 template <typename R>
 __device__ __forceinline__ void pair_limit(R &l, R &m, R u, R v, R psi1, R psi2, bool positive) {
     const R d = fabs(u - v), mean = R(0.5) * (u + v);
@@ -126,8 +127,8 @@ __device__ __forceinline__ void pair_limit(R &l, R &m, R u, R v, R psi1, R psi2,
     low = low > lox ? low : lox;
     high = high > bottom ? high : bottom;
     high = high < hix ? high : hix;
-    l = u == v ? u : up ? low : high;
-    m = u == v ? v : up ? high : low;
+    l = up ? low : high;
+    m = up ? high : low;
 }
 
 // r < h_j decided exactly (float path: band + double fallback)
@@ -205,6 +206,11 @@ __device__ __forceinline__ bool face_state(const FluxArgs &a, const GasK<R> &K, 
         for (int f = 0; f < 5; f++) {
             bool pos = (f == 0 || f == 4);
             pair_limit<R>(Lf[f], Rf[f], ri[R_RHO + f], rj[R_RHO + f], p1, p2, pos);
+        }
+        if (a.psi_inf) {
+#pragma unroll
+            for (int f = 0; f < 5; f++)
+                if (ri[R_RHO + f] == rj[R_RHO + f]) { Lf[f] = ri[R_RHO + f]; Rf[f] = rj[R_RHO + f]; }
         }
     }
     const R g = K.g;

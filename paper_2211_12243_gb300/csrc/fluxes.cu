@@ -3,6 +3,7 @@
 // run_fluxes, which clears the accumulators and runs the plain or the
 // learned (deferred hard faces) path.
 #include <algorithm>
+#include <cmath>
 
 #include "flux_kernel.cuh"
 
@@ -202,6 +203,7 @@ cudaError_t run_fluxes(hydro_ctx *c, double dt, const double *dt_dev, stream_t s
     a.rec_hard_only = c->rec_hard_only;
     a.psi1f = (float)c->cfg.psi1;
     a.psi2f = (float)c->cfg.psi2;
+    a.psi_inf = std::isinf(a.psi1f) || std::isinf(a.psi2f);
     a.ptolf = (float)std::max(c->cfg.p_tol, 2e-6);
     a.Kf = GasK<float>(c->cfg.gamma);
     a.Kd = GasK<double>(c->cfg.gamma);

@@ -68,7 +68,7 @@ __global__ void k_update(UpdArgs a) {
     }
     const double r0 = rcp64(m0);
     double vx0 = div1(px0, m0, r0), vy0 = div1(py0, m0, r0), vz0 = div1(pz0, m0, r0);
-    const bool moved = !dzero(dm);   // (mass: never in MFM)
+    const bool moved = (dbits(dm) << 1) != 0;   // (mass: never in MFM)
     double dU = dE - (vx0 * dpx + vy0 * dpy + vz0 * dpz);
     if (moved) dU += 0.5 * (vx0 * vx0 + vy0 * vy0 + vz0 * vz0) * dm;
     double m1 = m0 + dm, px1 = px0 + dpx, py1 = py0 + dpy, pz1 = pz0 + dpz;
@@ -95,7 +95,7 @@ __global__ void k_update(UpdArgs a) {
     double z = a.zs[s] + dt * 0.5 * (vz0 + vz1);
     // (-0.0 is not negative, but its bits are above those of L)
     auto wrap = [](double v, double L) {
-        if (!dlt_pos(v, L)) v = dneg(v) ? v + L : dzero(v) ? v : v - L;
+        if (!dlt_pos(v, L)) v = dneg(v) ? v + L : (dbits(v) << 1) == 0 ? v : v - L;
         return v;
     };
     x = wrap(x, bx.L[0]);

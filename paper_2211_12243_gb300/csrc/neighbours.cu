@@ -311,6 +311,10 @@ __global__ void __launch_bounds__(LIST_WARPS * 32, LIST_CTAS) k_build_lists(List
                 const uint32_t top = __reduce_max_sync(0xffffffffu, gap);
                 cut = __ffs(__ballot_sync(0xffffffffu, gap == top));   // owners [0, cut) and the rest
             }
+            // (the culls take the largest radius by its bits: -0, a negative one and NaN,
+            // whose bits are above every radius's, reach nothing)
+            const float hru = __double2float_ru(hs);
+            const uint32_t hbits = hru > 0.f ? __float_as_uint(hru) : 0u;
             uint4 qlo, qhi;
             __syncwarp();
 #pragma unroll
@@ -323,8 +327,7 @@ __global__ void __launch_bounds__(LIST_WARPS * 32, LIST_CTAS) k_build_lists(List
                 const uint32_t x = __shfl_sync(0xffffffffu, sqx, src);
                 const uint32_t y = __shfl_sync(0xffffffffu, sqy, src);
                 const uint32_t z = __shfl_sync(0xffffffffu, sqz, src);
-                const uint32_t r =
-                    __shfl_sync(0xffffffffu, __float_as_uint(__double2float_ru(hs)), src);
+                const uint32_t r = __shfl_sync(0xffffffffu, hbits, src);
                 uint4 lo, hi;
                 lo.x = __reduce_min_sync(0xffffffffu, x); hi.x = __reduce_max_sync(0xffffffffu, x);
                 lo.y = __reduce_min_sync(0xffffffffu, y); hi.y = __reduce_max_sync(0xffffffffu, y);

@@ -93,3 +93,33 @@ def test_export_of_rows_longer_than_shared_memory(orc, hyd):
     assert np.array_equal(off.cpu().numpy(), off_o)
     assert np.array_equal(idx.cpu().numpy(), idx_o)
     H.close()
+
+
+@pytest.mark.parametrize("n", [4099, 120011])
+def test_radii_of_zero_and_nan_leave_the_other_lists(hyd, n):
+    """A particle of radius +0, -0 or NaN has no neighbours; the lists of the
+    particles that share its bucket are those of the other radii alone."""
+    import torch
+    x, y, z = _uniform(n, (1, 1, 1), 30)
+    hs = np.full(n, _mean_h(n, (1, 1, 1), 40))
+    rng = np.random.default_rng(31)
+    odd = rng.choice(n, n // 50, replace=False)
+    out = []
+    for special in (False, True):
+        r = hs.copy()
+        r[odd] = np.resize([-0.0, np.nan, 0.0], odd.size) if special else 1e-9
+        H = hyd.Hydro(hyd.default_config())
+        H.set_boxes(np.array([0, n], dtype=np.int64), np.ones(3))
+        dev = lambda v: torch.as_tensor(np.ascontiguousarray(v, dtype=np.float64), device="cuda")
+        st = {"x": dev(x), "y": dev(y), "z": dev(z), "h": dev(hs)}
+        off, idx = H.build_neighbours(st, dev(r))
+        out.append((off.cpu().numpy(), idx.cpu().numpy()))
+        H.close()
+    (oa, ia), (ob, ib) = out
+    ca, cb = np.diff(oa), np.diff(ob)
+    assert np.all(cb[odd] == 0) and np.all(ca[odd] == 1)      # (the particle itself)
+    ca[odd] = 0
+    assert np.array_equal(ca, cb)
+    keep = np.ones(ia.size, dtype=bool)
+    keep[oa[odd]] = False
+    assert np.array_equal(ia[keep], ib)

@@ -143,7 +143,7 @@ __device__ __forceinline__ bool member_j(float r2, float hjf, const FluxArgs &a,
 }
 __device__ __forceinline__ bool member_j(double r2, double hj, const FluxArgs &, const Box &, int64_t,
                                          int64_t) {
-    return dlt_pos(r2, __dmul_rn(hj, hj));
+    return dlt_pos(r2, __dmul_rn(hj, hj));   // (a record holds no NaN h: k_primitives)
 }
 
 struct FaceStats {

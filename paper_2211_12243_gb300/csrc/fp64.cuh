@@ -57,7 +57,7 @@ __device__ __forceinline__ double dunkey(long long k) {
     return __longlong_as_double(k ^ (long long)((unsigned long long)(k >> 63) >> 1));
 }
 __device__ __forceinline__ bool dlt(double a, double b) { return dkey(a) < dkey(b); }
-// a < b for a, b >= 0 (false when a is NaN)
+// a < b for a, b >= 0 (false when a is NaN; b must not be: its bits are above all)
 __device__ __forceinline__ bool dlt_pos(double a, double b) {
     return (unsigned long long)dbits(a) < (unsigned long long)dbits(b);
 }

@@ -68,7 +68,7 @@ __device__ __forceinline__ void grad_one(const GradArgs &a, double *__restrict__
     const Box bx = a.boxes[a.pbox[s]];
     double ri[10];
     load_row<10>(rec, s, ri);
-    const double h = a.h[s], h2 = __dmul_rn(h, h);
+    const double h = a.h[s], h2 = radius2(h);
     const double h2lo = h2 * (1.0 - 1e-14), h2hi = h2 * (1.0 + 1e-14);
     const double ih = 1.0 / h, norm = kernel_norm<double>(a.kernel, h);
     const double fi[5] = {ri[R_RHO], ri[R_VX], ri[R_VY], ri[R_VZ], ri[R_P]};
@@ -552,7 +552,8 @@ __global__ void k_primitives(int64_t n, const double *__restrict__ Q,
             const double therm = from == 0 ? E - ekin : U;
             const double rho = m / w;
             pd = therm * gm1 / w;
-            r[R_H] = (R)h[s];
+            // (an h that is not a number has no pairs: 0, whose faces have no area)
+            r[R_H] = (R)(isnan(h[s]) ? 0.0 : h[s]);
             r[R_RHO] = (R)rho;
             r[R_VX] = (R)(px / m);
             r[R_VY] = (R)(py / m);

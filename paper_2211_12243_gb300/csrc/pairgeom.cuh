@@ -73,10 +73,15 @@ struct Member<float> {
         return member_exact(a, i, j, i);
     }
 };
+// h^2 for comparisons of bits (dlt_pos): no distance is below that of a NaN
+__device__ __forceinline__ double radius2(double h) {
+    const double h2 = __dmul_rn(h, h);
+    return dhi(h2) <= 0x7ff00000u ? h2 : 0.0;
+}
 template <>
 struct Member<double> {
     double h2;
-    __device__ __forceinline__ void init(double h, const Box &) { h2 = __dmul_rn(h, h); }
+    __device__ __forceinline__ void init(double h, const Box &) { h2 = radius2(h); }
     // r2 is already the exact value (r2, h2 >= 0)
     __device__ __forceinline__ bool operator()(const Exact &, double r2, int, int) const {
         return dlt_pos(r2, h2);

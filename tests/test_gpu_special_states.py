@@ -150,3 +150,31 @@ def test_particles_whose_squared_distance_is_subnormal(orc, gap):
     errs, bad = compare(g, o, 1e-12, what=("h", "omega", "B", "grad", "ncond", "dQ"))
     assert not bad, errs
     H.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_smoothing_length_that_is_not_a_number(precision):
+    """staged calls with one such h: that particle has no pairs, so its matrix is
+    singular (B and gradient 0) and its faces carry nothing; particles out of its
+    reach keep their values"""
+    import torch
+    from paper_2211_12243_gb300 import hydro
+    w = W.lattice_wave(12, jitter=0.05)
+    H = hydro.Hydro(hydro.default_config(gamma=w["gamma"], precision=precision))
+    H.set_boxes(*hydro.single_box(w))
+    st = hydro.to_device(w)
+    H.build_neighbours(st, st["h"] * 1.3, export=False)
+    H.density(st)
+    ref = H.gradients(st)
+    dQ0 = H.fluxes(st, *ref[:3], 1e-3)
+    st["h"][100] = float("nan")
+    B, G, A, N = H.gradients(st)
+    assert torch.all(B[100] == 0) and torch.all(G[100] == 0) and torch.isinf(N[100])
+    other = torch.arange(B.shape[0], device="cuda") != 100
+    for a, b in zip(ref, (B, G, A, N)):
+        assert torch.equal(a[other], b[other])
+    dQ = H.fluxes(st, *ref[:3], 1e-3)
+    assert torch.all(dQ[100] == 0) and torch.isfinite(dQ).all()
+    same = (dQ - dQ0).abs().amax(1) <= 1e-12 * dQ0.abs().max()
+    assert int((~same).sum()) < 120       # (its neighbours)
+    H.close()
